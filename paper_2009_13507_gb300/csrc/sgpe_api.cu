@@ -258,7 +258,13 @@ static void spin_eigvecs(int which, double* ur, double* ui) {
     }
 }
 
-static sgpe_status build_socn(sgpe_ctx* c) {
+// The table job of an n-point line with tables t.
+static CoefJob coef_job(void* const* t, int n, double bre, double bim, int skew) {
+    return CoefJob{t[0], t[1], t[2], t[3], n, chunk_len(n), table_len(n), n > kRegMaxN ? 1 : 0, skew, bre, bim};
+}
+
+// (its table jobs are added to jobs)
+static sgpe_status build_socn(sgpe_ctx* c, CoefJob* jobs, int* njobs) {
     const sgpe_params& p = c->params;
     c->socn_y = false;
     if (c->kp.so_case == 0 || c->nx > kRegMaxN || (c->dim == 2 && c->ny > kRegMaxN)) return SGPE_OK;
@@ -297,14 +303,8 @@ static sgpe_status build_socn(sgpe_ctx* c) {
                 L.lstride = 1;
             }
             if (a == 1 && !c->socn_y) continue;
-            void** tp = c->tabs_so[m][a][0];
-            void** tm = c->tabs_so[m][a][1];
-            cudaError_t e = with_prec(c->prec, [&](auto r) {
-                cudaError_t e1 = Launcher<decltype(r)>::coef_skew(c->stream, tp[0], tp[1], tp[2], tp[3], L.n, L.are, L.aim);
-                if (e1) return e1;
-                return Launcher<decltype(r)>::coef_skew(c->stream, tm[0], tm[1], tm[2], tm[3], L.n, -L.are, -L.aim);
-            });
-            CK(e, "SO Crank-Nicolson tables");
+            jobs[(*njobs)++] = coef_job(c->tabs_so[m][a][0], L.n, L.are, L.aim, 1);
+            jobs[(*njobs)++] = coef_job(c->tabs_so[m][a][1], L.n, -L.are, -L.aim, 1);
         }
     }
     return SGPE_OK;
@@ -399,7 +399,9 @@ sgpe_status sgpe_set_params(sgpe_ctx* c, const sgpe_params* p) {
     sgpe_params ph = *p;
     ph.dt = 0.5 * p->dt;
     c->kp_half = make_kparams(c->dim, c->nx, c->ny, c->dx, c->dy, &ph);
-    if (sgpe_status st = build_socn(c)) return st;
+    CoefJob jobs[8 + 6];  // SO by Crank-Nicolson: [mode][axis][m]; kinetic: [mode][axis]
+    int njobs = 0;
+    if (sgpe_status st = build_socn(c, jobs, &njobs)) return st;
     // COEF: Crank-Nicolson tables, bt = z/(4 h^2), z = dt (imaginary), i dt (real), -i dt (adjoint)
     for (int m = 0; m < 3; m++)
         for (int a = 0; a < (c->dim == 2 ? 2 : 1); a++) {
@@ -407,21 +409,20 @@ sgpe_status sgpe_set_params(sgpe_ctx* c, const sgpe_params* p) {
             int n = a == 0 ? c->nx : c->ny;
             double b = p->dt / (4.0 * h * h);
             double bre = m == 0 ? b : 0.0, bim = m == 0 ? 0.0 : (m == 1 ? b : -b);
-            void** t = c->tabs[m][a].t;
-            cudaError_t e = with_prec(c->prec, [&](auto r) {
-                return Launcher<decltype(r)>::coef(c->stream, t[0], t[1], t[2], t[3], n, bre, bim);
-            });
-            CK(e, "COEF kernel");
+            jobs[njobs++] = coef_job(c->tabs[m][a].t, n, bre, bim, 0);
             // lines longer than kRegMaxN (and the lines of a tiled grid): the constant-factor
             // form of the same solve
             c->tabs[m][a].u = UniHost{};
             if (n > kRegMaxN || c->geo.tiled) {
-                e = with_prec(c->prec, [&](auto r) {
+                cudaError_t e = with_prec(c->prec, [&](auto r) {
                     return Launcher<decltype(r)>::uni(c->stream, n, bre, bim, c->us[m][a], &c->tabs[m][a].u);
                 });
                 CK(e, "constant-factor form");
             }
         }
+    cudaError_t e = with_prec(
+        c->prec, [&](auto r) { return Launcher<decltype(r)>::coef(c->stream, jobs, njobs); });
+    CK(e, "COEF kernel");
     c->have_params = true;
     return SGPE_OK;
 }

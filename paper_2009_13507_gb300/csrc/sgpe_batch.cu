@@ -774,6 +774,7 @@ sgpe_status sgpe_batch_bind(sgpe_batch* b, void* psi_dev, void* workspace_dev) {
     kb_reset<<<(b->n + 127) / 128, 128, 0, s>>>(sc, b->n, 1);
     BCK(cudaGetLastError(), "reset");
     // COEF for every instance, both time modes and axes
+    std::vector<CoefJob> jobs;
     for (int i = 0; i < b->n; i++) {
         const BInst& I = b->hinst[i];
         for (int m = 0; m < 2; m++)
@@ -786,12 +787,12 @@ sgpe_status sgpe_batch_bind(sgpe_batch* b, void* psi_dev, void* workspace_dev) {
                 double bt = I.p.dt / (4.0 * h * h);
                 double bre = m == 0 ? bt : 0.0, bim = m == 0 ? 0.0 : bt;
                 size_t L = (size_t)b->esz * len;
-                cudaError_t e = b->prec == SGPE_C128
-                                    ? Launcher<double>::coef(s, t, t + L, t + 2 * L, t + 3 * L, nn, bre, bim)
-                                    : Launcher<float>::coef(s, t, t + L, t + 2 * L, t + 3 * L, nn, bre, bim);
-                BCK(e, "COEF kernel");
+                jobs.push_back(CoefJob{t, t + L, t + 2 * L, t + 3 * L, nn, chunk_len(nn), len, 0, 0, bre, bim});
             }
     }
+    BCK(b->prec == SGPE_C128 ? Launcher<double>::coef(s, jobs.data(), (int)jobs.size())
+                             : Launcher<float>::coef(s, jobs.data(), (int)jobs.size()),
+        "COEF kernel");
     BCK(cudaStreamSynchronize(s), "sync");  // host work lists must outlive the copies
     return SGPE_OK;
 }

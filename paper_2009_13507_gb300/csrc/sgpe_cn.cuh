@@ -50,7 +50,7 @@ template <typename R, bool IMAG, int C> struct LaneTabs {
 // Solve T w = x for the lane's chunk v (in: x, out: w), all 32 lanes together.
 // SKEW: T has opposite off-diagonals (lower -a, upper +a; the Crank-Nicolson
 // matrix of a first-derivative operator): the backward recurrence then runs with
-// -fg and fq holds the chunk products of -fg (k_coef_skew).
+// -fg and fq holds the chunk products of -fg (k_coef).
 template <typename R, bool IMAG, int C, bool SKEW = false>
 __device__ __forceinline__ void solve_chunk(cx<R> (&v)[C], const LaneTabs<R, IMAG, C>& t) {
     const int lane = threadIdx.x & 31;

@@ -671,8 +671,8 @@ static __global__ void __launch_bounds__(96 * kFinWarps) k_finalize_wide(const d
 
 // ---------------------------------------------------------------------------
 // COEF: build the Crank-Nicolson tables of one axis for bt = (bre, bim)
-// (bt = dt/(4h^2) in imaginary time, i dt/(4h^2) in real time). One thread;
-// FP64 arithmetic, stored rounded to R.
+// (bt = dt/(4h^2) in imaginary time, i dt/(4h^2) in real time). FP64 arithmetic,
+// stored rounded to R.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void cdiv(double ar, double ai, double br, double bi, double* r, double* i) {
     // (a / b) with Smith's scaling
@@ -692,42 +692,105 @@ __device__ __forceinline__ void cdiv(double ar, double ai, double br, double bi,
 // interleave (lines longer than 1024 points) entry i of every table is stored at
 // (i % C) * (len / C) + i / C: lane g of a line's warp group reads its chunk
 // entry m at m * G + g, G = len / C lanes, so a warp's table reads are coalesced.
-template <typename R>
-__global__ void k_coef(typename V2<R>::T* fa, typename V2<R>::T* fg, typename V2<R>::T* fp,
-                       typename V2<R>::T* fq, int n, int C, int len, int interleave, double bre, double bim) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    const double dr = 1.0 + 2.0 * bre, di = 2.0 * bim;  // diagonal 1 + 2 bt
+//
+// One block per table set (a grid's axes and time modes go out in one launch).
+// The pivot recurrence is a serial chain of FP64 divisions, about 1 us a point,
+// but also a contraction: after a few points (about 10 at bt = 0.02, some 130 at
+// bt = 50) a pivot equals its predecessor bit for bit and so do all that follow.
+// Thread 0 walks the chain in segments of kCoefThreads points only as far as
+// that; the divisions of the factors then go one thread per point and the chunk
+// products one thread per chunk. The values are those of the serial walk. The
+// tables of one 256^2 complex64 grid (14, SO by Crank-Nicolson included) measured
+// 17.9 ms with one thread a table, launch after launch; this is what a call that
+// sets parameters (every differentiated propagation does) waits for.
+constexpr int kCoefThreads = 256;
+
+// skew: T = tridiag(-a, 1, a) with a = (bre, bim) instead (sgpe_socn.cuh): u_0 = 1,
+// u_i = 1 + a^2 / u_(i-1), and fq holds the chunk products of -fg.
+struct CoefJob {
+    void *fa, *fg, *fp, *fq;
+    int n, C, len, interleave, skew;
+    double bre, bim;
+};
+constexpr int kCoefJobs = 48;  // (kernel parameters: 48 x 72 bytes)
+struct CoefJobs {
+    CoefJob job[kCoefJobs];
+};
+
+template <typename R> __global__ void __launch_bounds__(kCoefThreads) k_coef(CoefJobs jobs) {
+    using T = typename V2<R>::T;
+    __shared__ double su[kCoefThreads][2];
+    __shared__ int s_fixed;  // the pivots from this point of the segment on are su[s_fixed]
+    const CoefJob& J = jobs.job[blockIdx.x];
+    T *fa = (T*)J.fa, *fg = (T*)J.fg, *fp = (T*)J.fp, *fq = (T*)J.fq;
+    const int n = J.n, C = J.C, len = J.len, tid = threadIdx.x;
+    const double bre = J.bre, bim = J.bim;
+    const double sgn = J.skew ? 1.0 : -1.0;
+    const double dr = J.skew ? 1.0 : 1.0 + 2.0 * bre, di = J.skew ? 0.0 : 2.0 * bim;  // diagonal
+    const double b2r = bre * bre - bim * bim, b2i = 2.0 * bre * bim;
     const cx<R> zero = {R(0), R(0)};
     const int G = len / C;
-    auto at = [&](int i) { return interleave ? (i % C) * G + i / C : i; };
-    for (int i = n; i < len; i++) {
+    auto at = [&](int i) { return J.interleave ? (i % C) * G + i / C : i; };
+    for (int i = n + tid; i < len; i += kCoefThreads) {
         st<R>(fa, at(i), zero);
         st<R>(fg, at(i), zero);
     }
-    double ur = dr, ui = di;
-    for (int i = 0; i < n; i++) {
-        if (i > 0) {
-            // u_i = (1 + 2bt) - bt^2 / u_{i-1}
-            double b2r = bre * bre - bim * bim, b2i = 2.0 * bre * bim;
-            double qr, qi;
-            cdiv(b2r, b2i, ur, ui, &qr, &qi);
-            ur = dr - qr;
-            ui = di - qi;
-        }
+    auto factors = [&](double ur, double ui, cx<R>& a, cx<R>& g) {
         double ar, ai, gr, gi;
         cdiv(1.0, 0.0, ur, ui, &ar, &ai);
         cdiv(bre, bim, ur, ui, &gr, &gi);
-        st<R>(fa, at(i), cx<R>{to_r<R>(ar), to_r<R>(ai)});
-        st<R>(fg, at(i), cx<R>{to_r<R>(gr), to_r<R>(gi)});
+        a = {to_r<R>(ar), to_r<R>(ai)};
+        g = {to_r<R>(gr), to_r<R>(gi)};
+    };
+    double ur = dr, ui = di;  // thread 0: the last pivot
+    for (int i0 = 0; i0 < n; i0 += kCoefThreads) {
+        const int m = min(kCoefThreads, n - i0);
+        if (tid == 0) {
+            int fixed = m;
+            for (int k = 0; k < m; k++) {
+                if (i0 + k > 0) {
+                    // u_i = d -+ b^2 / u_(i-1)
+                    double qr, qi;
+                    cdiv(b2r, b2i, ur, ui, &qr, &qi);
+                    const double vr = dr + sgn * qr, vi = di + sgn * qi;
+                    const bool same = vr == ur && vi == ui;
+                    ur = vr;
+                    ui = vi;
+                    if (same) fixed = k;
+                }
+                su[k][0] = ur;
+                su[k][1] = ui;
+                if (fixed < m) break;
+            }
+            s_fixed = fixed;
+        }
+        __syncthreads();
+        const int fixed = s_fixed;
+        cx<R> a, g;
+        if (tid < m) {
+            factors(su[min(tid, fixed)][0], su[min(tid, fixed)][1], a, g);
+            st<R>(fa, at(i0 + tid), a);
+            st<R>(fg, at(i0 + tid), g);
+        }
+        if (fixed < m) {  // every later point of the line has this pivot
+            factors(su[fixed][0], su[fixed][1], a, g);
+            for (int i = i0 + m + tid; i < n; i += kCoefThreads) {
+                st<R>(fa, at(i), a);
+                st<R>(fg, at(i), g);
+            }
+            break;
+        }
+        __syncthreads();
     }
-    // chunk products, computed from the rounded-to-FP64 fg values
-    for (int k0 = 0; k0 < len; k0 += C) {
-        int k1 = k0 + C;
+    __syncthreads();
+    // chunk products, computed from the rounded-to-R fg values
+    for (int k0 = tid * C; k0 < len; k0 += kCoefThreads * C) {
+        const int k1 = k0 + C;
         double Pr = 1.0, Pi = 0.0;
         for (int i = k0; i < k1; i++) {
             const cx<R> g = unpack(fg[at(i)]);
-            double gr = dbl(g.re), gi = dbl(g.im);
-            double tr = Pr * gr - Pi * gi, ti = Pr * gi + Pi * gr;
+            const double gr = dbl(g.re), gi = dbl(g.im);
+            const double tr = Pr * gr - Pi * gi, ti = Pr * gi + Pi * gr;
             Pr = tr;
             Pi = ti;
             st<R>(fp, at(i), cx<R>{to_r<R>(Pr), to_r<R>(Pi)});
@@ -736,8 +799,8 @@ __global__ void k_coef(typename V2<R>::T* fa, typename V2<R>::T* fg, typename V2
         Pi = 0.0;
         for (int i = k1 - 1; i >= k0; i--) {
             const cx<R> g = unpack(fg[at(i)]);
-            double gr = dbl(g.re), gi = dbl(g.im);
-            double tr = Pr * gr - Pi * gi, ti = Pr * gi + Pi * gr;
+            const double gr = -sgn * dbl(g.re), gi = -sgn * dbl(g.im);
+            const double tr = Pr * gr - Pi * gi, ti = Pr * gi + Pi * gr;
             Pr = tr;
             Pi = ti;
             st<R>(fq, at(i), cx<R>{to_r<R>(Pr), to_r<R>(Pi)});

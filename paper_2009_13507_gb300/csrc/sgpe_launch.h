@@ -14,6 +14,7 @@ namespace sgpe {
 struct KParams;
 struct DevScalars;
 struct SoCnLines;
+struct CoefJob;
 
 // Launch a step kernel with programmatic stream serialization: its blocks may
 // be scheduled before the previous kernel on the stream completes; the kernel
@@ -180,7 +181,8 @@ template <typename R> struct Launcher {
     static cudaError_t pwx_long(cudaStream_t s, bool imag, const void* A, void* B, const KParams& p,
                                 const DevScalars* sc, const double* omega_tab, const TabSet& tabs_x, int mask,
                                 const double* partials = nullptr, int m = 0, int renorm = 0);
-    static cudaError_t coef(cudaStream_t s, void* fa, void* fg, void* fp, void* fq, int n, double bre, double bim);
+    // The coefficient tables of count lines (coef_job), kCoefJobs a launch.
+    static cudaError_t coef(cudaStream_t s, const CoefJob* jobs, int count);
     // The constant-factor form of an n-point line with bt = bre + i bim: fills u and
     // copies s to s_dev (kUniMaxS entries of room; s_dev null: no copy); u->ks = 0
     // where the correction would be longer than that (and always for complex128).
@@ -193,8 +195,6 @@ template <typename R> struct Launcher {
     // kRegMaxN points); tabs_p / tabs_m: the skew tables of m = +1 / -1.
     static cudaError_t socn(cudaStream_t s, const void* in, void* out, const SoCnLines& L, const void* const* tabs_p,
                             const void* const* tabs_m, const DevScalars* sc, int scale);
-    static cudaError_t coef_skew(cudaStream_t s, void* fa, void* fg, void* fp, void* fq, int n, double are,
-                                 double aim);
     static cudaError_t observables(cudaStream_t s, const void* A, const KParams& p, double omega_t,
                                    double* partials, DevScalars* sc);
 };

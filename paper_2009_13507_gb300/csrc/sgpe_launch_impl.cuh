@@ -222,15 +222,6 @@ cudaError_t Launcher<R>::socn(cudaStream_t s, const void* in, void* out, const S
     return cudaGetLastError();
 }
 
-template <typename R>
-cudaError_t Launcher<R>::coef_skew(cudaStream_t s, void* fa, void* fg, void* fp, void* fq, int n, double are,
-                                   double aim) {
-    using T = typename V2<R>::T;
-    const int C = chunk_len(n);
-    k_coef_skew<R><<<1, 32, 0, s>>>((T*)fa, (T*)fg, (T*)fp, (T*)fq, n, C, 32 * C, are, aim);
-    return cudaGetLastError();
-}
-
 template <typename R> cudaError_t Launcher<R>::setup() {
     cudaError_t e;
     if constexpr (kUniForm<R>) {
@@ -423,11 +414,13 @@ cudaError_t Launcher<R>::cn_y(cudaStream_t s, bool imag, const void* in, void* o
     return cudaGetLastError();
 }
 
-template <typename R>
-cudaError_t Launcher<R>::coef(cudaStream_t s, void* fa, void* fg, void* fp, void* fq, int n, double bre, double bim) {
-    using T = typename V2<R>::T;
-    k_coef<R><<<1, 32, 0, s>>>((T*)fa, (T*)fg, (T*)fp, (T*)fq, n, chunk_len(n), table_len(n), n > kRegMaxN ? 1 : 0,
-                               bre, bim);
+template <typename R> cudaError_t Launcher<R>::coef(cudaStream_t s, const CoefJob* jobs, int count) {
+    for (int i = 0; i < count; i += kCoefJobs) {
+        const int m = std::min(kCoefJobs, count - i);
+        CoefJobs J{};
+        std::copy(jobs + i, jobs + i + m, J.job);
+        k_coef<R><<<m, kCoefThreads, 0, s>>>(J);
+    }
     return cudaGetLastError();
 }
 

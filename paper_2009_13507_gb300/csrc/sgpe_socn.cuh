@@ -13,7 +13,9 @@
 // a tridiagonal matrix with opposite off-diagonals (S+-: shift by one point).
 // Each line is solved in increment form, phi' = phi + 2 e with
 // T e = -a_m (phi_(i+1) - phi_(i-1)), by the lane-chunk scan of the kinetic
-// sweeps with skew tables (k_coef_skew). The result is psi' = U phi'.
+// sweeps with skew tables (k_coef, CoefJob::skew): u_0 = 1, u_i = 1 + a^2 / u_(i-1);
+// forward y_i = fa_i x_i + fg_i y_(i-1) with fa = 1/u, fg = a/u; backward w_i = y_i -
+// fg_i w_(i+1). The result is psi' = U phi'.
 //
 // One block of three warps per line (n <= 1024 points): the line's three
 // components are loaded, rotated and staged in shared memory in the lanes'
@@ -55,59 +57,6 @@ __device__ __forceinline__ cx<R> rot_term(cx<R> u, cx<R> ul, cx<R> v) {
 
 template <typename R, int C> constexpr size_t socn_smem_bytes() {
     return (size_t)3 * 32 * (C + 1) * sizeof(typename V2<R>::T);
-}
-
-// COEF of the skew matrix T = tridiag(-a, 1, a) of n points for one m:
-// u_0 = 1, u_i = 1 + a^2 / u_(i-1); forward y_i = fa_i x_i + fg_i y_(i-1) with
-// fa = 1/u, fg = a/u; backward w_i = y_i - fg_i w_(i+1). fp: chunk prefix
-// products of fg, fq: chunk suffix products of -fg. Tables padded with zeros
-// to len = 32 C entries. One thread; FP64, stored rounded to R.
-template <typename R>
-__global__ void k_coef_skew(typename V2<R>::T* fa, typename V2<R>::T* fg, typename V2<R>::T* fp,
-                            typename V2<R>::T* fq, int n, int C, int len, double are, double aim) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    const cx<R> zero = {R(0), R(0)};
-    for (int i = n; i < len; i++) {
-        st<R>(fa, i, zero);
-        st<R>(fg, i, zero);
-    }
-    const double a2r = are * are - aim * aim, a2i = 2.0 * are * aim;
-    double ur = 1.0, ui = 0.0;
-    for (int i = 0; i < n; i++) {
-        if (i > 0) {
-            double qr, qi;
-            cdiv(a2r, a2i, ur, ui, &qr, &qi);
-            ur = 1.0 + qr;
-            ui = qi;
-        }
-        double xr, xi, gr, gi;
-        cdiv(1.0, 0.0, ur, ui, &xr, &xi);
-        cdiv(are, aim, ur, ui, &gr, &gi);
-        st<R>(fa, i, cx<R>{to_r<R>(xr), to_r<R>(xi)});
-        st<R>(fg, i, cx<R>{to_r<R>(gr), to_r<R>(gi)});
-    }
-    for (int k0 = 0; k0 < len; k0 += C) {
-        const int k1 = k0 + C;
-        double Pr = 1.0, Pi = 0.0;
-        for (int i = k0; i < k1; i++) {
-            const cx<R> g = unpack(fg[i]);
-            const double gr = dbl(g.re), gi = dbl(g.im);
-            const double tr = Pr * gr - Pi * gi, ti = Pr * gi + Pi * gr;
-            Pr = tr;
-            Pi = ti;
-            st<R>(fp, i, cx<R>{to_r<R>(Pr), to_r<R>(Pi)});
-        }
-        Pr = 1.0;
-        Pi = 0.0;
-        for (int i = k1 - 1; i >= k0; i--) {
-            const cx<R> g = unpack(fg[i]);
-            const double gr = -dbl(g.re), gi = -dbl(g.im);
-            const double tr = Pr * gr - Pi * gi, ti = Pr * gi + Pi * gr;
-            Pr = tr;
-            Pi = ti;
-            st<R>(fq, i, cx<R>{to_r<R>(Pr), to_r<R>(Pi)});
-        }
-    }
 }
 
 // The SO-CN substep on one family of lines: in -> out (may be the same buffer).
