@@ -35,8 +35,8 @@ struct BInst {
     int lenx, leny; // table lengths per axis
     int slot0;      // first partial-norm slot of the instance's final sweep
     int nslot;
-    int tile0;      // first pointwise / observable tile
-    int ntile;
+    int obs0;       // first observable block
+    int nobs;
 };
 
 // Tables of an instance: [mode 0 imag, 1 real][axis x, y][fa, fg, fp, fq].
@@ -248,33 +248,48 @@ __global__ void kb_reset(DevScalars* scs, int n, int clear_err) {
     if (i < n && clear_err) scs[i].err = 0;
 }
 
+// Rows a warp of the batched observables takes (a block: 32 columns x 4 strips in
+// 2D, 128 points in 1D). The instances together fill the GPU many times over.
+constexpr int kBatchObsRows = 8;
+
+// Observable block: (instance, block of the instance).
 template <typename R>
 __global__ void __launch_bounds__(128) kb_obs_tiles(const typename V2<R>::T* __restrict__ A,
                                                     const BInst* __restrict__ insts, const int2* __restrict__ tiles,
                                                     double* partials) {
-    __shared__ double red[4 * NACC];
+    __shared__ double red[NACC][kObsPad];
     const int2 tl = tiles[blockIdx.x];
     const BInst& I = insts[tl.x];
-    int ix, iy;
-    tile_point(I.p, tl.y, &ix, &iy);
+    const int tid = threadIdx.x;
     double v[NACC];
-    for (int q = 0; q < NACC; q++) v[q] = 0.0;
-    if (ix < I.p.nx && iy < I.p.ny) obs_point<R>(A + I.off, I.p, I.p.omega_t, ix, iy, v);
-    block_reduce<NACC>(v, red);
-    if (threadIdx.x == 0)
-        for (int q = 0; q < NACC; q++) partials[(size_t)blockIdx.x * NACC + q] = v[q];
+    if (I.p.dim == 2) {
+        const int ntx = (I.p.nx + 31) / 32;
+        obs_strip<R>(A + I.off, I.p, I.p.omega_t, (tl.y % ntx) * 32 + (tid & 31),
+                     (4 * (tl.y / ntx) + (tid >> 5)) * kBatchObsRows, kBatchObsRows, v);
+    } else {
+        obs_strip<R>(A + I.off, I.p, I.p.omega_t, 128 * tl.y + tid, 0, 1, v);
+    }
+    const double s = obs_block_sum(v, red);
+    if (tid < 8 * NACC && (tid & 7) == 0) partials[(size_t)blockIdx.x * NACC + (tid >> 3)] = s;
 }
 
 __global__ void __launch_bounds__(128) kb_obs_final(const BInst* __restrict__ insts, const double* partials,
                                                     DevScalars* scs) {
-    __shared__ double red[4 * NACC];
+    __shared__ double red[NACC][kObsPad];
     const BInst& I = insts[blockIdx.x];
-    double s[NACC];
-    for (int q = 0; q < NACC; q++) s[q] = 0.0;
-    for (int b = threadIdx.x; b < I.ntile; b += blockDim.x)
-        for (int q = 0; q < NACC; q++) s[q] += __ldcg(partials + (size_t)(I.tile0 + b) * NACC + q);
-    block_reduce<NACC>(s, red);
-    if (threadIdx.x == 0) obs_finish(s, I.p.cell, scs[blockIdx.x].obs, &scs[blockIdx.x].err);
+    const int tid = threadIdx.x;
+    double v[NACC];
+    for (int q = 0; q < NACC; q++) v[q] = 0.0;
+    for (int b = tid; b < I.nobs; b += 128)
+        for (int q = 0; q < NACC; q++) v[q] += __ldcg(partials + (size_t)(I.obs0 + b) * NACC + q);
+    const double s = obs_block_sum(v, red);
+    if (tid < 8 * NACC && (tid & 7) == 0) red[0][tid >> 3] = s;
+    __syncthreads();
+    if (tid == 0) {
+        double t[NACC];
+        for (int q = 0; q < NACC; q++) t[q] = red[0][q];
+        obs_finish(t, I.p.cell, scs[blockIdx.x].obs, &scs[blockIdx.x].err);
+    }
 }
 
 }  // namespace sgpe
@@ -296,7 +311,8 @@ struct sgpe_batch {
     cudaStream_t stream;
     std::vector<sgpe_instance> inst;
     std::vector<BInst> hinst;
-    std::vector<int2> tiles;    // every instance's tiles (flush, observables)
+    std::vector<int2> tiles;    // every instance's tiles (flush)
+    std::vector<int2> otiles;   // every instance's observable blocks
     std::vector<int2> pwtiles;  // the tiles of the pointwise kernel (instances on the register path)
     std::map<int, std::vector<int4>> cnx, cny, rows;  // work lists by chunk length (rows: the fused x part)
     // tiled instances (complex64): row entries by warps a line, tile entries by halo depth
@@ -307,7 +323,7 @@ struct sgpe_batch {
     int nslots;
     // workspace layout (byte offsets)
     size_t o_inst, o_sc, o_tiles, o_part, o_tab, o_mid, total;
-    size_t o_pwtiles, o_uni, o_us;
+    size_t o_pwtiles, o_otiles, o_uni, o_us;
     std::map<int, size_t> o_cnx, o_cny, o_rows, o_rows_t, o_ytile;
     // bound buffers
     void* psi;
@@ -574,8 +590,10 @@ sgpe_status sgpe_batch_create(sgpe_batch** out, int n, const sgpe_instance* inst
         I.leny = q.dim == 2 ? table_len(q.ny) : 0;
         I.tab = tab;
         tab += 2LL * 4 * (I.lenx + I.leny);
-        I.tile0 = (int)b->tiles.size();
-        I.ntile = q.dim == 2 ? ceil_div(q.nx, 32) * ceil_div(q.ny, 4) : ceil_div(q.nx, 128);
+        const int ntile = q.dim == 2 ? ceil_div(q.nx, 32) * ceil_div(q.ny, 4) : ceil_div(q.nx, 128);
+        I.obs0 = (int)b->otiles.size();
+        I.nobs = q.dim == 2 ? ceil_div(q.nx, 32) * ceil_div(q.ny, 4 * kBatchObsRows) : ntile;
+        for (int t = 0; t < I.nobs; t++) b->otiles.push_back(make_int2(i, t));
         // complex64 2D instances of 128..1024 points an axis with even rows take the tiled
         // step when both axes have the constant-factor form in both time modes (from 128
         // points: inside a batch the grouped launches fill the GPU; 64-instance workload
@@ -594,7 +612,7 @@ sgpe_status sgpe_batch_create(sgpe_batch** out, int n, const sgpe_instance* inst
                     hcmax = std::max(hcmax, u.hc);
             }
         b->tiled.push_back(tl ? 1 : 0);
-        for (int t = 0; t < I.ntile; t++) {
+        for (int t = 0; t < ntile; t++) {
             b->tiles.push_back(make_int2(i, t));
             if (!tl) b->pwtiles.push_back(make_int2(i, t));
         }
@@ -640,6 +658,8 @@ sgpe_status sgpe_batch_create(sgpe_batch** out, int n, const sgpe_instance* inst
     o = al256(o + sizeof(int2) * b->tiles.size());
     b->o_pwtiles = o;
     o = al256(o + sizeof(int2) * b->pwtiles.size());
+    b->o_otiles = o;
+    o = al256(o + sizeof(int2) * b->otiles.size());
     for (auto& kv : b->rows_t) {
         b->o_rows_t[kv.first] = o;
         o = al256(o + sizeof(int4) * kv.second.size());
@@ -666,7 +686,7 @@ sgpe_status sgpe_batch_create(sgpe_batch** out, int n, const sgpe_instance* inst
         o = al256(o + sizeof(int4) * kv.second.size());
     }
     b->o_part = o;
-    size_t np = std::max((size_t)3 * b->nslots, (size_t)NACC * b->tiles.size());
+    size_t np = std::max((size_t)3 * b->nslots, (size_t)NACC * b->otiles.size());
     o = al256(o + sizeof(double) * np);
     b->o_tab = o;
     o = al256(o + (size_t)b->esz * b->tab_elems);
@@ -703,6 +723,8 @@ sgpe_status sgpe_batch_bind(sgpe_batch* b, void* psi_dev, void* workspace_dev) {
     BCK(cudaMemsetAsync(b->work + b->o_sc, 0, sizeof(DevScalars) * b->n, s), "memset");
     BCK(cudaMemcpyAsync(b->work + b->o_tiles, b->tiles.data(), sizeof(int2) * b->tiles.size(), cudaMemcpyHostToDevice,
                         s), "copy");
+    BCK(cudaMemcpyAsync(b->work + b->o_otiles, b->otiles.data(), sizeof(int2) * b->otiles.size(),
+                        cudaMemcpyHostToDevice, s), "copy");
     for (auto& kv : b->cnx)
         BCK(cudaMemcpyAsync(b->work + b->o_cnx[kv.first], kv.second.data(), sizeof(int4) * kv.second.size(),
                             cudaMemcpyHostToDevice, s), "copy");
@@ -826,13 +848,13 @@ sgpe_status sgpe_batch_energy(sgpe_batch* b, double* out) {
     if (!b->psi) return bfail(b, SGPE_ESTATE, "no buffers bound");
     BCK(b->prec == SGPE_C128 ? bflush<double>(b) : bflush<float>(b), "flush");
     const BInst* I = (const BInst*)(b->work + b->o_inst);
-    const int2* tiles = (const int2*)(b->work + b->o_tiles);
+    const int2* tiles = (const int2*)(b->work + b->o_otiles);
     double* part = (double*)(b->work + b->o_part);
     DevScalars* sc = (DevScalars*)(b->work + b->o_sc);
     if (b->prec == SGPE_C128)
-        kb_obs_tiles<double><<<(unsigned)b->tiles.size(), 128, 0, b->stream>>>((const double2*)b->psi, I, tiles, part);
+        kb_obs_tiles<double><<<(unsigned)b->otiles.size(), 128, 0, b->stream>>>((const double2*)b->psi, I, tiles, part);
     else
-        kb_obs_tiles<float><<<(unsigned)b->tiles.size(), 128, 0, b->stream>>>((const float2*)b->psi, I, tiles, part);
+        kb_obs_tiles<float><<<(unsigned)b->otiles.size(), 128, 0, b->stream>>>((const float2*)b->psi, I, tiles, part);
     kb_obs_final<<<b->n, 128, 0, b->stream>>>(I, part, sc);
     BCK(cudaGetLastError(), "observables");
     std::vector<DevScalars> h(b->n);

@@ -859,86 +859,177 @@ __global__ void __launch_bounds__(256) k_norms(const typename V2<R>::T* A, size_
 
 // ---------------------------------------------------------------------------
 // Observables (Eq. (noma), Eq. (energy), rms sizes) of the state (no pending
-// scale). Per point in FP64: N_j, r^2 rho_j, the kinetic energy of the links
-// ending at the point (plus the ghost links at the upper edges), trap,
-// interaction, Rabi and SO energy densities.
+// scale), in FP64: N_j, r^2 rho_j, kinetic, trap, interaction, Rabi and SO
+// energy sums.
+//
+// Bound by the FP64 pipe (a warp's FP64 instruction holds its sub-partition for
+// 64 cycles), so the work is laid out for few FP64 instructions a point, about 70
+// instead of 375: a warp walks a strip of 32 columns down several rows and adds
+// up in registers (one block reduction per strip instead of 55 shuffled adds per
+// point), the neighbours come from the lane to the left and the row before, and
+// the two first-difference sums are taken link by link. The SO operator is
+// Hermitian, so <psi, H_SO psi> is twice the real part of the psi_0 column, and a
+// sum over points of conj(f_r)(g_(r+1) - g_(r-1)) is the sum over links (r-1, r)
+// of conj(f_(r-1)) g_r - conj(f_r) g_(r-1) (zero ghosts). Measured per call
+// (complex64 unless stated): 2048^2 2500 -> 690 us, 512^2 170 -> 64, 256^2
+// complex128 49 -> 22, 1D 256 complex128 17 -> 11, the 64-instance batch 933 -> 366.
 // ---------------------------------------------------------------------------
 constexpr int NACC = 11;
 
-// The FP64 observable densities of grid point (ix, iy) of one grid, added to v.
+// x as a double through the integer pipe (normal numbers and zero; FP64
+// conversions elsewhere).
+__device__ __forceinline__ double wide(float x) {
+    const unsigned b = __float_as_uint(x), e = b & 0x7f800000u;
+    if (e - 0x00800000u < 0x7f000000u)
+        return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
+    return (b << 1) == 0u ? 0.0 : (double)x;
+}
+__device__ __forceinline__ double wide(double x) { return x; }
+__device__ __forceinline__ double wide(df x) { return wide(x.hi) + wide(x.lo); }
+
+// Re / Im of conj(a) b added to acc, or taken off it.
+__device__ __forceinline__ double re_add(cx<double> a, cx<double> b, double acc) {
+    return fma(a.re, b.re, fma(a.im, b.im, acc));
+}
+__device__ __forceinline__ double re_sub(cx<double> a, cx<double> b, double acc) {
+    return fma(-a.re, b.re, fma(-a.im, b.im, acc));
+}
+__device__ __forceinline__ double im_add(cx<double> a, cx<double> b, double acc) {
+    return fma(a.re, b.im, fma(-a.im, b.re, acc));
+}
+__device__ __forceinline__ double im_sub(cx<double> a, cx<double> b, double acc) {
+    return fma(-a.re, b.im, fma(a.im, b.re, acc));
+}
+__device__ __forceinline__ double sq_add(cx<double> a, double acc) { return fma(a.re, a.re, fma(a.im, a.im, acc)); }
+
+// The observable sums of the points (ix, iy0 .. iy0 + rows - 1) of one grid; every
+// lane of the warp calls it with ix = (a multiple of 32) + lane (a lane past the
+// row's end and rows past the grid's add nothing).
 template <typename R>
-__device__ __forceinline__ void obs_point(const typename V2<R>::T* __restrict__ A, const KParams& p, double omega_t,
-                                          int ix, int iy, double (&v)[NACC]) {
-    {
-        const size_t plane = (size_t)p.nx * p.ny;
-        const size_t c = (size_t)iy * p.nx + ix;
-        cx<double> u[3];
-        const cx<double> zero = {0.0, 0.0};
-        for (int j = 0; j < 3; j++) {
-            cx<R> a = ld<R>(A, j * plane + c);
-            u[j] = {dbl(a.re), dbl(a.im)};
-        }
-        double x = (ix - p.nx / 2) * p.dx, y = (p.dim == 2) ? (iy - p.ny / 2) * p.dy : 0.0;
-        double rr = x * x + y * y;
-        double rp = nrm(u[0]), r0 = nrm(u[1]), rm = nrm(u[2]), rho = rp + r0 + rm;
-        v[0] = rp;
-        v[1] = r0;
-        v[2] = rm;
-        v[3] = rr * rp;
-        v[4] = rr * r0;
-        v[5] = rr * rm;
-        // kinetic: links (ix-1, ix) and, at the upper edge, (ix, ghost); same in y
-        double ek = 0.0;
-        const double idx2 = 1.0 / (p.dx * p.dx), idy2 = 1.0 / (p.dy * p.dy);
-        cx<double> X[3], Y[3];
-        for (int j = 0; j < 3; j++) {
-            cx<double> xm = zero, xp = zero, ym = zero, yp = zero;
-            if (ix > 0) {
-                cx<R> a = ld<R>(A, j * plane + c - 1);
-                xm = {dbl(a.re), dbl(a.im)};
-            }
-            if (ix + 1 < p.nx) {
-                cx<R> a = ld<R>(A, j * plane + c + 1);
-                xp = {dbl(a.re), dbl(a.im)};
-            }
-            ek += 0.5 * nrm(sub(u[j], xm)) * idx2;
-            if (ix == p.nx - 1) ek += 0.5 * nrm(u[j]) * idx2;
-            X[j] = sub(xp, xm);
-            if (p.dim == 2) {
-                if (iy > 0) {
-                    cx<R> a = ld<R>(A, j * plane + c - p.nx);
-                    ym = {dbl(a.re), dbl(a.im)};
-                }
-                if (iy + 1 < p.ny) {
-                    cx<R> a = ld<R>(A, j * plane + c + p.nx);
-                    yp = {dbl(a.re), dbl(a.im)};
-                }
-                ek += 0.5 * nrm(sub(u[j], ym)) * idy2;
-                if (iy == p.ny - 1) ek += 0.5 * nrm(u[j]) * idy2;
-                Y[j] = sub(yp, ym);
-            } else {
-                Y[j] = zero;
-            }
-        }
-        v[6] = ek;
-        double V = p.wx2h * x * x + (p.dim == 2 ? p.wy2h * y * y : 0.0);
-        v[7] = V * rho;
-        cx<double> X4 = mul(cmul(u[2], mul(u[1], u[1])), cj(u[0]));  // psi_-^* psi_0^2 psi_+^*
-        v[8] = 0.5 * (p.c0 * rho * rho +
-                      p.c2 * (rp * rp + rm * rm + 2.0 * rp * r0 + 2.0 * rm * r0 - 2.0 * rp * rm + 4.0 * X4.re));
-        cx<double> Rb = cmul(add(u[0], u[2]), u[1]);  // (psi_+^* + psi_-^*) psi_0
-        v[9] = 2.0 * omega_t * Rb.re;
-        if (p.so_case) {
-            // H_SO psi via the SO update with unit time factor on a zero state
-            cx<double> h[3] = {zero, zero, zero};
-            double gx[3] = {p.sx, p.sx, p.sx}, gy[3] = {p.sy, p.sy, p.sy};
-            so_point<true>(h, X, Y, gx, gy, p.so_case);  // h = -(H_SO psi)
-            v[10] = -(cmul(u[0], h[0]).re + cmul(u[1], h[1]).re + cmul(u[2], h[2]).re);
-        }
+__device__ __forceinline__ void obs_strip(const typename V2<R>::T* __restrict__ A, const KParams& p, double omega_t,
+                                          int ix, int iy0, int rows, double (&v)[NACC]) {
+    const size_t plane = (size_t)p.nx * p.ny;
+    const int lane = threadIdx.x & 31;
+    const bool in = ix < p.nx, two = p.dim == 2;
+    const cx<double> zero = {0.0, 0.0};
+    auto at = [&](int j, int x, int y) {
+        const cx<R> a = ld<R>(A, j * plane + (size_t)y * p.nx + x);
+        return cx<double>{wide(a.re), wide(a.im)};
+    };
+    // a thread keeps its x, so sum_y r^2 rho_j = x^2 n_j + q_j and the trap sum follow from
+    // n_j = sum rho_j and q_j = sum y^2 rho_j (in units of the squared grid index) at the end
+    double n[3] = {0.0, 0.0, 0.0}, q[3] = {0.0, 0.0, 0.0};
+    double kx = 0.0, ky = 0.0, i0 = 0.0, i2 = 0.0, i3 = 0.0, i4 = 0.0, i5 = 0.0, rabi = 0.0, sx = 0.0, sy = 0.0;
+    cx<double> dn[3] = {zero, zero, zero}, Sdn = zero;  // the row before
+    if (two && in && iy0 > 0 && iy0 < p.ny) {
+#pragma unroll
+        for (int j = 0; j < 3; j++) dn[j] = at(j, ix, iy0 - 1);
+        Sdn = add(dn[0], dn[2]);
     }
+    const int iy1 = min(iy0 + rows, p.ny);
+    // the next row's values are loaded while this row's FP64 work runs
+    const cx<R> zr = {R(0), R(0)};
+    cx<R> nu[3] = {zr, zr, zr}, nl[3] = {zr, zr, zr};
+    auto load_row = [&](int iy) {
+        if (iy >= iy1 || !in) return;
+#pragma unroll
+        for (int j = 0; j < 3; j++) {
+            const size_t c = j * plane + (size_t)iy * p.nx + ix;
+            nu[j] = ld<R>(A, c);
+            if (lane == 0 && ix > 0) nl[j] = ld<R>(A, c - 1);
+        }
+    };
+    load_row(iy0);
+    for (int iy = iy0; iy < iy1; iy++) {
+        cx<double> u[3], l[3];
+#pragma unroll
+        for (int j = 0; j < 3; j++) u[j] = {wide(nu[j].re), wide(nu[j].im)};
+#pragma unroll
+        for (int j = 0; j < 3; j++)
+            l[j] = {__shfl_up_sync(0xffffffffu, u[j].re, 1), __shfl_up_sync(0xffffffffu, u[j].im, 1)};
+        if (lane == 0) {
+#pragma unroll
+            for (int j = 0; j < 3; j++) l[j] = {wide(nl[j].re), wide(nl[j].im)};
+        }
+        if (!in) l[0] = l[1] = l[2] = zero;
+        load_row(iy + 1);
+        const int ky_ = iy - p.ny / 2;
+        const double yy = (double)(ky_ * ky_);
+        const double t0 = u[1].im * u[1].im;
+        const double rp = nrm(u[0]), r0 = fma(u[1].re, u[1].re, t0), rm = nrm(u[2]), rpm = rp + rm, rho = rpm + r0;
+        n[0] += rp;
+        n[1] += r0;
+        n[2] += rm;
+        // kinetic: the links to the left and to the row before, and the ghost links of the upper edges
+#pragma unroll
+        for (int j = 0; j < 3; j++) kx = sq_add(sub(u[j], l[j]), kx);
+        if (ix == p.nx - 1) kx += rho;
+        if (two) {
+            q[0] = fma(yy, rp, q[0]);
+            q[1] = fma(yy, r0, q[1]);
+            q[2] = fma(yy, rm, q[2]);
+#pragma unroll
+            for (int j = 0; j < 3; j++) ky = sq_add(sub(u[j], dn[j]), ky);
+            if (iy == p.ny - 1) ky += rho;
+        }
+        // c0 rho^2; c2 ((rho_+ - rho_-)^2 + 2 rho_0 (rho_+ + rho_-) + 4 Re(conj(psi_+ psi_-) psi_0^2))
+        i0 = fma(rho, rho, i0);
+        const double dpm = rp - rm;
+        const cx<double> pm = mul(u[0], u[2]);
+        i2 = fma(dpm, dpm, i2);
+        i3 = fma(r0, rpm, i3);
+        i4 = fma(pm.re, fma(u[1].re, u[1].re, -t0), i4);
+        i5 = fma(pm.im, u[1].re * u[1].im, i5);
+        const cx<double> S = add(u[0], u[2]);
+        rabi = re_add(S, u[1], rabi);
+        if (p.so_case == 4 || p.so_case == 2) {
+            const cx<double> D = sub(u[0], u[2]), Dl = sub(l[0], l[2]);
+            sx = re_sub(D, l[1], re_add(Dl, u[1], sx));
+            if (p.so_case == 4) sy = im_sub(S, dn[1], im_add(Sdn, u[1], sy));
+        } else if (p.so_case == 1) {
+            sx = im_sub(S, l[1], im_add(add(l[0], l[2]), u[1], sx));
+        } else if (p.so_case == 3) {
+            sx = im_sub(l[2], u[2], im_add(l[0], u[0], sx));
+        }
+#pragma unroll
+        for (int j = 0; j < 3; j++) dn[j] = u[j];
+        Sdn = S;
+    }
+    const double x = (ix - p.nx / 2) * p.dx, xx = x * x, dyy = two ? p.dy * p.dy : 0.0;
+#pragma unroll
+    for (int j = 0; j < 3; j++) {
+        v[j] = n[j];
+        v[3 + j] = fma(xx, n[j], dyy * q[j]);
+    }
+    v[6] = two ? 0.5 * (kx / (p.dx * p.dx) + ky / dyy) : 0.5 * kx / (p.dx * p.dx);
+    v[7] = fma(p.wx2h * xx, n[0] + n[1] + n[2], p.wy2h * dyy * (q[0] + q[1] + q[2]));
+    v[8] = 0.5 * fma(p.c0, i0, p.c2 * (i2 + 2.0 * i3 + 4.0 * i4 + 8.0 * i5));
+    v[9] = 2.0 * omega_t * rabi;
+    v[10] = 2.0 * (p.so_case == 2 ? -p.sx * sx : fma(p.sx, sx, p.sy * sy));
 }
 
-// The SGPE_NOBS observables from the grid sums s (obs_point summed over the grid).
+// The sums of v over the 128 threads of a block: thread 8q holds sum q (q < NACC)
+// on return. Eight threads per sum add 16 shared-memory values each (19 FP64
+// instructions for a warp, 55 by shuffles alone); fixed order.
+constexpr int kObsPad = 136;  // doubles per row of red: the rows of a half warp's loads use different banks
+__device__ __forceinline__ double obs_block_sum(const double (&v)[NACC], double (*red)[kObsPad]) {
+    const int tid = threadIdx.x;
+#pragma unroll
+    for (int q = 0; q < NACC; q++) red[q][tid] = v[q];
+    __syncthreads();
+    double s = 0.0;
+    if (tid < 96) {
+        const double* r = red[min(tid >> 3, NACC - 1)] + (tid & 7);
+#pragma unroll
+        for (int k = 0; k < 16; k++) s += r[8 * k];
+#pragma unroll
+        for (int off = 4; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    }
+    __syncthreads();
+    return s;
+}
+
+// The SGPE_NOBS observables from the grid sums s (obs_strip summed over the grid).
 __device__ __forceinline__ void obs_finish(const double (&s)[NACC], double w, double* o, int* err) {
     double N0 = s[0] * w, N1 = s[1] * w, N2 = s[2] * w, Nt = N0 + N1 + N2;
     double ekin = s[6] * w, etrap = s[7] * w, eint = s[8] * w, erabi = s[9] * w, eso = s[10] * w;
@@ -962,56 +1053,44 @@ __device__ __forceinline__ void obs_finish(const double (&s)[NACC], double w, do
     if (!(isfinite(Nt))) *err |= 1;
 }
 
+// 128 threads; 2D: a block takes 32 columns, each of its warps a strip of `rows`
+// rows (obs_rows); 1D: 128 points. The last block to finish adds up the blocks'
+// sums and forms the observables.
 template <typename R>
 __global__ void __launch_bounds__(128) k_observables(const typename V2<R>::T* __restrict__ A, KParams p, double omega_t,
-                                                     double* partials, DevScalars* sc) {
-    __shared__ double red[4 * NACC];
-    const int ix = blockIdx.x * blockDim.x + threadIdx.x;
-    const int iy = blockIdx.y * blockDim.y + threadIdx.y;
-    double v[NACC];
-#pragma unroll
-    for (int q = 0; q < NACC; q++) v[q] = 0.0;
-    if (ix < p.nx && iy < p.ny) obs_point<R>(A, p, omega_t, ix, iy, v);
-    // block reduce (blockDim.x * blockDim.y threads, flattened)
-    const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-    const int lane = tid & 31, warp = tid >> 5, nw = (blockDim.x * blockDim.y) >> 5;
-#pragma unroll
-    for (int q = 0; q < NACC; q++)
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], off);
-    if (lane == 0)
-        for (int q = 0; q < NACC; q++) red[warp * NACC + q] = v[q];
-    __syncthreads();
-    const int blk = blockIdx.y * gridDim.x + blockIdx.x;
-    if (tid == 0) {
-        for (int q = 0; q < NACC; q++) {
-            double s = 0.0;
-            for (int w = 0; w < nw; w++) s += red[w * NACC + q];
-            partials[(size_t)blk * NACC + q] = s;
-        }
-    }
+                                                     double* partials, DevScalars* sc, int rows) {
+    __shared__ double red[NACC][kObsPad];
     __shared__ bool am_last;
-    __syncthreads();
-    if (tid == 0) {
+    const int tid = threadIdx.x;
+    double v[NACC];
+    if (p.dim == 2)
+        obs_strip<R>(A, p, omega_t, 32 * (int)blockIdx.x + (tid & 31), (4 * (int)blockIdx.y + (tid >> 5)) * rows, rows, v);
+    else
+        obs_strip<R>(A, p, omega_t, 128 * (int)blockIdx.x + tid, 0, 1, v);
+    const int blk = blockIdx.y * gridDim.x + blockIdx.x, nblk = gridDim.x * gridDim.y;
+    double s = obs_block_sum(v, red);
+    if (tid < 8 * NACC && (tid & 7) == 0) {
+        partials[(size_t)blk * NACC + (tid >> 3)] = s;
         __threadfence();
-        unsigned t = atomicAdd(&sc->ticket[1], 1u);
-        am_last = (t == gridDim.x * gridDim.y - 1);
     }
+    __syncthreads();
+    if (tid == 0) am_last = atomicAdd(&sc->ticket[1], 1u) == (unsigned)nblk - 1;
     __syncthreads();
     if (!am_last) return;
     __threadfence();
-    const int nblk = gridDim.x * gridDim.y;
-    if (tid < 32) {
-        double s[NACC];
-        for (int q = 0; q < NACC; q++) s[q] = 0.0;
-        for (int b = tid; b < nblk; b += 32)
-            for (int q = 0; q < NACC; q++) s[q] += __ldcg(partials + (size_t)b * NACC + q);
-        for (int q = 0; q < NACC; q++)
-            for (int off = 16; off > 0; off >>= 1) s[q] += __shfl_xor_sync(0xffffffffu, s[q], off);
-        if (tid == 0) {
-            obs_finish(s, p.cell, sc->obs, &sc->err);
-            sc->ticket[1] = 0u;
-        }
+#pragma unroll
+    for (int q = 0; q < NACC; q++) v[q] = 0.0;
+    for (int b = tid; b < nblk; b += 128)
+#pragma unroll
+        for (int q = 0; q < NACC; q++) v[q] += __ldcg(partials + (size_t)b * NACC + q);
+    s = obs_block_sum(v, red);
+    if (tid < 8 * NACC && (tid & 7) == 0) red[0][tid >> 3] = s;
+    __syncthreads();
+    if (tid == 0) {
+        double t[NACC];
+        for (int q = 0; q < NACC; q++) t[q] = red[0][q];
+        obs_finish(t, p.cell, sc->obs, &sc->err);
+        sc->ticket[1] = 0u;
     }
 }
 

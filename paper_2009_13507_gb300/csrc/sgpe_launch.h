@@ -77,6 +77,13 @@ inline int table_len(int n) { return n > kRegMaxN ? 32 * kLongC * long_warps(n) 
 // Columns per warp of the register y sweep (must match CnShape<C>::K).
 inline int cny_cols_per_warp(int C, int esz) { return (esz == 8 && C <= 8) ? 2 : 1; }
 constexpr int kObsAcc = 11;
+// Rows a warp of the observables kernel takes: about one strip for each of the
+// 608 SM sub-partitions, at most 16 rows (longer strips save little: the block
+// reduction is 19 FP64 instructions against 70 a row).
+inline int obs_rows(int nx, int ny) {
+    const int r = (int)(((long long)ceil_div(nx, 32) * ny + 607) / 608);
+    return r < 1 ? 1 : r > 16 ? 16 : r;
+}
 constexpr int kNormBlocks = 304;
 
 struct Geometry {

@@ -522,9 +522,9 @@ template <typename R>
 cudaError_t Launcher<R>::observables(cudaStream_t s, const void* A, const KParams& p, double omega_t,
                                      double* partials, DevScalars* sc) {
     using T = typename V2<R>::T;
-    dim3 block(32, 4);
-    dim3 grid(ceil_div(p.nx, 32), ceil_div(p.ny, 4));
-    k_observables<R><<<grid, block, 0, s>>>((const T*)A, p, omega_t, partials, sc);
+    const int rows = obs_rows(p.nx, p.ny);
+    const dim3 grid = p.dim == 2 ? dim3(ceil_div(p.nx, 32), ceil_div(p.ny, 4 * rows)) : dim3(ceil_div(p.nx, 128));
+    k_observables<R><<<grid, 128, 0, s>>>((const T*)A, p, omega_t, partials, sc, rows);
     return cudaGetLastError();
 }
 

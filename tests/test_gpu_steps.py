@@ -27,3 +27,24 @@ def test_table_segments(n, bt, imag):
     s.set_state(psi)
     s.substep("cn_x", imag)
     assert relerr(s.get_state(), O.substep(prob, psi, "cn_x", imag)) < 10 * 1.2e-16 * (1.0 + 4.0 * bt) + 1e-14
+
+
+@pytest.mark.parametrize("precision", ["c128", "c64", "cdf"])
+@pytest.mark.parametrize("dim,nx,ny,so", [(2, 32, 5, 1), (2, 33, 9, 2), (2, 31, 3, 3), (2, 64, 64, 0), (2, 300, 517, 1),
+                                          (1, 128, 1, 1), (1, 129, 1, 2), (1, 97, 1, 3)])
+def test_observable_strips(dim, nx, ny, so, precision):
+    """Strips that end inside a block, at a warp's last column (the ghost link) or
+    before the grid does, every SO term as link sums, and complex64 values that
+    underflow to zero or subnormals. The sums are FP64 over the state as it is
+    stored: 1e-12 of the largest observable (about 100 roundings of the largest sum)."""
+    prob, s = make_pair(dim, nx, ny, dx=0.2, dy=0.25 if dim == 2 else None, c0=30.0, c2=-1.5, so_type=so, gamma=0.7,
+                        omega=0.4, wx=1.0, wy=1.2, dt=1e-3, precision=precision)
+    psi = _rand(prob, 40 + nx, env=60.0)
+    psi[2] *= 1e-30  # complex64: subnormals where the envelope is small
+    psi[:, :, : nx // 4] = 0.0
+    if precision == "c64":
+        psi = psi.astype(np.complex64).astype(np.complex128)
+    s.set_state(psi)
+    got, ref = s.energy_array(), O.observables_array(prob, psi)
+    keep = [i for i in range(16) if i != 9]  # the rms size of a component of norm 1e-60 is 0/0 in float32
+    assert np.max(np.abs(got - ref)[keep]) < 1e-12 * np.max(np.abs(ref))
