@@ -230,7 +230,7 @@ sgpe_status sgpe_substep(sgpe_ctx* ctx, int which, int imag, double omega);
  * points an axis, which launch all four kinds) kind 0 is a fused kernel (pending
  * scale, pointwise substeps and the x sweep), kind 1 has no launches, and the end
  * of step runs inside kinds 0 and 2 (kind 3 has no launches; one untimed
- * end-of-steps launch follows the last step). On complex64 2D grids with even
+ * end-of-steps launch follows the last step). On complex64 2D grids with
  * rows of 1025..2048 points kind 0 is the fused pointwise + x-sweep kernel too
  * and kind 1 has no launches (kind 3 only in imaginary time).
  * Advances the state exactly like the step functions. Synchronises the stream.
@@ -424,7 +424,8 @@ sgpe_status sgpe_batch_autotune(sgpe_batch* b, int nsteps, int* choice);
  * beyond rounding. */
 sgpe_status sgpe_batch_set_tiles(sgpe_batch* b, int x, int y);
 
-/* Kernel launches per batched step; last error of a batch; release (not the buffers). */
+/* Kernel launches per batched step (with the fused x part the 1D instances take one
+ * launch per call for all its steps, not counted here); last error of a batch; release (not the buffers). */
 int sgpe_batch_launches_per_step(const sgpe_batch* b);
 const char* sgpe_batch_last_error(const sgpe_batch* b);
 sgpe_status sgpe_batch_destroy(sgpe_batch* b);
@@ -434,7 +435,7 @@ sgpe_status sgpe_batch_destroy(sgpe_batch* b);
  * accounting): 2 on 2D grids with lines of at most 1024 points whose step needs
  * no finalize launch (the register path; the tiled complex64 path of grids of
  * 129..1024 points an axis), plus one end-of-steps launch per sgpe_step_imag /
- * sgpe_step_real call; 3 on complex64 grids with even rows of 1025..2048 points
+ * sgpe_step_real call; 3 on complex64 grids with rows of 1025..2048 points
  * (fused pointwise + x sweep, row-tiled y sweep, finalize) and 4 on other 2D
  * paths (double-float tiled grids, longer lines); 0 on 1D grids whose whole step
  * loop is one launch per call (lines of at most 1024 points in SGPE_C64 and

@@ -9,6 +9,10 @@
 //               the register kernels are compiled per C)
 //   CN along y  one warp per column or column pair (2D instances), one launch per C
 //   finalize    one block per instance (norms, renormalisation scale)
+// With the fused row kernel the 1D instances leave the per-step launches: one
+// block each runs all steps of a call (or graph) in one launch, beside the 2D
+// instances' launches on streams of the batch's own. The kernels of one kind that
+// differ in C (or row parity) run side by side too.
 // The x part and the warps per block of the sweeps are chosen by
 // sgpe_batch_autotune (or set by sgpe_batch_set_tiles).
 #include <math.h>
@@ -72,18 +76,16 @@ __global__ void __launch_bounds__(128) kb_pointwise(const typename V2<R>::T* __r
     pointwise_at<R, IMAG>(A + I.off, B + I.off, I.p, scs + tl.x, kc<R>(I.p, KC_OMEGA), ix, iy, 7);
 }
 
-// Fused row kernel (the batched form of k_pwx): one block per row of one
-// instance, work entry (instance, row iy, first partial slot or -1). The
-// pointwise substeps (pending scale of the instance, SO, CALCNU, HERM) of the
-// row's points are staged in shared memory in the lanes' chunk layout, then
-// warp j solves the x line of component j. 2D rows go to B for the y sweep; a 1D
-// instance is one row, written back to A in place (every read of the row is done
-// before the staging barrier) with its three norm partials.
+// Fused row kernel (the batched form of k_pwx): one block per row of one 2D
+// instance, work entry (instance, row iy). The pointwise substeps (pending scale
+// of the instance, SO, CALCNU, HERM) of the row's points are staged in shared
+// memory in the lanes' chunk layout, then warp j solves the x line of component j
+// into B for the y sweep.
 template <typename R, bool IMAG, int C>
 __global__ void __launch_bounds__(kPwxThreads, pwx_min_blocks<R, C, IMAG>())
-    kb_pwx(typename V2<R>::T* A, typename V2<R>::T* B, const BInst* __restrict__ insts,
+    kb_pwx(const typename V2<R>::T* __restrict__ A, typename V2<R>::T* __restrict__ B, const BInst* __restrict__ insts,
            const typename V2<R>::T* __restrict__ pool, const int4* __restrict__ rows,
-           const DevScalars* __restrict__ scs, double* partials) {
+           const DevScalars* __restrict__ scs) {
     using T = typename V2<R>::T;
     extern __shared__ __align__(16) unsigned char kbpwx_smem[];
     T* row = reinterpret_cast<T*>(kbpwx_smem);
@@ -119,11 +121,26 @@ __global__ void __launch_bounds__(kPwxThreads, pwx_min_blocks<R, C, IMAG>())
     if (warp < 3) {
         const T* r = row + warp * S;
         const Tabs<R> t = inst_tabs<R>(pool, I, IMAG ? 0 : 1, 0);
-        T* out = (p.dim == 2 ? B : A) + I.off;
         const size_t base = ((size_t)warp * p.ny + iy) * nx;
-        cnx_solve_line<R, IMAG, C>([&](int i) { return unpack(r[(i / C) * (C + 1) + (i % C)]); }, out, base, nx, t,
-                                   e.z >= 0 ? partials + e.z + warp : nullptr);
+        cnx_solve_line<R, IMAG, C>([&](int i) { return unpack(r[(i / C) * (C + 1) + (i % C)]); }, B + I.off, base, nx, t,
+                                   nullptr);
     }
+}
+
+// The whole step loop of the 1D instances of one chunk length, one block each
+// (step1d_loop; ids: their instance numbers). Step by step they cost a launch per
+// chunk length and step, each as long as the latency of its longest line (19, 45
+// and 36 us of the 244 us of a step of the 64-instance complex64 workload, whose 50
+// steps went from 12.2 to 5.2 ms together with the odd rows on the tiled step); here
+// they run under the 2D instances' launches.
+template <typename R, bool IMAG, int C>
+__global__ void __launch_bounds__(kStep1dThreads, 1)
+    kb_step1d(typename V2<R>::T* A, const BInst* __restrict__ insts, const typename V2<R>::T* __restrict__ pool,
+              const int* __restrict__ ids, DevScalars* scs, int nsteps) {
+    const int i = ids[blockIdx.x];
+    const BInst& I = insts[i];
+    step1d_loop<R, IMAG, C>(A + I.off, I.p, scs + i, nullptr, inst_tabs<R>(pool, I, IMAG ? 0 : 1, 0), nsteps,
+                            IMAG ? I.p.renorm : 0);
 }
 
 // Work entry of the x sweep: (instance, line, partial slot or -1).
@@ -156,12 +173,13 @@ __global__ void kb_cny(typename V2<R>::T* A, const typename V2<R>::T* B, const B
 // Shortest axis of a batch instance on the tiled step.
 constexpr int kBatchMidMinN = 128;
 
-// Tiled instances (complex64 2D grids of 128..1024 points an axis with even rows,
+// Tiled instances (complex64 2D grids of 128..1024 points an axis,
 // the constant-factor form in both time modes): the kernels of the single-grid
 // tiled step through work lists. uni holds the instances' constant-factor forms as
 // Tabs, [instance][mode][axis].
-// Row entry: (instance, row, -, -); one launch per warps-a-line count (blockDim 96 nwl).
-template <bool IMAG>
+// Row entry: (instance, row, -, -); one launch per warps-a-line count (blockDim 96 nwl)
+// and row parity.
+template <bool IMAG, bool EVEN>
 __global__ void __launch_bounds__(96 * kPwxLongMaxGroupWarps, 2)
     kb_pwx_long(const float2* __restrict__ A, float2* __restrict__ B, const BInst* __restrict__ insts,
                 const Tabs<float>* __restrict__ uni, const int4* __restrict__ rows,
@@ -172,7 +190,7 @@ __global__ void __launch_bounds__(96 * kPwxLongMaxGroupWarps, 2)
     float Ot;
     pair_constants(I.p, scs + e.x, nullptr, 7, ds, Ot);
     const Tabs<float> t = uni[4 * e.x + (IMAG ? 0 : 2)];
-    pwx_long_row<IMAG, false>(A + I.off, B + I.off, I.p, ds, Ot, t, 7, e.y);
+    pwx_long_row<IMAG, false, EVEN>(A + I.off, B + I.off, I.p, ds, Ot, t, 7, e.y);
 }
 
 // Tile entry: (instance, component j + 4 column tile, row tile, partial slot); one
@@ -188,12 +206,13 @@ __global__ void __launch_bounds__(32 * (kTileReal + 2 * HC), (tile_min_blocks<fl
     if (threadIdx.x == 0) partials[e.w] = (double)sum.hi + (double)sum.lo;
 }
 
-// One block per instance: sum its partial slots in order, publish norms and the
+// One block per instance of ids: sum its partial slots in order, publish norms and the
 // next pending scale (imaginary time with renorm != 0), advance its step count.
-__global__ void __launch_bounds__(128) kb_finalize(const BInst* __restrict__ insts, const double* partials,
-                                                   DevScalars* scs, int imag) {
+__global__ void __launch_bounds__(128) kb_finalize(const BInst* __restrict__ insts, const int* __restrict__ ids,
+                                                   const double* partials, DevScalars* scs, int imag) {
     __shared__ double red[4 * 3];
-    const BInst& I = insts[blockIdx.x];
+    const int inst = ids[blockIdx.x];
+    const BInst& I = insts[inst];
     double s[3] = {0.0, 0.0, 0.0};
     // slots of component j: [slot0 + j*m, slot0 + (j+1)*m)
     const int m = I.nslot / 3;
@@ -205,7 +224,7 @@ __global__ void __launch_bounds__(128) kb_finalize(const BInst* __restrict__ ins
     }
     block_reduce<3>(s, red);
     if (threadIdx.x == 0) {
-        DevScalars* sc = scs + blockIdx.x;
+        DevScalars* sc = scs + inst;
         double N[3] = {s[0] * I.p.cell, s[1] * I.p.cell, s[2] * I.p.cell};
         bool finite = isfinite(N[0]) && isfinite(N[1]) && isfinite(N[2]);
         double d[3];
@@ -299,6 +318,11 @@ using namespace sgpe;
 // ---------------------------------------------------------------------------
 // Host side
 // ---------------------------------------------------------------------------
+// Side streams: kLoopStreams for the 1D step loops (one per chunk length), the rest
+// for the kernels of one kind of a step.
+constexpr int kLoopStreams = 6;
+constexpr int kSideStreams = kLoopStreams + 7;
+
 struct BGraphKey {
     int imag, count;
     bool operator<(const BGraphKey& o) const { return imag != o.imag ? imag < o.imag : count < o.count; }
@@ -315,7 +339,11 @@ struct sgpe_batch {
     std::vector<int2> otiles;   // every instance's observable blocks
     std::vector<int2> pwtiles;  // the tiles of the pointwise kernel (instances on the register path)
     std::map<int, std::vector<int4>> cnx, cny, rows;  // work lists by chunk length (rows: the fused x part)
-    // tiled instances (complex64): row entries by warps a line, tile entries by halo depth
+    std::vector<int> ids;                  // instance numbers: the 2D instances, then the 1D instances by chunk length
+    int n2d;                               // 2D instances
+    std::map<int, std::pair<int, int>> l1; // 1D instances by chunk length: first place in ids, count
+    std::map<int, int> n1max;              // their longest line
+    // tiled instances (complex64): row entries by 2 x warps a line + row parity, tile entries by halo depth
     std::vector<char> tiled;
     std::map<int, std::vector<int4>> rows_t, ytile;
     size_t state_elems;
@@ -323,7 +351,7 @@ struct sgpe_batch {
     int nslots;
     // workspace layout (byte offsets)
     size_t o_inst, o_sc, o_tiles, o_part, o_tab, o_mid, total;
-    size_t o_pwtiles, o_otiles, o_uni, o_us;
+    size_t o_pwtiles, o_otiles, o_ids, o_uni, o_us;
     std::map<int, size_t> o_cnx, o_cny, o_rows, o_rows_t, o_ytile;
     // bound buffers
     void* psi;
@@ -333,6 +361,9 @@ struct sgpe_batch {
     int wx, wy;
     std::map<BGraphKey, cudaGraphExec_t> graphs;
     bool graphs_ok;
+    // the batch's own streams (kernels that may run side by side) and the events that order them
+    cudaStream_t side[kSideStreams];
+    cudaEvent_t ev_side[kSideStreams], ev_fork, ev_fork1;
     char err[512];
 };
 
@@ -360,10 +391,9 @@ static void binvalidate(sgpe_batch* b) {
 }
 
 template <typename R, bool IMAG, int C>
-static void kb_pwx_c(dim3 grid, dim3 block, cudaStream_t s, typename V2<R>::T* A, typename V2<R>::T* B,
-                     const BInst* I, const typename V2<R>::T* pool, const int4* w, const DevScalars* sc,
-                     double* part) {
-    kb_pwx<R, IMAG, C><<<grid, block, pwx_smem_bytes<R, C>(), s>>>(A, B, I, pool, w, sc, part);
+static void kb_pwx_c(dim3 grid, dim3 block, cudaStream_t s, const typename V2<R>::T* A, typename V2<R>::T* B,
+                     const BInst* I, const typename V2<R>::T* pool, const int4* w, const DevScalars* sc) {
+    kb_pwx<R, IMAG, C><<<grid, block, pwx_smem_bytes<R, C>(), s>>>(A, B, I, pool, w, sc);
 }
 
 // Shared-memory allowance of the fused row kernels (rows of 1024 points stage 51 KB).
@@ -376,7 +406,58 @@ template <typename R, bool IMAG> static cudaError_t kb_pwx_allow() {
     return e;
 }
 
-// Enqueue one step for all instances.
+template <typename R, bool IMAG> static cudaError_t kb_step1d_allow() {
+    cudaError_t e = cudaFuncSetAttribute(kb_step1d<R, IMAG, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)step1d_smem_bytes<R, 16>(32 * 16));
+    if (!e) e = cudaFuncSetAttribute(kb_step1d<R, IMAG, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)step1d_smem_bytes<R, 32>(32 * 32));
+    return e;
+}
+template <typename R, bool IMAG, int C>
+static cudaError_t kb_step1d_c(unsigned blocks, int nxmax, cudaStream_t s, typename V2<R>::T* A, const BInst* I,
+                               const typename V2<R>::T* pool, const int* ids, DevScalars* sc, int nsteps) {
+    kb_step1d<R, IMAG, C><<<blocks, kStep1dThreads, step1d_smem_bytes<R, C>(nxmax), s>>>(A, I, pool, ids, sc, nsteps);
+    return cudaGetLastError();
+}
+
+// Fork: the side streams [first, first + count) of the batch start from the main
+// stream's present end; join: the main stream waits for them.
+static cudaError_t bfork(sgpe_batch* b, cudaEvent_t ev, int first, int count) {
+    cudaError_t e = count > 0 ? cudaEventRecord(ev, b->stream) : cudaSuccess;
+    for (int i = first; i < first + count && !e; i++) e = cudaStreamWaitEvent(b->side[i], ev, 0);
+    return e;
+}
+static cudaError_t bjoin(sgpe_batch* b, int first, int count) {
+    cudaError_t e = cudaSuccess;
+    for (int i = first; i < first + count && !e; i++) {
+        e = cudaEventRecord(b->ev_side[i], b->side[i]);
+        if (!e) e = cudaStreamWaitEvent(b->stream, b->ev_side[i], 0);
+    }
+    return e;
+}
+
+// A set of launches that may run side by side: the first on the main stream, the
+// others on side streams in turn.
+struct SideBySide {
+    sgpe_batch* b;
+    int used = 0;
+    cudaError_t e = cudaSuccess;
+    static constexpr int kRoom = kSideStreams - kLoopStreams;
+    template <typename F> void run(int total, F&& f) {
+        if (e) return;
+        if (used == 0 && total > 1) e = bfork(b, b->ev_fork, kLoopStreams, std::min(total - 1, kRoom));
+        if (e) return;
+        f(used == 0 ? b->stream : b->side[kLoopStreams + (used - 1) % kRoom]);
+        e = cudaGetLastError();
+        used++;
+        if (used == total && total > 1 && !e) e = bjoin(b, kLoopStreams, std::min(total - 1, kRoom));
+    }
+};
+
+// Whether the 1D instances run in their step loops (the fused x part).
+static bool loops_1d(const sgpe_batch* b) { return b->wx == 0 && !b->l1.empty(); }
+
+// Enqueue one step for all instances (the 2D instances only where loops_1d).
 template <typename R, bool IMAG>
 static cudaError_t benqueue_step(sgpe_batch* b) {
     using T = typename V2<R>::T;
@@ -384,33 +465,44 @@ static cudaError_t benqueue_step(sgpe_batch* b) {
     T* B = (T*)(b->work + b->o_mid);
     const BInst* I = (const BInst*)(b->work + b->o_inst);
     DevScalars* sc = (DevScalars*)(b->work + b->o_sc);
-    const int2* tiles = (const int2*)(b->work + b->o_tiles);
     double* part = (double*)(b->work + b->o_part);
     const T* pool = (const T*)(b->work + b->o_tab);
+    const int nfin = loops_1d(b) ? b->n2d : b->n;
+    if (nfin == 0) return cudaSuccess;
+    SideBySide px{b}, py{b};
     if (b->wx == 0) {
+        const int total = (int)(b->rows.size() + b->rows_t.size());
         for (auto& kv : b->rows) {
             const int4* w = (const int4*)(b->work + b->o_rows[kv.first]);
             const dim3 grid((unsigned)kv.second.size()), block(kPwxThreads);
-            switch (kv.first) {
-                case 1: kb_pwx_c<R, IMAG, 1>(grid, block, b->stream, A, B, I, pool, w, sc, part); break;
-                case 2: kb_pwx_c<R, IMAG, 2>(grid, block, b->stream, A, B, I, pool, w, sc, part); break;
-                case 4: kb_pwx_c<R, IMAG, 4>(grid, block, b->stream, A, B, I, pool, w, sc, part); break;
-                case 8: kb_pwx_c<R, IMAG, 8>(grid, block, b->stream, A, B, I, pool, w, sc, part); break;
-                case 16: kb_pwx_c<R, IMAG, 16>(grid, block, b->stream, A, B, I, pool, w, sc, part); break;
-                default: kb_pwx_c<R, IMAG, 32>(grid, block, b->stream, A, B, I, pool, w, sc, part); break;
-            }
+            px.run(total, [&](cudaStream_t s) {
+                switch (kv.first) {
+                    case 1: kb_pwx_c<R, IMAG, 1>(grid, block, s, A, B, I, pool, w, sc); break;
+                    case 2: kb_pwx_c<R, IMAG, 2>(grid, block, s, A, B, I, pool, w, sc); break;
+                    case 4: kb_pwx_c<R, IMAG, 4>(grid, block, s, A, B, I, pool, w, sc); break;
+                    case 8: kb_pwx_c<R, IMAG, 8>(grid, block, s, A, B, I, pool, w, sc); break;
+                    case 16: kb_pwx_c<R, IMAG, 16>(grid, block, s, A, B, I, pool, w, sc); break;
+                    default: kb_pwx_c<R, IMAG, 32>(grid, block, s, A, B, I, pool, w, sc); break;
+                }
+            });
         }
     } else if (!b->pwtiles.empty()) {
         const int2* pwt = (const int2*)(b->work + b->o_pwtiles);
         kb_pointwise<R, IMAG><<<(unsigned)b->pwtiles.size(), 128, 0, b->stream>>>(A, B, I, pwt, sc);
     }
+    const int xtotal = (int)(b->wx == 0 ? b->rows.size() + b->rows_t.size() : b->cnx.size() + b->rows_t.size());
     if constexpr (std::is_same<R, float>::value) {
         const Tabs<float>* uni = (const Tabs<float>*)(b->work + b->o_uni);
         for (auto& kv : b->rows_t) {
             const int4* w = (const int4*)(b->work + b->o_rows_t[kv.first]);
-            const size_t sm = (size_t)3 * 32 * kv.first * kLongS * sizeof(cx<float>);
-            kb_pwx_long<IMAG><<<(unsigned)kv.second.size(), 96 * kv.first, sm, b->stream>>>(
-                (const float2*)A, (float2*)B, I, uni, w, sc);
+            const int nwl = kv.first >> 1;
+            const size_t sm = (size_t)3 * 32 * nwl * kLongS * sizeof(cx<float>);
+            px.run(xtotal, [&](cudaStream_t s) {
+                auto go = [&](auto kern) {
+                    kern<<<(unsigned)kv.second.size(), 96 * nwl, sm, s>>>((const float2*)A, (float2*)B, I, uni, w, sc);
+                };
+                (kv.first & 1) ? go(kb_pwx_long<IMAG, false>) : go(kb_pwx_long<IMAG, true>);
+            });
         }
     }
     for (auto& kv : b->cnx) {
@@ -418,27 +510,32 @@ static cudaError_t benqueue_step(sgpe_batch* b) {
         const int4* w = (const int4*)(b->work + b->o_cnx[kv.first]);
         int nw = (int)kv.second.size();
         dim3 grid((nw + b->wx - 1) / b->wx), block(32 * b->wx);
-        switch (kv.first) {
-            case 1: kb_cnx<R, IMAG, 1><<<grid, block, 0, b->stream>>>(A, B, I, pool, w, nw, part); break;
-            case 2: kb_cnx<R, IMAG, 2><<<grid, block, 0, b->stream>>>(A, B, I, pool, w, nw, part); break;
-            case 4: kb_cnx<R, IMAG, 4><<<grid, block, 0, b->stream>>>(A, B, I, pool, w, nw, part); break;
-            case 8: kb_cnx<R, IMAG, 8><<<grid, block, 0, b->stream>>>(A, B, I, pool, w, nw, part); break;
-            case 16: kb_cnx<R, IMAG, 16><<<grid, block, 0, b->stream>>>(A, B, I, pool, w, nw, part); break;
-            default: kb_cnx<R, IMAG, 32><<<grid, block, 0, b->stream>>>(A, B, I, pool, w, nw, part); break;
-        }
+        px.run(xtotal, [&](cudaStream_t s) {
+            switch (kv.first) {
+                case 1: kb_cnx<R, IMAG, 1><<<grid, block, 0, s>>>(A, B, I, pool, w, nw, part); break;
+                case 2: kb_cnx<R, IMAG, 2><<<grid, block, 0, s>>>(A, B, I, pool, w, nw, part); break;
+                case 4: kb_cnx<R, IMAG, 4><<<grid, block, 0, s>>>(A, B, I, pool, w, nw, part); break;
+                case 8: kb_cnx<R, IMAG, 8><<<grid, block, 0, s>>>(A, B, I, pool, w, nw, part); break;
+                case 16: kb_cnx<R, IMAG, 16><<<grid, block, 0, s>>>(A, B, I, pool, w, nw, part); break;
+                default: kb_cnx<R, IMAG, 32><<<grid, block, 0, s>>>(A, B, I, pool, w, nw, part); break;
+            }
+        });
     }
+    const int ytotal = (int)(b->cny.size() + b->ytile.size());
     for (auto& kv : b->cny) {
         const int4* w = (const int4*)(b->work + b->o_cny[kv.first]);
         int nw = (int)kv.second.size();
         dim3 grid((nw + b->wy - 1) / b->wy), block(32 * b->wy);
-        switch (kv.first) {
-            case 1: kb_cny<R, IMAG, 1><<<grid, block, 0, b->stream>>>(A, B, I, pool, w, nw, part); break;
-            case 2: kb_cny<R, IMAG, 2><<<grid, block, 0, b->stream>>>(A, B, I, pool, w, nw, part); break;
-            case 4: kb_cny<R, IMAG, 4><<<grid, block, 0, b->stream>>>(A, B, I, pool, w, nw, part); break;
-            case 8: kb_cny<R, IMAG, 8><<<grid, block, 0, b->stream>>>(A, B, I, pool, w, nw, part); break;
-            case 16: kb_cny<R, IMAG, 16><<<grid, block, 0, b->stream>>>(A, B, I, pool, w, nw, part); break;
-            default: kb_cny<R, IMAG, 32><<<grid, block, 0, b->stream>>>(A, B, I, pool, w, nw, part); break;
-        }
+        py.run(ytotal, [&](cudaStream_t s) {
+            switch (kv.first) {
+                case 1: kb_cny<R, IMAG, 1><<<grid, block, 0, s>>>(A, B, I, pool, w, nw, part); break;
+                case 2: kb_cny<R, IMAG, 2><<<grid, block, 0, s>>>(A, B, I, pool, w, nw, part); break;
+                case 4: kb_cny<R, IMAG, 4><<<grid, block, 0, s>>>(A, B, I, pool, w, nw, part); break;
+                case 8: kb_cny<R, IMAG, 8><<<grid, block, 0, s>>>(A, B, I, pool, w, nw, part); break;
+                case 16: kb_cny<R, IMAG, 16><<<grid, block, 0, s>>>(A, B, I, pool, w, nw, part); break;
+                default: kb_cny<R, IMAG, 32><<<grid, block, 0, s>>>(A, B, I, pool, w, nw, part); break;
+            }
+        });
     }
     if constexpr (std::is_same<R, float>::value) {
         const Tabs<float>* uni = (const Tabs<float>*)(b->work + b->o_uni);
@@ -447,26 +544,58 @@ static cudaError_t benqueue_step(sgpe_batch* b) {
             const int hc = kv.first;
             const size_t sm = (size_t)(kTileReal + 2 * hc) * kLongC * 32 * sizeof(cx<float>);
             const dim3 grid((unsigned)kv.second.size()), block(32 * (kTileReal + 2 * hc));
-            if (hc == 1)
-                kb_cny_tile<IMAG, 1><<<grid, block, sm, b->stream>>>((float2*)A, (const float2*)B, I, uni, w, part);
-            else
-                kb_cny_tile<IMAG, 2><<<grid, block, sm, b->stream>>>((float2*)A, (const float2*)B, I, uni, w, part);
+            py.run(ytotal, [&](cudaStream_t s) {
+                if (hc == 1)
+                    kb_cny_tile<IMAG, 1><<<grid, block, sm, s>>>((float2*)A, (const float2*)B, I, uni, w, part);
+                else
+                    kb_cny_tile<IMAG, 2><<<grid, block, sm, s>>>((float2*)A, (const float2*)B, I, uni, w, part);
+            });
         }
     }
-    kb_finalize<<<b->n, 128, 0, b->stream>>>(I, part, sc, IMAG ? 1 : 0);
+    if (px.e || py.e) return px.e ? px.e : py.e;
+    kb_finalize<<<nfin, 128, 0, b->stream>>>(I, (const int*)(b->work + b->o_ids), part, sc, IMAG ? 1 : 0);
     return cudaGetLastError();
 }
 
-static cudaError_t benqueue_steps(sgpe_batch* b, int n, bool imag) {
-    for (int i = 0; i < n; i++) {
-        cudaError_t e;
-        if (b->prec == SGPE_C128)
-            e = imag ? benqueue_step<double, true>(b) : benqueue_step<double, false>(b);
-        else
-            e = imag ? benqueue_step<float, true>(b) : benqueue_step<float, false>(b);
-        if (e != cudaSuccess) return e;
+// n steps of all instances: the 1D step loops beside the launches of the 2D instances.
+template <typename R, bool IMAG> static cudaError_t benqueue_n(sgpe_batch* b, int n) {
+    using T = typename V2<R>::T;
+    if (n <= 0) return cudaSuccess;
+    cudaError_t e = cudaSuccess;
+    const bool loops = loops_1d(b);
+    const int nl = loops ? (int)b->l1.size() : 0;
+    if (loops) {
+        T* A = (T*)b->psi;
+        const BInst* I = (const BInst*)(b->work + b->o_inst);
+        DevScalars* sc = (DevScalars*)(b->work + b->o_sc);
+        const T* pool = (const T*)(b->work + b->o_tab);
+        const int* ids = (const int*)(b->work + b->o_ids);
+        e = bfork(b, b->ev_fork1, 0, nl);
+        int k = 0;
+        // the longest lines first: they take the longest
+        for (auto it = b->l1.rbegin(); it != b->l1.rend() && !e; ++it, ++k) {
+            const int* w = ids + it->second.first;
+            const unsigned m = (unsigned)it->second.second;
+            const int nm = b->n1max[it->first];
+            cudaStream_t s = b->side[k];
+            switch (it->first) {
+                case 1: e = kb_step1d_c<R, IMAG, 1>(m, nm, s, A, I, pool, w, sc, n); break;
+                case 2: e = kb_step1d_c<R, IMAG, 2>(m, nm, s, A, I, pool, w, sc, n); break;
+                case 4: e = kb_step1d_c<R, IMAG, 4>(m, nm, s, A, I, pool, w, sc, n); break;
+                case 8: e = kb_step1d_c<R, IMAG, 8>(m, nm, s, A, I, pool, w, sc, n); break;
+                case 16: e = kb_step1d_c<R, IMAG, 16>(m, nm, s, A, I, pool, w, sc, n); break;
+                default: e = kb_step1d_c<R, IMAG, 32>(m, nm, s, A, I, pool, w, sc, n); break;
+            }
+        }
     }
-    return cudaSuccess;
+    for (int i = 0; i < n && !e; i++) e = benqueue_step<R, IMAG>(b);
+    const cudaError_t ej = bjoin(b, 0, nl);  // (also after an error: a capture must not leave forked streams)
+    return e ? e : ej;
+}
+
+static cudaError_t benqueue_steps(sgpe_batch* b, int n, bool imag) {
+    if (b->prec == SGPE_C128) return imag ? benqueue_n<double, true>(b, n) : benqueue_n<double, false>(b, n);
+    return imag ? benqueue_n<float, true>(b, n) : benqueue_n<float, false>(b, n);
 }
 
 static sgpe_status brun(sgpe_batch* b, int nsteps, bool imag) {
@@ -594,11 +723,10 @@ sgpe_status sgpe_batch_create(sgpe_batch** out, int n, const sgpe_instance* inst
         I.obs0 = (int)b->otiles.size();
         I.nobs = q.dim == 2 ? ceil_div(q.nx, 32) * ceil_div(q.ny, 4 * kBatchObsRows) : ntile;
         for (int t = 0; t < I.nobs; t++) b->otiles.push_back(make_int2(i, t));
-        // complex64 2D instances of 128..1024 points an axis with even rows take the tiled
-        // step when both axes have the constant-factor form in both time modes (from 128
+        // complex64 2D instances of 128..1024 points an axis take the tiled step when both axes have the constant-factor form in both time modes (from 128
         // points: inside a batch the grouped launches fill the GPU; 64-instance workload
         // 6.87e9 -> 7.49e9 point-steps/s against a 256-point threshold)
-        bool tl = prec == SGPE_C64 && q.dim == 2 && q.nx % 2 == 0 && q.nx >= kBatchMidMinN && q.ny >= kBatchMidMinN;
+        bool tl = prec == SGPE_C64 && q.dim == 2 && q.nx >= kBatchMidMinN && q.ny >= kBatchMidMinN;
         int hcmax = 0;
         for (int m = 0; m < 2 && tl; m++)
             for (int a = 0; a < 2 && tl; a++) {
@@ -620,7 +748,7 @@ sgpe_status sgpe_batch_create(sgpe_batch** out, int n, const sgpe_instance* inst
         I.slot0 = slot;
         if (tl) {
             const int nwl = long_warps(q.nx);
-            for (int r = 0; r < q.ny; r++) b->rows_t[nwl].push_back(make_int4(i, r, 0, 0));
+            for (int r = 0; r < q.ny; r++) b->rows_t[2 * nwl + (q.nx & 1)].push_back(make_int4(i, r, 0, 0));
             const int nct = ceil_div(q.nx, 32), nrt = ceil_div(q.ny, kTileRows);
             for (int j = 0; j < 3; j++)
                 for (int ct = 0; ct < nct; ct++)
@@ -631,11 +759,10 @@ sgpe_status sgpe_batch_create(sgpe_batch** out, int n, const sgpe_instance* inst
         } else if (q.dim == 1) {
             I.nslot = 3;
             for (int l = 0; l < 3; l++) b->cnx[Cx].push_back(make_int4(i, l, slot + l, 0));
-            b->rows[Cx].push_back(make_int4(i, 0, slot, 0));
             slot += 3;
         } else {
             for (int l = 0; l < 3 * q.ny; l++) b->cnx[Cx].push_back(make_int4(i, l, -1, 0));
-            for (int r = 0; r < q.ny; r++) b->rows[Cx].push_back(make_int4(i, r, -1, 0));
+            for (int r = 0; r < q.ny; r++) b->rows[Cx].push_back(make_int4(i, r, 0, 0));
             const int Cy = chunk_len(q.ny);
             const int K = cny_cols_per_warp(Cy, b->esz);
             int cnt = 0;
@@ -646,6 +773,19 @@ sgpe_status sgpe_batch_create(sgpe_batch** out, int n, const sgpe_instance* inst
         }
         b->hinst.push_back(I);
     }
+    // instance numbers: the 2D instances, then the 1D instances by chunk length
+    for (int i = 0; i < n; i++)
+        if (b->hinst[i].p.dim == 2) b->ids.push_back(i);
+    b->n2d = (int)b->ids.size();
+    for (int C = 1; C <= 32; C *= 2)
+        for (int i = 0; i < n; i++) {
+            const KParams& q = b->hinst[i].p;
+            if (q.dim == 2 || chunk_len(q.nx) != C) continue;
+            if (!b->l1.count(C)) b->l1[C] = {(int)b->ids.size(), 0};
+            b->l1[C].second++;
+            b->n1max[C] = std::max(b->n1max[C], q.nx);
+            b->ids.push_back(i);
+        }
     b->state_elems = (size_t)off;
     b->tab_elems = tab;
     b->nslots = slot;
@@ -660,6 +800,8 @@ sgpe_status sgpe_batch_create(sgpe_batch** out, int n, const sgpe_instance* inst
     o = al256(o + sizeof(int2) * b->pwtiles.size());
     b->o_otiles = o;
     o = al256(o + sizeof(int2) * b->otiles.size());
+    b->o_ids = o;
+    o = al256(o + sizeof(int) * b->ids.size());
     for (auto& kv : b->rows_t) {
         b->o_rows_t[kv.first] = o;
         o = al256(o + sizeof(int4) * kv.second.size());
@@ -693,6 +835,17 @@ sgpe_status sgpe_batch_create(sgpe_batch** out, int n, const sgpe_instance* inst
     b->o_mid = o;
     o = al256(o + (size_t)b->esz * b->state_elems);
     b->total = o;
+    cudaError_t e = cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming);
+    if (!e) e = cudaEventCreateWithFlags(&b->ev_fork1, cudaEventDisableTiming);
+    for (int i = 0; i < kSideStreams && !e; i++) {
+        e = cudaStreamCreateWithFlags(&b->side[i], cudaStreamNonBlocking);
+        if (!e) e = cudaEventCreateWithFlags(&b->ev_side[i], cudaEventDisableTiming);
+    }
+    if (e) {
+        set_thread_error("sgpe_batch_create: streams");
+        sgpe_batch_destroy(b);
+        return SGPE_ECUDA;
+    }
     *out = b;
     return SGPE_OK;
 }
@@ -723,6 +876,8 @@ sgpe_status sgpe_batch_bind(sgpe_batch* b, void* psi_dev, void* workspace_dev) {
     BCK(cudaMemsetAsync(b->work + b->o_sc, 0, sizeof(DevScalars) * b->n, s), "memset");
     BCK(cudaMemcpyAsync(b->work + b->o_tiles, b->tiles.data(), sizeof(int2) * b->tiles.size(), cudaMemcpyHostToDevice,
                         s), "copy");
+    BCK(cudaMemcpyAsync(b->work + b->o_ids, b->ids.data(), sizeof(int) * b->ids.size(), cudaMemcpyHostToDevice, s),
+        "copy");
     BCK(cudaMemcpyAsync(b->work + b->o_otiles, b->otiles.data(), sizeof(int2) * b->otiles.size(),
                         cudaMemcpyHostToDevice, s), "copy");
     for (auto& kv : b->cnx)
@@ -788,7 +943,11 @@ sgpe_status sgpe_batch_bind(sgpe_batch* b, void* psi_dev, void* workspace_dev) {
     if (b->prec == SGPE_C128) {
         BCK((kb_pwx_allow<double, true>()), "kernel attributes");
         BCK((kb_pwx_allow<double, false>()), "kernel attributes");
+        BCK((kb_step1d_allow<double, true>()), "kernel attributes");
+        BCK((kb_step1d_allow<double, false>()), "kernel attributes");
     } else {
+        BCK((kb_step1d_allow<float, true>()), "kernel attributes");
+        BCK((kb_step1d_allow<float, false>()), "kernel attributes");
         BCK((kb_pwx_allow<float, true>()), "kernel attributes");
         BCK((kb_pwx_allow<float, false>()), "kernel attributes");
     }
@@ -927,7 +1086,8 @@ sgpe_status sgpe_batch_set_tiles(sgpe_batch* b, int x, int y) {
 int sgpe_batch_launches_per_step(const sgpe_batch* b) {
     if (!b) return 0;
     const int t = (int)b->rows_t.size() + (int)b->ytile.size();
-    if (b->wx == 0) return 1 + (int)b->rows.size() + (int)b->cny.size() + t;
+    // (the 1D step loops are launches per call, not per step)
+    if (b->wx == 0) return (b->n2d ? 1 : 0) + (int)b->rows.size() + (int)b->cny.size() + t;
     return 1 + (b->pwtiles.empty() ? 0 : 1) + (int)b->cnx.size() + (int)b->cny.size() + t;
 }
 
@@ -936,6 +1096,12 @@ const char* sgpe_batch_last_error(const sgpe_batch* b) { return b ? b->err : "nu
 sgpe_status sgpe_batch_destroy(sgpe_batch* b) {
     if (!b) return SGPE_OK;
     binvalidate(b);
+    for (int i = 0; i < kSideStreams; i++) {
+        if (b->side[i]) cudaStreamDestroy(b->side[i]);
+        if (b->ev_side[i]) cudaEventDestroy(b->ev_side[i]);
+    }
+    if (b->ev_fork) cudaEventDestroy(b->ev_fork);
+    if (b->ev_fork1) cudaEventDestroy(b->ev_fork1);
     delete b;
     return SGPE_OK;
 }

@@ -429,10 +429,12 @@ template <typename R, int C> constexpr size_t step1d_smem_bytes(int nx) {
     return ((size_t)3 * nx + (size_t)3 * 32 * (C + 1)) * sizeof(typename V2<R>::T);
 }
 
+// The loop of one grid by the calling block (kStep1dThreads threads,
+// step1d_smem_bytes of dynamic shared memory).
 template <typename R, bool IMAG, int C>
-__global__ void __launch_bounds__(kStep1dThreads, 1)
-    k_step1d(typename V2<R>::T* __restrict__ A, KParams p, DevScalars* sc, const double* __restrict__ omega_tab,
-             Tabs<R> t, int nsteps, int renorm) {
+__device__ __forceinline__ void step1d_loop(typename V2<R>::T* __restrict__ A, const KParams& p, DevScalars* sc,
+                                            const double* __restrict__ omega_tab, const Tabs<R>& t, int nsteps,
+                                            int renorm) {
     using T = typename V2<R>::T;
     extern __shared__ __align__(16) unsigned char step1d_smem[];
     const int nx = p.nx;
@@ -508,6 +510,13 @@ __global__ void __launch_bounds__(kStep1dThreads, 1)
         if (!finite) sc->err |= 1;
         sc->step_idx = step0 + nsteps;
     }
+}
+
+template <typename R, bool IMAG, int C>
+__global__ void __launch_bounds__(kStep1dThreads, 1)
+    k_step1d(typename V2<R>::T* __restrict__ A, KParams p, DevScalars* sc, const double* __restrict__ omega_tab,
+             Tabs<R> t, int nsteps, int renorm) {
+    step1d_loop<R, IMAG, C>(A, p, sc, omega_tab, t, nsteps, renorm);
 }
 
 // ---------------------------------------------------------------------------
@@ -1068,7 +1077,7 @@ constexpr int kPwxLongMaxGroupWarps = 4;
 // point pairs into the three lines' chunk layout in shared memory, the three line
 // solves by the block's warp groups (blockDim = 96 nwl), the lines to B. Every
 // thread of the block calls it.
-template <bool IMAG, bool STD>
+template <bool IMAG, bool STD, bool EVEN>
 __device__ __forceinline__ void pwx_long_row(const float2* __restrict__ A, float2* __restrict__ B, const KParams& p,
                                              const f32x2 (&ds)[3], float Ot, const Tabs<float>& t, int mask, int iy) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1080,12 +1089,12 @@ __device__ __forceinline__ void pwx_long_row(const float2* __restrict__ A, float
     const int span = 32 * kLongC * nwl, S = 32 * nwl * kLongS;
     for (int q = threadIdx.x; 2 * q < nx; q += blockDim.x) {
         cx<f32x2> u[3];
-        pair_substeps<IMAG, STD>(A, p, ds, Ot, mask, 2 * q, iy, u);
+        pair_substeps<IMAG, STD, EVEN>(A, p, ds, Ot, mask, 2 * q, iy, u);
         const int s0 = long_slot(2 * q);  // 2q is even: 2q + 1 sits in the next slot of the same chunk
 #pragma unroll
         for (int j = 0; j < 3; j++) {
             lines[j * S + s0] = cx<float>{u[j].re.v.x, u[j].im.v.x};
-            lines[j * S + s0 + 1] = cx<float>{u[j].re.v.y, u[j].im.v.y};
+            if (EVEN || 2 * q + 1 < nx) lines[j * S + s0 + 1] = cx<float>{u[j].re.v.y, u[j].im.v.y};
         }
     }
     for (int i = nx + threadIdx.x; i < span; i += blockDim.x)
@@ -1104,9 +1113,9 @@ __device__ __forceinline__ void pwx_long_row(const float2* __restrict__ A, float
     }
 }
 
-// Pointwise substeps and CN along x of one row of a 2D complex64 grid with even
+// Pointwise substeps and CN along x of one row of a 2D complex64 grid with
 // rows of at most 2048 points (1025..2048, or the rows of a tiled grid; the
-// constant-factor solve, Tabs::uks > 0): one block per row, 3 groups of nwl =
+// constant-factor solve, Tabs::uks > 0; EVEN: nx is even, see pair_substeps): one block per row, 3 groups of nwl =
 // ceil(nx / 512) warps (one group per component line). The threads evaluate the
 // row's point pairs (pair_substeps) into the padded chunk layout of the three
 // lines in shared memory (slots past nx zero), then group j solves line j
@@ -1114,7 +1123,7 @@ __device__ __forceinline__ void pwx_long_row(const float2* __restrict__ A, float
 // streams the state twice (A -> B here, B -> A in the y sweep) instead of three
 // times. With partials (the tiled step) every block first forms the pending
 // scale from the previous y tiles' norm partials, as k_pwx does.
-template <bool IMAG, bool STD>
+template <bool IMAG, bool STD, bool EVEN>
 __global__ void __launch_bounds__(96 * kPwxLongMaxGroupWarps, 2)
     k_pwx_long(const float2* __restrict__ A, float2* __restrict__ B, KParams p, const DevScalars* __restrict__ sc,
                const double* __restrict__ omega_tab, Tabs<float> t, int mask, const double* __restrict__ partials,
@@ -1148,7 +1157,7 @@ __global__ void __launch_bounds__(96 * kPwxLongMaxGroupWarps, 2)
 #pragma unroll
         for (int j = 0; j < 3; j++) ds[j] = f32x2(dsh[j]);
     }
-    pwx_long_row<IMAG, STD>(A, B, p, ds, Ot, t, mask, iy);
+    pwx_long_row<IMAG, STD, EVEN>(A, B, p, ds, Ot, t, mask, iy);
 }
 
 // CN along y for columns of 1025..8192 points: one block per tile of kc (1, 2

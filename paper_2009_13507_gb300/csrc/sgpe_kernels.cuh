@@ -393,10 +393,21 @@ __global__ void __launch_bounds__(128) k_pointwise(const typename V2<R>::T* __re
 // point is pointwise_apply's, as in k_pointwise. The complex64 pointwise kernel
 // is bound by instruction issue, half of it loads and their index arithmetic.
 // The pointwise substeps of the two neighbouring points (ix, ix + 1) of row iy
-// (complex64, nx even) as one f32x2 pair (lane 0: ix, lane 1: ix + 1): the
-// 16-byte loads of each component's pair, the x and y neighbours (zero ghosts;
-// inner points without the selects), then pointwise_apply.
-template <bool IMAG, bool STD>
+// (complex64) as one f32x2 pair (lane 0: ix, lane 1: ix + 1): the loads of each
+// component's pair and its x and y neighbours (zero ghosts; inner points without
+// the selects), then pointwise_apply. EVEN: nx is even, so a pair is one 16-byte
+// load; odd rows start on 8-byte boundaries and take two 8-byte loads a pair, and
+// their last pair has its second point past the row (it loads as zero; the caller
+// drops its result).
+template <bool EVEN> __device__ __forceinline__ float4 ld_pair(const float2* a) {
+    if constexpr (EVEN) {
+        return __ldg(reinterpret_cast<const float4*>(a));
+    } else {
+        const float2 p = __ldg(a), q = __ldg(a + 1);
+        return make_float4(p.x, p.y, q.x, q.y);
+    }
+}
+template <bool IMAG, bool STD, bool EVEN>
 __device__ __forceinline__ void pair_substeps(const float2* __restrict__ A, const KParams& p, const f32x2 (&ds)[3],
                                               float Ot, int mask, int ix, int iy, cx<f32x2> (&u)[3]) {
     const size_t plane = (size_t)p.nx * p.ny;
@@ -404,11 +415,17 @@ __device__ __forceinline__ void pair_substeps(const float2* __restrict__ A, cons
     const bool so = STD || ((mask & 1) && p.so_case);
     const float4 z4 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     const float2 z2 = make_float2(0.0f, 0.0f);
+    const bool pair = EVEN || ix + 1 < p.nx;  // the second point lies in the row
+    auto ld_edge = [&](const float2* a) {
+        if (EVEN || pair) return ld_pair<EVEN>(a);
+        const float2 q = __ldg(a);
+        return make_float4(q.x, q.y, 0.0f, 0.0f);
+    };
     PointIn<f32x2> in;
     float4 v[3];
 #pragma unroll
     for (int j = 0; j < 3; j++) {
-        v[j] = __ldg(reinterpret_cast<const float4*>(A + j * plane + c));
+        v[j] = ld_edge(A + j * plane + c);
         in.u[j] = {f32x2(v[j].x, v[j].z), f32x2(v[j].y, v[j].w)};
         in.X[j] = in.Y[j] = {f32x2(0.0f), f32x2(0.0f)};
     }
@@ -424,8 +441,7 @@ __device__ __forceinline__ void pair_substeps(const float2* __restrict__ A, cons
 #pragma unroll
             for (int j = 0; j < 3; j++) {
                 const float2* a = A + j * plane + c;
-                diffs(j, __ldg(a - 1), __ldg(a + 2), __ldg(reinterpret_cast<const float4*>(a - p.nx)),
-                      __ldg(reinterpret_cast<const float4*>(a + p.nx)));
+                diffs(j, __ldg(a - 1), __ldg(a + 2), ld_pair<EVEN>(a - p.nx), ld_pair<EVEN>(a + p.nx));
             }
         } else {
             const bool two = STD || p.dim == 2;
@@ -434,8 +450,8 @@ __device__ __forceinline__ void pair_substeps(const float2* __restrict__ A, cons
                 const float2* a = A + j * plane + c;
                 const float2 xm = ix > 0 ? __ldg(a - 1) : z2;
                 const float2 xp = ix + 2 < p.nx ? __ldg(a + 2) : z2;
-                const float4 ym = two && iy > 0 ? __ldg(reinterpret_cast<const float4*>(a - p.nx)) : z4;
-                const float4 yp = two && iy + 1 < p.ny ? __ldg(reinterpret_cast<const float4*>(a + p.nx)) : z4;
+                const float4 ym = two && iy > 0 ? ld_edge(a - p.nx) : z4;
+                const float4 yp = two && iy + 1 < p.ny ? ld_edge(a + p.nx) : z4;
                 diffs(j, xm, xp, ym, yp);
             }
         }
@@ -465,7 +481,7 @@ __global__ void __launch_bounds__(256) k_pointwise2(const float2* __restrict__ A
     float Ot;
     pair_constants(p, sc, omega_tab, mask, ds, Ot);
     cx<f32x2> u[3];
-    pair_substeps<IMAG, STD>(A, p, ds, Ot, mask, ix, iy, u);
+    pair_substeps<IMAG, STD, true>(A, p, ds, Ot, mask, ix, iy, u);
     pdl_trigger();  // the next kernel's blocks may take the slots this grid frees
     const size_t plane = (size_t)p.nx * p.ny;
     const size_t c = (size_t)iy * p.nx + ix;

@@ -230,10 +230,14 @@ template <typename R> cudaError_t Launcher<R>::setup() {
         if ((e = allow_smem(k_cn_y<R, true, true>))) return e;
         if ((e = allow_smem(k_cn_y<R, false, true>))) return e;
         if constexpr (std::is_same<R, float>::value) {
-            if ((e = allow_smem(k_pwx_long<true, true>))) return e;
-            if ((e = allow_smem(k_pwx_long<false, true>))) return e;
-            if ((e = allow_smem(k_pwx_long<true, false>))) return e;
-            if ((e = allow_smem(k_pwx_long<false, false>))) return e;
+            if ((e = allow_smem(k_pwx_long<true, true, true>))) return e;
+            if ((e = allow_smem(k_pwx_long<false, true, true>))) return e;
+            if ((e = allow_smem(k_pwx_long<true, false, true>))) return e;
+            if ((e = allow_smem(k_pwx_long<false, false, true>))) return e;
+            if ((e = allow_smem(k_pwx_long<true, true, false>))) return e;
+            if ((e = allow_smem(k_pwx_long<false, true, false>))) return e;
+            if ((e = allow_smem(k_pwx_long<true, false, false>))) return e;
+            if ((e = allow_smem(k_pwx_long<false, false, false>))) return e;
         }
         if ((e = allow_smem(k_cn_y_tile<R, true, 1, kTileReal>))) return e;
         if ((e = allow_smem(k_cn_y_tile<R, false, 1, kTileReal>))) return e;
@@ -324,7 +328,7 @@ cudaError_t Launcher<R>::pwx_long(cudaStream_t s, bool imag, const void* A, void
         return cudaErrorNotSupported;
     } else {
         const int nwl = long_warps(p.nx);
-        if (p.dim != 2 || p.nx % 2 || nwl > kPwxLongMaxGroupWarps || tabs_x.u.ks <= 0)
+        if (p.dim != 2 || nwl > kPwxLongMaxGroupWarps || tabs_x.u.ks <= 0)
             return cudaErrorInvalidValue;
         const Tabs<float> t = make_tabs<float>(tabs_x);
         KParams q = p;
@@ -335,10 +339,17 @@ cudaError_t Launcher<R>::pwx_long(cudaStream_t s, bool imag, const void* A, void
             launch_pdl(kern, dim3(p.ny), dim3(96 * nwl), smem, s, (const float2*)A, (float2*)B, q, sc, omega_tab, t,
                        mask, partials, m, renorm);
         };
-        if (std2d)
-            imag ? go(k_pwx_long<true, true>) : go(k_pwx_long<false, true>);
-        else
-            imag ? go(k_pwx_long<true, false>) : go(k_pwx_long<false, false>);
+        if (p.nx % 2 == 0) {
+            if (std2d)
+                imag ? go(k_pwx_long<true, true, true>) : go(k_pwx_long<false, true, true>);
+            else
+                imag ? go(k_pwx_long<true, false, true>) : go(k_pwx_long<false, false, true>);
+        } else {
+            if (std2d)
+                imag ? go(k_pwx_long<true, true, false>) : go(k_pwx_long<false, true, false>);
+            else
+                imag ? go(k_pwx_long<true, false, false>) : go(k_pwx_long<false, false, false>);
+        }
         return cudaGetLastError();
     }
 }

@@ -48,3 +48,39 @@ def test_observable_strips(dim, nx, ny, so, precision):
     got, ref = s.energy_array(), O.observables_array(prob, psi)
     keep = [i for i in range(16) if i != 9]  # the rms size of a component of norm 1e-60 is 0/0 in float32
     assert np.max(np.abs(got - ref)[keep]) < 1e-12 * np.max(np.abs(ref))
+
+
+@pytest.mark.parametrize("imag", [True, False])
+@pytest.mark.parametrize("nx,ny", [(129, 130), (257, 140), (511, 129), (1025, 36), (1501, 33)])
+def test_odd_rows_in_the_fused_row_kernel(nx, ny, imag):
+    """complex64 grids with odd rows: 8-byte loads, the last pair's second point past
+    the row, zero ghosts there. The bound is the precision form's 1e-5."""
+    prob, s = make_pair(2, nx, ny, dx=0.05, c0=40.0, c2=1.0, so_type=1, gamma=0.8, omega=0.5, dt=2e-4,
+                        renorm=1 if imag else 0, precision="c64")
+    psi = _rand(prob, nx)
+    s.set_state(psi)
+    (s.step_imag if imag else s.step_real)(12)
+    assert relerr(s.get_state(), O.step(prob, psi, 12, imag)) < 1e-5
+
+
+@pytest.mark.parametrize("precision", ["c128", "c64"])
+def test_batch_of_lines_only(precision):
+    """1D instances in their step loops: every chunk length from 1 to 32 points a
+    lane, the shortest and longest lines, a graph of 32 steps and the rest, both
+    time modes."""
+    from paper_2009_13507_gb300 import sgpe
+    lens = [3, 32, 33, 100, 128, 129, 300, 513, 1024]
+    phys = [dict(c0=5.0 + i, c2=-0.5 + 0.1 * i, so_type=1 + i % 3, gamma=0.5, omega=0.2, dt=2e-3, renorm=1)
+            for i in range(len(lens))]
+    bs = sgpe.BatchSolver([dict(dim=1, nx=n, dx=0.1, **p) for n, p in zip(lens, phys)], precision=precision)
+    states = [I.gaussian_jitter_1d(n, 0.1, seed=n, amp=1e-2) for n in lens]
+    bs.load_state(bs.pack(states))
+    bs.step_imag(40)
+    bs.step_real(5)
+    obs = bs.energy()
+    for i, (n, p) in enumerate(zip(lens, phys)):
+        prob = O.Problem(dim=1, nx=n, ny=1, dx=0.1, dy=0.1, **p)
+        ref = O.step(prob, O.step(prob, states[i], 40, True), 5, False)
+        tol = 1e-10 if precision == "c128" else 1e-5
+        assert relerr(bs.states()[i], ref) < tol, n
+        assert abs(obs[i, 5] - O.observables(prob, ref)["E"]) < tol * max(1.0, abs(obs[i, 5])), n
