@@ -225,14 +225,13 @@ sgpe_status sgpe_substep(sgpe_ctx* ctx, int which, int imag, double omega);
  * context's stream around every kernel; writes the summed device time in ms of
  * each kernel kind to ms_out[0..3] (0 pointwise SO/CALCNU/HERM, 1 Crank-Nicolson
  * along x, 2 along y, 3 end-of-step norm reduction and renormalisation scale;
- * unused kinds 0) and the launch counts to launches_out[0..3]. On 2D grids
- * with lines of at most 1024 points (except double-float grids of 320..1024
- * points an axis, which launch all four kinds) kind 0 is a fused kernel (pending
- * scale, pointwise substeps and the x sweep), kind 1 has no launches, and the end
- * of step runs inside kinds 0 and 2 (kind 3 has no launches; one untimed
- * end-of-steps launch follows the last step). On complex64 2D grids with
- * rows of 1025..2048 points kind 0 is the fused pointwise + x-sweep kernel too
- * and kind 1 has no launches (kind 3 only in imaginary time).
+ * unused kinds 0) and the launch counts to launches_out[0..3]. Where the step
+ * fuses the pointwise substeps and the x sweep (2D complex128 grids; 2D
+ * double-float grids outside the tiled imaginary-time step of 320..~630 points an
+ * axis; complex64 grids with lines of at most 1024 points or rows of at most
+ * 2048) kind 0 is that kernel and kind 1 has no launches. Kind 3 has launches only
+ * where a step ends with one (more than 256 norm partials a component, and the
+ * unfused paths); otherwise one untimed end-of-steps launch follows the last step.
  * Advances the state exactly like the step functions. Synchronises the stream.
  */
 sgpe_status sgpe_profile_steps(sgpe_ctx* ctx, int nsteps, int imag, double* ms_out, int* launches_out);
@@ -432,14 +431,12 @@ sgpe_status sgpe_batch_destroy(sgpe_batch* b);
 
 /*
  * Number of kernel launches one imaginary-time step enqueues (for launch
- * accounting): 2 on 2D grids with lines of at most 1024 points whose step needs
- * no finalize launch (the register path; the tiled complex64 path of grids of
- * 129..1024 points an axis), plus one end-of-steps launch per sgpe_step_imag /
- * sgpe_step_real call; 3 on complex64 grids with rows of 1025..2048 points
- * (fused pointwise + x sweep, row-tiled y sweep, finalize) and 4 on other 2D
- * paths (double-float tiled grids, longer lines); 0 on 1D grids whose whole step
- * loop is one launch per call (lines of at most 1024 points in SGPE_C64 and
- * SGPE_CDF, at most 256 in SGPE_C128), 3 on other 1D grids.
+ * accounting): 2 on 2D grids whose step fuses the pointwise substeps and the x
+ * sweep and leaves at most 256 norm partials a component (plus one end-of-steps
+ * launch per sgpe_step_imag / sgpe_step_real call), 3 where a finalize launch ends
+ * the step, 4 on the unfused 2D paths; 0 on 1D grids whose whole step loop is one
+ * launch per call (lines of at most 1024 points in SGPE_C64 and SGPE_CDF, at most
+ * 256 in SGPE_C128), 3 on other 1D grids.
  */
 int sgpe_launches_per_step(const sgpe_ctx* ctx);
 

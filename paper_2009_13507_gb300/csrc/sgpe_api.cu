@@ -8,6 +8,7 @@
 
 #include <map>
 #include <algorithm>
+#include <complex>
 #include <vector>
 #include <tuple>
 
@@ -49,6 +50,7 @@ Geometry make_geometry(int dim, int nx, int ny, int esz) {
     g.tiled = dim == 2 && nx >= mid_min && ny >= mid_min && g.reg_x && g.reg_y;
     g.tile_rt = ny <= kTileShortMaxN ? kTileRealShort : kTileReal;
     g.blocks_yt = dim == 2 && (!g.reg_y || g.tiled) ? 3 * ceil_div(nx, 32) * ceil_div(ny, kLongC * g.tile_rt) : 0;
+    g.blocks_pair = dim == 2 && esz == 16 ? 3 * pair_parts(nx, ny) : 0;
     g.blocks_obs = ceil_div(nx, 32) * ceil_div(ny, 4);
     g.blocks_norm = kNormBlocks;
     return g;
@@ -166,9 +168,9 @@ static Layout layout_of(const sgpe_ctx* c) {
     L.partials = off;
     size_t np = 0;
     const Geometry& g = c->geo;
-    size_t cand[5] = {(size_t)g.blocks_x * 3, (size_t)g.blocks_y * 3, (size_t)g.blocks_obs * kObsAcc,
-                      (size_t)g.blocks_norm * 3, (size_t)g.blocks_yt * 3};
-    for (int i = 0; i < 5; i++)
+    size_t cand[6] = {(size_t)g.blocks_x * 3, (size_t)g.blocks_y * 3, (size_t)g.blocks_obs * kObsAcc,
+                      (size_t)g.blocks_norm * 3, (size_t)g.blocks_yt * 3, (size_t)g.blocks_pair};
+    for (int i = 0; i < 6; i++)
         if (cand[i] > np) np = cand[i];
     off = align256(off + np * sizeof(double));
     L.total = off;
@@ -234,6 +236,34 @@ KParams make_kparams(int dim, int nx, int ny, double dx, double dy, const sgpe_p
     k.split = p->split;
     k.so_mode = p->so_mode;
     return k;
+}
+}  // namespace sgpe
+
+namespace sgpe {
+PairHost pair_form(int n, double bre, double bim) {
+    using C = std::complex<double>;
+    PairHost h{};
+    // the root u of u^2 - (1 + 2bt) u + bt^2 with |u| > |bt| (as Launcher::uni)
+    const C b(bre, bim), d = 1.0 + 2.0 * b;
+    const C disc = std::sqrt(d * d - 4.0 * b * b);
+    C u = (d + disc) * 0.5, alt = (d - disc) * 0.5;
+    if (std::abs(alt) > std::abs(u)) u = alt;
+    for (int k = 0; k < 8; k++) u = d - b * b / u;
+    const C g = b / u;
+    // v_k = 2 bt g^k / (u (1 + g)), until |g|^k < 2^-56; pairs until |g|^k < 2^-26
+    C v = 2.0 * b / (u * (1.0 + g));
+    double w = 1.0;
+    int kt = 0;
+    for (; kt < kPairTaps && !(w < std::ldexp(1.0, -56)); kt++) {
+        if (!(w < std::ldexp(1.0, -26))) h.kp = kt + 1;
+        h.wr[kt] = v.real();
+        h.wi[kt] = v.imag();
+        v *= g;
+        w *= std::abs(g);
+    }
+    // (lines shorter than the taps would need images of images)
+    if (w < std::ldexp(1.0, -56) && h.kp <= kPairPairTaps && n > kPairTaps) h.kt = kt;
+    return h;
 }
 }  // namespace sgpe
 
@@ -374,6 +404,7 @@ sgpe_status sgpe_bind(sgpe_ctx* c, void* psi_dev, void* workspace_dev) {
         for (int a = 0; a < 2; a++) {
             for (int k = 0; k < 4; k++) c->tabs[m][a].t[k] = c->work + L.tabs[m][a][k];
             c->tabs[m][a].u = UniHost{};
+            c->tabs[m][a].pair = PairHost{};
             c->us[m][a] = c->work + L.us[m][a];
         }
     for (int m = 0; m < 2; m++)
@@ -413,6 +444,7 @@ sgpe_status sgpe_set_params(sgpe_ctx* c, const sgpe_params* p) {
             // lines longer than kRegMaxN (and the lines of a tiled grid): the constant-factor
             // form of the same solve
             c->tabs[m][a].u = UniHost{};
+            c->tabs[m][a].pair = c->dim == 2 && c->prec != SGPE_C64 ? pair_form(n, bre, bim) : PairHost{};
             if (n > kRegMaxN || c->geo.tiled) {
                 cudaError_t e = with_prec(c->prec, [&](auto r) {
                     return Launcher<decltype(r)>::uni(c->stream, n, bre, bim, c->us[m][a], &c->tabs[m][a].u);
@@ -439,6 +471,29 @@ sgpe_status sgpe_set_params(sgpe_ctx* c, const sgpe_params* p) {
 // enqueue_step_general.
 static bool general_path(const sgpe_ctx* c) { return c->params.split != 0 || c->params.so_mode != 0; }
 
+// The step of a complex128 or double-float 2D grid in the given time mode (0
+// imaginary, 1 real) as increments in FP32 pairs (sgpe_pair.cuh), where both axes'
+// sweeps are short convolutions (bt up to about 0.08, lines of more than 16 points).
+// Double-float grids of 320..~630 points an axis keep the tiled step in imaginary time, where it
+// is the faster one (us a step, tiled against pair: 320^2 29.5 / 31.8, 512^2 55 / 68, 700^2 108 /
+// 97; in real time 400 x 330 53 / 37).
+constexpr long long kPairCdfTiledMax = 400000;
+// Grids of fewer points keep the register kernels (24 x 20: 15.6 us a step against 17.6; 48 x 40
+// 16.3 / 14.5), and so do complex128 steps longer than this, whose dt mu passes 2^-5 where the
+// state lives so often that most blocks leave the increments (256^2 at dt = 4e-3 with c0 rho = 16:
+// 48 / 53 us; 500 x 400 at 2e-3 167 / 90).
+constexpr long long kPairMinPoints = 1536;
+constexpr double kPairMaxDt = 2.5e-3;
+static bool pair_mode(const sgpe_ctx* c, int mode) {
+    if (c->prec == SGPE_CDF && mode == 0 && (long long)c->nx * c->ny <= kPairCdfTiledMax && c->geo.tiled &&
+        tiled_step(c->geo, c->tabs[0][0], c->tabs[0][1]))
+        return false;
+    if ((long long)c->nx * c->ny < kPairMinPoints || (c->prec == SGPE_C128 && c->params.dt > kPairMaxDt)) return false;
+    return c->dim == 2 && c->prec != SGPE_C64 && !general_path(c) && c->tabs[mode][0].pair.kt > 0 &&
+           c->tabs[mode][1].pair.kt > 0;
+}
+static int pair_parts(const sgpe_ctx* c) { return sgpe::pair_parts(c->nx, c->ny); }
+
 // A tiled grid's step in the given time mode (0 imaginary, 1 real) on the kernels of long lines.
 static bool tiled_mode(const sgpe_ctx* c, int mode) {
     return c->geo.tiled && !general_path(c) && tiled_step(c->geo, c->tabs[mode][0], c->tabs[mode][1]);
@@ -459,20 +514,30 @@ static bool tiled_head(const sgpe_ctx* c, int mode) {
 }
 static bool head_scale(const sgpe_ctx* c, int mode) {
     if (general_path(c)) return false;
+    if (pair_mode(c, mode)) return (mode == 0 ? c->params.renorm : 0) == 0 || pair_parts(c) <= kHeadMaxParts;
     return (c->geo.fused && c->geo.reg_y && !tiled_mode(c, mode)) || tiled_head(c, mode);
 }
 
 // The y sweeps (2D) and the long x sweep (1D) of the complex64 and double-float
 // forms leave their norm partials as double-float pairs (summed on the FP32
-// pipe); the 1D register x sweep and every complex128 sweep leave FP64 sums.
-static int parts_df(const sgpe_ctx* c) { return c->prec != SGPE_C128 && (c->dim == 2 || !c->geo.reg_x); }
+// pipe); the 1D register x sweep, every complex128 sweep and the pair step leave FP64 sums.
+static int parts_df(const sgpe_ctx* c, int mode) {
+    return c->prec != SGPE_C128 && !pair_mode(c, mode) && (c->dim == 2 || !c->geo.reg_x);
+}
+
+// The end-of-step launch: norms, next pending scale, step counter (advance).
+static cudaError_t finalize(sgpe_ctx* c, int mode, int advance) {
+    const int renorm = mode == 0 ? c->params.renorm : 0;
+    const int nblk = pair_mode(c, mode) ? 3 * pair_parts(c)
+                     : c->dim == 2      ? y_parts(c->geo, c->tabs[mode][1], c->mid, c->psi)
+                                        : 3 * c->ny;  // 1D: one partial per line
+    return finalize_step(c->stream, c->partials, nblk, c->kp.cell, renorm, c->kp.mag, advance, c->sc,
+                         parts_df(c, mode));
+}
 
 static cudaError_t end_steps(sgpe_ctx* c, bool imag) {
     const int mode = imag ? 0 : 1;
-    if (!head_scale(c, mode)) return cudaSuccess;
-    const int renorm = imag ? c->params.renorm : 0;
-    return finalize_step(c->stream, c->partials, y_parts(c->geo, c->tabs[mode][1], c->mid, c->psi), c->kp.cell,
-                         renorm, c->kp.mag, 0, c->sc, parts_df(c));
+    return head_scale(c, mode) ? finalize(c, mode, 0) : cudaSuccess;
 }
 
 // The SO substep by Crank-Nicolson on the line families of the grid, in -> out:
@@ -542,6 +607,16 @@ static cudaError_t enqueue_step(sgpe_ctx* c, bool imag, const double* omega_tab)
     const int mode = imag ? 0 : 1;
     const int renorm = imag ? c->params.renorm : 0;
     if (general_path(c)) return enqueue_step_general<R>(c, imag, omega_tab);
+    if (pair_mode(c, mode)) {
+        const bool head = head_scale(c, mode);
+        if ((e = Launcher<R>::pair_x(c->stream, imag, c->psi, c->mid, c->kp, c->sc, omega_tab, c->tabs[mode][0].pair,
+                                     head ? c->partials : nullptr, pair_parts(c), renorm)))
+            return e;
+        if ((e = Launcher<R>::pair_y(c->stream, imag, c->mid, c->psi, c->kp, c->tabs[mode][1].pair, c->partials, c->sc,
+                                     renorm, 1, head)))
+            return e;
+        return head ? cudaSuccess : finalize(c, mode, 1);
+    }
     if (c->geo.fused && !tiled_mode(c, mode)) {
         if ((e = Launcher<R>::pwx(c->stream, imag, c->psi, c->mid, c->kp, c->sc, omega_tab, c->tabs[mode][0].t,
                                   c->partials, c->geo.blocks_y / 3, renorm)))
@@ -551,8 +626,7 @@ static cudaError_t enqueue_step(sgpe_ctx* c, bool imag, const double* omega_tab)
                                    c->sc, renorm, 1, 1, head)))
             return e;
         if (head) return cudaSuccess;  // the next head kernel (or end_steps) takes the scale from the partials
-        return finalize_step(c->stream, c->partials, y_parts(c->geo, c->tabs[mode][1], c->mid, c->psi), c->kp.cell,
-                             renorm, c->kp.mag, 1, c->sc, parts_df(c));
+        return finalize(c, mode, 1);
     }
     if (tiled_head(c, mode)) {
         // tiled complex64 grid: the fused kernel forms the pending scale from the row
@@ -579,14 +653,12 @@ static cudaError_t enqueue_step(sgpe_ctx* c, bool imag, const double* omega_tab)
         if ((e = Launcher<R>::cn_y(c->stream, imag, c->mid, c->psi, c->kp, c->tabs[mode][1], c->geo, c->partials,
                                    c->sc, renorm, 1, 1)))
             return e;
-        return finalize_step(c->stream, c->partials, y_parts(c->geo, c->tabs[mode][1], c->mid, c->psi), c->kp.cell,
-                             renorm, c->kp.mag, 1, c->sc, parts_df(c));
+        return finalize(c, mode, 1);
     }
     if ((e = Launcher<R>::cn_x(c->stream, imag, true, c->mid, c->psi, c->kp, c->tabs[mode][0], c->geo, c->partials,
                                c->sc, renorm, 1)))
         return e;
-    // 1D: one partial per line (3 lines)
-    return finalize_step(c->stream, c->partials, 3 * c->ny, c->kp.cell, renorm, c->kp.mag, 1, c->sc, parts_df(c));
+    return finalize(c, mode, 1);
 }
 
 static cudaError_t enqueue_steps(sgpe_ctx* c, int n, bool imag, const double* omega_tab) {
@@ -872,8 +944,9 @@ sgpe_status sgpe_profile_steps(sgpe_ctx* c, int nsteps, int imag, double* ms_out
     double acc[4] = {0, 0, 0, 0};
     int cnt[4] = {0, 0, 0, 0};
     const bool two = c->dim == 2;
-    const bool fused = c->geo.fused && !tiled_mode(c, mode);
-    const bool long_fused = !general_path(c) && !fused && pwx_long_fits(c->geo, c->tabs[mode][0]) &&
+    const bool pair = pair_mode(c, mode);
+    const bool fused = !pair && c->geo.fused && !tiled_mode(c, mode);
+    const bool long_fused = !pair && !general_path(c) && !fused && pwx_long_fits(c->geo, c->tabs[mode][0]) &&
                             (!c->geo.reg_x || tiled_mode(c, mode));
     const bool head = head_scale(c, mode);
     sgpe_status out = SGPE_OK;
@@ -883,6 +956,12 @@ sgpe_status sgpe_profile_steps(sgpe_ctx* c, int nsteps, int imag, double* ms_out
       for (int bi = 0; bi < nb && !e; bi++) {
         cudaEvent_t* ev = evs[bi];
         e = cudaEventRecord(ev[0], c->stream);
+        if (!e && pair)
+            e = with_prec(c->prec, [&](auto r) {
+                return Launcher<decltype(r)>::pair_x(c->stream, im, c->psi, c->mid, c->kp, c->sc, nullptr,
+                                                     c->tabs[mode][0].pair, head ? c->partials : nullptr,
+                                                     pair_parts(c), renorm);
+            });
         if (!e && fused)
             e = with_prec(c->prec, [&](auto r) {
                 return Launcher<decltype(r)>::pwx(c->stream, im, c->psi, c->mid, c->kp, c->sc, nullptr,
@@ -894,28 +973,31 @@ sgpe_status sgpe_profile_steps(sgpe_ctx* c, int nsteps, int imag, double* ms_out
                                                        c->tabs[mode][0], 7, head ? c->partials : nullptr,
                                                        c->geo.blocks_yt / 3, renorm);
             });
-        if (!e && !fused && !long_fused)
+        if (!e && !pair && !fused && !long_fused)
             e = with_prec(c->prec, [&](auto r) {
                 return Launcher<decltype(r)>::pointwise(c->stream, im, c->psi, c->mid, c->kp, c->sc, nullptr, 7);
             });
         if (!e) e = cudaEventRecord(ev[1], c->stream);
         void* xout = two ? c->mid : c->psi;
-        if (!e && !fused && !long_fused)
+        if (!e && !pair && !fused && !long_fused)
             e = with_prec(c->prec, [&](auto r) {
                 return Launcher<decltype(r)>::cn_x(c->stream, im, !two, c->mid, xout, c->kp, c->tabs[mode][0], c->geo,
                                                    c->partials, c->sc, renorm, 1);
             });
         if (!e) e = cudaEventRecord(ev[2], c->stream);
-        if (!e && two)
+        if (!e && pair)
+            e = with_prec(c->prec, [&](auto r) {
+                return Launcher<decltype(r)>::pair_y(c->stream, im, c->mid, c->psi, c->kp, c->tabs[mode][1].pair,
+                                                     c->partials, c->sc, renorm, 1, head);
+            });
+        if (!e && two && !pair)
             e = with_prec(c->prec, [&](auto r) {
                 return Launcher<decltype(r)>::cn_y(c->stream, im, c->mid, c->psi, c->kp, c->tabs[mode][1], c->geo,
                                                    c->partials, c->sc, renorm, 1, 1, head);
             });
         if (!e) e = cudaEventRecord(ev[3], c->stream);
         if (!e && !head)
-            e = finalize_step(c->stream, c->partials,
-                              two ? y_parts(c->geo, c->tabs[mode][1], c->mid, c->psi) : 3 * c->ny, c->kp.cell, renorm,
-                              c->kp.mag, 1, c->sc, parts_df(c));
+            e = finalize(c, mode, 1);
         if (!e) e = cudaEventRecord(ev[4], c->stream);
       }
       if (!e) e = cudaEventSynchronize(evs[nb - 1][4]);
@@ -925,7 +1007,7 @@ sgpe_status sgpe_profile_steps(sgpe_ctx* c, int nsteps, int imag, double* ms_out
       }
       for (int bi = 0; bi < nb; bi++)
           for (int k = 0; k < 4; k++) {
-              if ((k == 2 && !two) || (k == 1 && (fused || long_fused)) || (k == 3 && head)) continue;
+              if ((k == 2 && !two) || (k == 1 && (pair || fused || long_fused)) || (k == 3 && head)) continue;
               float ms = 0.f;
               cudaEventElapsedTime(&ms, evs[bi][k], evs[bi][k + 1]);
               acc[k] += ms;
@@ -951,6 +1033,7 @@ int sgpe_launches_per_step(const sgpe_ctx* c) {
     }
     if (one_block_1d(c)) return 0;  // one launch per step call
     if (head_scale(c, 0)) return 2;  // plus one end-of-steps launch per step call
+    if (pair_mode(c, 0)) return 3;
     if (c->geo.fused && !tiled_mode(c, 0)) return 3;
     if (c->dim == 2 && pwx_long_fits(c->geo, c->tabs[0][0]) && (!c->geo.reg_x || tiled_mode(c, 0))) return 3;
     return c->dim == 2 ? 4 : 3;

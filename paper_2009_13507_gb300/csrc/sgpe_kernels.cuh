@@ -34,6 +34,10 @@ struct DevScalars {
     int step_idx;        // index into a per-step Omega table (real time)
     int err;             // bit 0: non-finite norm
     unsigned ticket[4];  // last-block tickets: 0 step finalize, 1 observables, 2 norms
+    // the pair step (complex128): steps done, and the high word of the largest |Re|, |Im| of the
+    // state as the y sweep of step k saw it in umax[k % 3] (0: unknown); umax_slot: the running step's
+    int pair_tick, umax_slot;
+    unsigned umax[3];
 };
 
 // Crank-Nicolson coefficient tables for one axis and one time mode.
@@ -845,6 +849,7 @@ static __global__ void k_reset_scale(DevScalars* sc) {
         sc->scale_f[threadIdx.x] = 1.0f;
         sc->scale_l[threadIdx.x] = 0.0f;
     }
+    if (threadIdx.x < 3) sc->umax[threadIdx.x] = 0u;
     if (threadIdx.x == 0) sc->scale_src = 0;
 }
 

@@ -86,6 +86,38 @@ inline int obs_rows(int nx, int ny) {
 }
 constexpr int kNormBlocks = 304;
 
+// The pair step (sgpe_pair.cuh): most taps of a sweep (as pairs, in all); points of a row
+// segment's block (three threads a point); columns and rows of a y tile.
+constexpr int kPairPairTaps = 8;
+constexpr int kPairTaps = 16;
+constexpr int kPairXPts = 160;
+constexpr int kPairPPts = 256;  // (of a block with one thread a point)
+constexpr int kPairCols = 8, kPairRows = 64;
+// A stretch of an n-point line: segment sg of nseg writes [o0, o1) and works on [a0, a1).
+struct PairSeg {
+    int o0, o1, a0, a1;
+};
+__host__ __device__ inline PairSeg pair_seg(int n, int nseg, int halo, int sg) {
+    const int per = (n + nseg - 1) / nseg;
+    PairSeg s;
+    s.o0 = sg * per < n ? sg * per : n;
+    s.o1 = (sg + 1) * per < n ? (sg + 1) * per : n;
+    s.a0 = s.o0 - halo > 0 ? s.o0 - halo : 0;
+    s.a1 = s.o1 + halo < n ? s.o1 + halo : n;
+    return s;
+}
+// Segments of an n-point row, and the points of the longest, with a halo inside the row.
+inline int pair_nseg(int n, int halo, int pts) { return n <= pts ? 1 : ceil_div(n, pts - 2 * halo); }
+inline int pair_pts(int n, int halo, int pts) {
+    const int ns = pair_nseg(n, halo, pts);
+    return ns == 1 ? n : ceil_div(n, ns) + 2 * halo;
+}
+// Points of a grid up to which the head kernel takes three threads a point (96^2 13.1 against
+// 17.3 us a step, 128^2 14.7 against 16.4; 144^2 18.5 against 17.3 with one thread a point).
+constexpr int kPairSplitMax = 128 * 128;
+// Tiles of a component in the y sweep (= norm partials).
+inline int pair_parts(int nx, int ny) { return ceil_div(nx, kPairCols) * ceil_div(ny, kPairRows); }
+
 struct Geometry {
     int dim, nx, ny, esz;
     int wx;  // lines longer than kRegMaxN: warps per block (one line) of the x sweep
@@ -95,6 +127,7 @@ struct Geometry {
     size_t smem_x, smem_y;
     int blocks_x, blocks_y, blocks_obs, blocks_norm;
     int blocks_yt;  // long columns (and tiled grids): blocks (= norm partials) of the row-tiled y sweep
+    int blocks_pair;  // most norm partials of the pair step
     int tile_rt;    // chunks of 16 rows that a y tile writes (kTileReal, or kTileRealShort on short columns)
     bool tiled;     // 2D grid of kMidMinN (kMidMinN16)..kRegMaxN points an axis: its steps take the kernels of long
                     // lines (complex64: fused pointwise + x sweep; double-float: pointwise kernel and the
@@ -122,10 +155,16 @@ struct UniHost {
     int hc;                     // halo chunks of the row-tiled y sweep (0: not applicable)
     const void* s;              // device: s_i, i < ks, in the state's element type
 };
-// The coefficient tables of one axis and time mode, and their constant-factor form.
+// The taps of the pair step's sweeps (PairTab), FP64.
+struct PairHost {
+    double wr[kPairTaps], wi[kPairTaps];
+    int kp, kt;  // taps as pairs, in all (0: not applicable)
+};
+// The coefficient tables of one axis and time mode, and their constant-factor forms.
 struct TabSet {
     void* t[4];  // device: fa, fg, fp, fq
     UniHost u;
+    PairHost pair;
 };
 
 // Whether the y sweep of these tables runs in row tiles (k_cn_y_tile: long
@@ -196,6 +235,13 @@ template <typename R> struct Launcher {
     // copies s to s_dev (kUniMaxS entries of room; s_dev null: no copy); u->ks = 0
     // where the correction would be longer than that (and always for complex128).
     static cudaError_t uni(cudaStream_t s, int n, double bre, double bim, void* s_dev, UniHost* u);
+    // The pair step (complex128 and double-float 2D grids whose axes have PairHost::kt > 0):
+    // pending scale, pointwise substeps and CN along x, A -> B, then CN along y, B -> A.
+    // partials / m / renorm as for pwx (FP64 partials); head as head_scale of cn_y.
+    static cudaError_t pair_x(cudaStream_t s, bool imag, const void* A, void* B, const KParams& p, DevScalars* sc,
+                              const double* omega_tab, const PairHost& tx, const double* partials, int m, int renorm);
+    static cudaError_t pair_y(cudaStream_t s, bool imag, const void* in, void* out, const KParams& p, const PairHost& ty,
+                              double* partials, DevScalars* sc, int renorm, int advance, bool head);
     static cudaError_t flush(cudaStream_t s, void* A, size_t plane, const DevScalars* sc);
     // advance: also move the step counter on (the last kernel of a step).
     static cudaError_t norms(cudaStream_t s, const void* A, size_t plane, double cell, int renorm, double mag,
@@ -207,6 +253,9 @@ template <typename R> struct Launcher {
     static cudaError_t observables(cudaStream_t s, const void* A, const KParams& p, double omega_t,
                                    double* partials, DevScalars* sc);
 };
+
+// The taps of an n-point line with bt = bre + i bim for the pair step.
+PairHost pair_form(int n, double bre, double bim);
 
 cudaError_t reset_scale(cudaStream_t s, DevScalars* sc);
 

@@ -8,6 +8,7 @@
 #include "sgpe_cn.cuh"
 #include "sgpe_kernels.cuh"
 #include "sgpe_launch.h"
+#include "sgpe_pair.cuh"
 #include "sgpe_socn.cuh"
 #include "sgpe_step1d_cl.cuh"
 
@@ -510,6 +511,68 @@ cudaError_t Launcher<R>::uni(cudaStream_t s, int n, double bre, double bim, void
     }
     u->s = s_dev;
     return cudaSuccess;
+}
+
+static inline PairTab pair_tab(const PairHost& h) {
+    PairTab t{};
+    for (int k = 0; k < kPairPairTaps; k++) {
+        const df r = df_from(h.wr[k]), i = df_from(h.wi[k]);
+        t.wr[k] = make_float4(r.hi, r.hi, r.lo, r.lo);
+        t.wi[k] = make_float4(i.hi, i.hi, i.lo, i.lo);
+    }
+    for (int k = 0; k < kPairTaps; k++) {
+        const float r = (float)h.wr[k], i = (float)h.wi[k];
+        t.wf[k] = make_float4(r, r, -i, i);
+    }
+    t.kp = h.kp;
+    t.kt = h.kt;
+    return t;
+}
+
+template <typename R>
+cudaError_t Launcher<R>::pair_x(cudaStream_t s, bool imag, const void* A, void* B, const KParams& p,
+                                DevScalars* sc, const double* omega_tab, const PairHost& tx,
+                                const double* partials, int m, int renorm) {
+    if constexpr (is_f32<R>()) {
+        return cudaErrorNotSupported;
+    } else {
+        using T = typename V2<R>::T;
+        if (p.dim != 2 || tx.kt < 1 || tx.kt > kPairTaps) return cudaErrorInvalidValue;
+        KParams q = p;
+        fill_derived(q);
+        const bool split = (long long)p.nx * p.ny <= kPairSplitMax;
+        const int pts = split ? kPairXPts : kPairPPts, halo = tx.kt + 1, nseg = pair_nseg(p.nx, halo, pts);
+        const dim3 block((split ? 96 : 32) * ceil_div(pair_pts(p.nx, halo, pts), 32));
+        auto go = [&](auto kern) {
+            return launch_pdl(kern, dim3((unsigned)p.ny * nseg), block, 0, s, (const T*)A, (T*)B, q, sc, omega_tab,
+                              pair_tab(tx), nseg, partials, m, renorm);
+        };
+        cudaError_t e;
+        if (split)
+            e = imag ? go(k_pair_x<R, true>) : go(k_pair_x<R, false>);
+        else
+            e = imag ? go(k_pair_xp<R, true>) : go(k_pair_xp<R, false>);
+        return e ? e : cudaGetLastError();
+    }
+}
+
+template <typename R>
+cudaError_t Launcher<R>::pair_y(cudaStream_t s, bool imag, const void* in, void* out, const KParams& p,
+                                const PairHost& ty, double* partials, DevScalars* sc, int renorm, int advance,
+                                bool head) {
+    if constexpr (is_f32<R>()) {
+        return cudaErrorNotSupported;
+    } else {
+        using T = typename V2<R>::T;
+        if (p.dim != 2 || ty.kt < 1 || ty.kt > kPairTaps) return cudaErrorInvalidValue;
+        const int nrt = ceil_div(p.ny, kPairRows);
+        auto go = [&](auto kern) {
+            return launch_pdl(kern, dim3(3 * ceil_div(p.nx, kPairCols) * nrt), dim3(256), 0, s, (const T*)in, (T*)out, p,
+                              pair_tab(ty), nrt, partials, sc, head ? 1 : 0, renorm, advance);
+        };
+        const cudaError_t e = imag ? go(k_pair_y<R, true>) : go(k_pair_y<R, false>);
+        return e ? e : cudaGetLastError();
+    }
 }
 
 template <typename R> cudaError_t Launcher<R>::flush(cudaStream_t s, void* A, size_t plane, const DevScalars* sc) {

@@ -25,10 +25,12 @@ using namespace sgpe;
 namespace {
 
 // Scratch: a DevScalars block (tickets, error flag, observables) in the first
-// 256 bytes, then the per-block partial sums (kObsAcc doubles per block).
+// 512 bytes, then the per-block partial sums (kObsAcc doubles per block). The limit on the
+// grid counts one block per 32 x 4 points, kMaxBlocks of them; the kernel launches fewer
+// (strips of obs_rows rows a warp: at most 16 x 608 warps' worth on the largest grids).
 constexpr size_t kScratchBytes = 1u << 20;  // 1 MiB per device
-constexpr size_t kScalarsBytes = 256;
-constexpr size_t kMaxBlocks = (kScratchBytes - kScalarsBytes) / (kObsAcc * sizeof(double));
+constexpr size_t kScalarsBytes = 512;
+constexpr size_t kMaxBlocks = (kScratchBytes - 256) / (kObsAcc * sizeof(double));
 static_assert(sizeof(DevScalars) <= kScalarsBytes, "DevScalars must fit its slot");
 
 static __device__ __align__(256) unsigned char g_obs_scratch[kScratchBytes];

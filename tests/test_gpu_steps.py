@@ -84,3 +84,63 @@ def test_batch_of_lines_only(precision):
         tol = 1e-10 if precision == "c128" else 1e-5
         assert relerr(bs.states()[i], ref) < tol, n
         assert abs(obs[i, 5] - O.observables(prob, ref)["E"]) < tol * max(1.0, abs(obs[i, 5])), n
+
+
+PAIR_SIZES = [(17, 91), (33, 47), (128, 128), (127, 129), (160, 64), (161, 65), (256, 48), (257, 47), (300, 81), (18, 200)]
+# 20 steps of about ten roundings each, of 2^-53 (complex128) or 2^-48 (double-float), all one way
+PAIR_TOL = {"c128": 20 * 10 * 2.0 ** -53, "cdf": 20 * 10 * 2.0 ** -48}
+
+
+@pytest.mark.parametrize("precision", ["c128", "cdf"])
+@pytest.mark.parametrize("imag", [True, False])
+@pytest.mark.parametrize("nx,ny", PAIR_SIZES)
+def test_pair_step(nx, ny, imag, precision):
+    """The pair step at the edges of its row segments (160 and 256 points) and tiles (8
+    columns, 64 rows), just above the shortest line, with both head kernels."""
+    prob, s = make_pair(2, nx, ny, dx=0.1, dy=0.11, c0=40.0, c2=1.5, so_type=1 + nx % 3, gamma=0.7, omega=0.4, wy=1.1,
+                        dt=1e-3, renorm=1 if imag else 0, precision=precision)
+    psi = _rand(prob, nx + ny, env=20.0)
+    s.set_state(psi)
+    (s.step_imag if imag else s.step_real)(20)
+    assert relerr(s.get_state(), O.step(prob, psi, 20, imag)) < PAIR_TOL[precision]
+
+
+@pytest.mark.parametrize("nx", [96, 300])
+@pytest.mark.parametrize("what", ["large_dt", "magnetisation", "norm", "tiny", "huge", "table"])
+def test_pair_step_outside_its_increments(what, nx):
+    """Blocks that leave the increments for FP64 (dt mu, dt A above their limits), scale
+    factors far from 1 or unequal, states far from order 1 in linear runs, and a table."""
+    kw = dict(c0=40.0, c2=1.5, so_type=1, gamma=0.7, omega=0.4, dt=1e-3, renorm=0)
+    imag, scale = False, 1.0
+    if what == "large_dt":
+        kw.update(dt=2.5e-3, omega=30.0)
+    elif what in ("magnetisation", "norm"):
+        imag, scale = True, 7.0
+        kw.update(renorm=2 if what == "magnetisation" else 1, mag=0.2, so_type=0 if what == "magnetisation" else 1)
+    elif what in ("tiny", "huge"):
+        scale = 1e-80 if what == "tiny" else 1e60
+        kw.update(c0=0.0, c2=0.0)
+    prob, s = make_pair(2, nx, 70, dx=0.1, **kw)
+    psi = _rand(prob, 5, env=20.0) * scale
+    s.set_state(psi)
+    if what == "table":
+        import torch
+        om = np.linspace(0.1, 1.5, 20)
+        s.step_real(20, torch.from_numpy(om).cuda())
+        ref = O.step(prob, psi, 20, False, om)
+    else:
+        (s.step_imag if imag else s.step_real)(20)
+        ref = O.step(prob, psi, 20, imag)
+    assert relerr(s.get_state(), ref) < PAIR_TOL["c128"]
+
+
+def test_pair_step_reports_a_non_finite_state():
+    from paper_2009_13507_gb300 import sgpe
+    prob, s = make_pair(2, 64, 40, dx=0.1, c0=1.0, so_type=1, gamma=0.3, dt=1e-3)
+    psi = _rand(prob, 1)
+    psi[1, 20, 30] = np.nan
+    s.set_state(psi)
+    s.step_imag(3)
+    with pytest.raises(sgpe.SgpeError) as e:
+        s.energy()
+    assert e.value.status == sgpe.ENONFINITE
