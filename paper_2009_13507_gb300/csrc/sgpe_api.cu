@@ -240,29 +240,45 @@ KParams make_kparams(int dim, int nx, int ny, double dx, double dy, const sgpe_p
 }  // namespace sgpe
 
 namespace sgpe {
-PairHost pair_form(int n, double bre, double bim) {
+// The pivot limit: the root u of u^2 - (1 + 2bt) u + bt^2 with |u| > |bt| (as Launcher::uni).
+static std::complex<double> pivot_limit(std::complex<double> b) {
     using C = std::complex<double>;
-    PairHost h{};
-    // the root u of u^2 - (1 + 2bt) u + bt^2 with |u| > |bt| (as Launcher::uni)
-    const C b(bre, bim), d = 1.0 + 2.0 * b;
-    const C disc = std::sqrt(d * d - 4.0 * b * b);
-    C u = (d + disc) * 0.5, alt = (d - disc) * 0.5;
+    const C d = 1.0 + 2.0 * b, disc = std::sqrt(d * d - 4.0 * b * b), alt = (d - disc) * 0.5;
+    C u = (d + disc) * 0.5;
     if (std::abs(alt) > std::abs(u)) u = alt;
     for (int k = 0; k < 8; k++) u = d - b * b / u;
-    const C g = b / u;
-    // v_k = 2 bt g^k / (u (1 + g)), until |g|^k < 2^-56; pairs until |g|^k < 2^-26
-    C v = 2.0 * b / (u * (1.0 + g));
+    return u;
+}
+
+// v0 g^k into wr, wi until |g|^k < 2^-bits: the taps needed, or 0 where room does not hold
+// them. kp (nullable): those with |g|^k >= 2^-26.
+static int geometric_taps(std::complex<double> v, std::complex<double> g, int bits, int room, double* wr, double* wi,
+                          int* kp) {
     double w = 1.0;
     int kt = 0;
-    for (; kt < kPairTaps && !(w < std::ldexp(1.0, -56)); kt++) {
-        if (!(w < std::ldexp(1.0, -26))) h.kp = kt + 1;
-        h.wr[kt] = v.real();
-        h.wi[kt] = v.imag();
+    for (; kt < room && !(w < std::ldexp(1.0, -bits)); kt++) {
+        if (kp && !(w < std::ldexp(1.0, -26))) *kp = kt + 1;
+        wr[kt] = v.real();
+        wi[kt] = v.imag();
         v *= g;
         w *= std::abs(g);
     }
-    // (lines shorter than the taps would need images of images)
-    if (w < std::ldexp(1.0, -56) && h.kp <= kPairPairTaps && n > kPairTaps) h.kt = kt;
+    return w < std::ldexp(1.0, -bits) ? kt : 0;
+}
+
+// (lines shorter than the taps would need images of images)
+PairHost pair_form(int n, double bre, double bim) {
+    PairHost h{};
+    const std::complex<double> b(bre, bim), u = pivot_limit(b), g = b / u;
+    const int kt = geometric_taps(2.0 * b / (u * (1.0 + g)), g, 56, kPairTaps, h.wr, h.wi, &h.kp);
+    if (h.kp <= kPairPairTaps && n > kPairTaps) h.kt = kt;
+    return h;
+}
+ConvHost conv_form(int n, double bre, double bim) {
+    ConvHost h{};
+    const std::complex<double> b(bre, bim), u = pivot_limit(b), g = b / u;
+    const int kt = geometric_taps(2.0 * b / (u * (1.0 - g * g)), g, 34, kConvTaps, h.wr, h.wi, nullptr);
+    if (n > kConvTaps) h.kt = kt;
     return h;
 }
 }  // namespace sgpe
@@ -405,6 +421,7 @@ sgpe_status sgpe_bind(sgpe_ctx* c, void* psi_dev, void* workspace_dev) {
             for (int k = 0; k < 4; k++) c->tabs[m][a].t[k] = c->work + L.tabs[m][a][k];
             c->tabs[m][a].u = UniHost{};
             c->tabs[m][a].pair = PairHost{};
+            c->tabs[m][a].conv = ConvHost{};
             c->us[m][a] = c->work + L.us[m][a];
         }
     for (int m = 0; m < 2; m++)
@@ -444,6 +461,7 @@ sgpe_status sgpe_set_params(sgpe_ctx* c, const sgpe_params* p) {
             // lines longer than kRegMaxN (and the lines of a tiled grid): the constant-factor
             // form of the same solve
             c->tabs[m][a].u = UniHost{};
+            c->tabs[m][a].conv = c->dim == 1 && c->prec == SGPE_C64 ? conv_form(n, bre, bim) : ConvHost{};
             c->tabs[m][a].pair = c->dim == 2 && c->prec != SGPE_C64 ? pair_form(n, bre, bim) : PairHost{};
             if (n > kRegMaxN || c->geo.tiled) {
                 cudaError_t e = with_prec(c->prec, [&](auto r) {
@@ -686,7 +704,7 @@ static sgpe_status run_steps(sgpe_ctx* c, int nsteps, bool imag, const double* o
         const int mode = imag ? 0 : 1;
         const int renorm = imag ? c->params.renorm : 0;
         cudaError_t e = with_prec(c->prec, [&](auto r) {
-            return Launcher<decltype(r)>::step1d(c->stream, imag, c->psi, c->kp, c->sc, omega_tab, c->tabs[mode][0].t,
+            return Launcher<decltype(r)>::step1d(c->stream, imag, c->psi, c->kp, c->sc, omega_tab, c->tabs[mode][0],
                                                  nsteps, renorm);
         });
         CK(e, "1D step loop");

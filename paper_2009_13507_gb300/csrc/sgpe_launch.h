@@ -93,6 +93,8 @@ constexpr int kPairTaps = 16;
 constexpr int kPairXPts = 160;
 constexpr int kPairPPts = 256;  // (of a block with one thread a point)
 constexpr int kPairCols = 8, kPairRows = 64;
+// Most taps of the 1D complex64 loop's sweep (k_step1d_conv).
+constexpr int kConvTaps = 16;
 // A stretch of an n-point line: segment sg of nseg writes [o0, o1) and works on [a0, a1).
 struct PairSeg {
     int o0, o1, a0, a1;
@@ -160,11 +162,17 @@ struct PairHost {
     double wr[kPairTaps], wi[kPairTaps];
     int kp, kt;  // taps as pairs, in all (0: not applicable)
 };
+// The taps of the 1D complex64 loop's sweep.
+struct ConvHost {
+    double wr[kConvTaps], wi[kConvTaps];
+    int kt;  // 0: not applicable
+};
 // The coefficient tables of one axis and time mode, and their constant-factor forms.
 struct TabSet {
     void* t[4];  // device: fa, fg, fp, fq
     UniHost u;
     PairHost pair;
+    ConvHost conv;
 };
 
 // Whether the y sweep of these tables runs in row tiles (k_cn_y_tile: long
@@ -205,7 +213,7 @@ template <typename R> struct Launcher {
     // points), the state in shared memory; A is read at the start and written
     // at the end.
     static cudaError_t step1d(cudaStream_t s, bool imag, void* A, const KParams& p, DevScalars* sc,
-                              const double* omega_tab, const void* const* tabs_x, int nsteps, int renorm);
+                              const double* omega_tab, const TabSet& tabs_x, int nsteps, int renorm);
     // Fused pointwise substeps + CN along x of a 2D grid (Geometry::fused): A -> B.
     // partials / m / renorm: the previous y sweep's norm partials (m per component)
     // and the renormalisation mode, for the pending scale (DevScalars::scale_src).
@@ -256,6 +264,7 @@ template <typename R> struct Launcher {
 
 // The taps of an n-point line with bt = bre + i bim for the pair step.
 PairHost pair_form(int n, double bre, double bim);
+ConvHost conv_form(int n, double bre, double bim);
 
 cudaError_t reset_scale(cudaStream_t s, DevScalars* sc);
 

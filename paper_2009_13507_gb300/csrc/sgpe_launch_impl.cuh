@@ -11,6 +11,7 @@
 #include "sgpe_pair.cuh"
 #include "sgpe_socn.cuh"
 #include "sgpe_step1d_cl.cuh"
+#include "sgpe_step1d_conv.cuh"
 
 namespace sgpe {
 
@@ -166,10 +167,10 @@ static void step1d_c(bool imag, cudaStream_t s, typename V2<R>::T* A, const KPar
 
 template <typename R>
 cudaError_t Launcher<R>::step1d(cudaStream_t s, bool imag, void* A, const KParams& p, DevScalars* sc,
-                                const double* omega_tab, const void* const* tabs_x, int nsteps, int renorm) {
+                                const double* omega_tab, const TabSet& tabs_x, int nsteps, int renorm) {
     using T = typename V2<R>::T;
     if (p.dim != 1 || p.nx > kRegMaxN) return cudaErrorInvalidValue;
-    Tabs<R> t = make_tabs<R>(tabs_x);
+    Tabs<R> t = make_tabs<R>((const void* const*)tabs_x.t);
     KParams q = p;
     fill_derived(q);
     T* a = (T*)A;
@@ -182,6 +183,23 @@ cudaError_t Launcher<R>::step1d(cudaStream_t s, bool imag, void* A, const KParam
                                    : launch_cluster(k_step1d_cl<false>, Q, dim3(kCl1dThreads), 0, s, a, q, sc,
                                                     omega_tab, t, nsteps, renorm);
         return e ? e : cudaGetLastError();
+    }
+    if constexpr (is_f32<R>()) {
+        if (tabs_x.conv.kt > 0) {
+            ConvTab ct{};
+            ct.kt = tabs_x.conv.kt;
+            for (int k = 0; k < kConvTaps; k++) {
+                const float r = (float)tabs_x.conv.wr[k], i = (float)tabs_x.conv.wi[k];
+                ct.w[k] = make_float4(r, r, -i, i);
+            }
+            const size_t sm = step1d_conv_smem(p.nx);
+            const unsigned threads = 32u * ceil_div(p.nx, 32);
+            if (imag)
+                k_step1d_conv<true><<<1, threads, sm, s>>>(a, q, sc, omega_tab, ct, nsteps, renorm);
+            else
+                k_step1d_conv<false><<<1, threads, sm, s>>>(a, q, sc, omega_tab, ct, nsteps, renorm);
+            return cudaGetLastError();
+        }
     }
     switch (chunk_len(p.nx)) {
         case 1: step1d_c<R, 1>(imag, s, a, q, sc, omega_tab, t, nsteps, renorm); break;
@@ -231,6 +249,8 @@ template <typename R> cudaError_t Launcher<R>::setup() {
         if ((e = allow_smem(k_cn_y<R, true, true>))) return e;
         if ((e = allow_smem(k_cn_y<R, false, true>))) return e;
         if constexpr (std::is_same<R, float>::value) {
+            if ((e = allow_smem(k_step1d_conv<true>))) return e;
+            if ((e = allow_smem(k_step1d_conv<false>))) return e;
             if ((e = allow_smem(k_pwx_long<true, true, true>))) return e;
             if ((e = allow_smem(k_pwx_long<false, true, true>))) return e;
             if ((e = allow_smem(k_pwx_long<true, false, true>))) return e;

@@ -144,3 +144,25 @@ def test_pair_step_reports_a_non_finite_state():
     with pytest.raises(sgpe.SgpeError) as e:
         s.energy()
     assert e.value.status == sgpe.ENONFINITE
+
+
+@pytest.mark.parametrize("imag", [True, False])
+@pytest.mark.parametrize("nx,bt", [(17, 0.02), (31, 0.02), (32, 0.3), (33, 0.02), (257, 0.1), (1024, 0.02), (16, 0.02), (64, 0.5)])
+def test_1d_complex64_loop(nx, bt, imag):
+    """The one-block loop with its convolution sweep: the shortest and longest lines, taps that
+    reach across the line's images, and the lines and bt that stay on the lane-chunk loop. The
+    bound is the precision form's 1e-5."""
+    dx = 0.1
+    prob, s = make_pair(1, nx, 1, dx=dx, c0=20.0, c2=-0.8, so_type=1 + nx % 3, gamma=0.5, omega=0.3,
+                        dt=4.0 * dx * dx * bt * (1.0 if bt < 0.05 else 0.1), renorm=(2 if nx == 33 else 1) if imag else 0,
+                        mag=0.1, precision="c64")
+    if bt >= 0.05:  # a larger bt at an affordable dt: a finer grid
+        prob, s = make_pair(1, nx, 1, dx=dx / np.sqrt(10.0), c0=20.0, c2=-0.8, so_type=1 + nx % 3, gamma=0.5, omega=0.3,
+                            dt=4.0 * dx * dx * bt * 0.1, renorm=1 if imag else 0, precision="c64")
+    psi = _rand(prob, nx, env=10.0)
+    s.set_state(psi)
+    (s.step_imag if imag else s.step_real)(15)
+    assert relerr(s.get_state(), O.step(prob, psi, 15, imag)) < 1e-5
+    N = s.normalize()
+    ref = O.observables(prob, O.step(prob, psi, 15, imag))
+    assert np.max(np.abs(N - [ref["N+"], ref["N0"], ref["N-"]])) < 1e-5
