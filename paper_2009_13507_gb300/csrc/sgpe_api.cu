@@ -333,6 +333,7 @@ static sgpe_status build_socn(sgpe_ctx* c, CoefJob* jobs, int* njobs) {
         for (int m = 0; m < 2; m++) {
             SoCnLines& L = c->socn[m][a];
             spin_eigvecs(which, L.ur, L.ui);
+            L.which = which;
             const double q = dts * g / (4.0 * h);
             L.are = m == 0 ? 0.0 : q;   // imaginary time: a = -i dt g/(4h)
             L.aim = m == 0 ? -q : 0.0;  // real time: a = dt g/(4h)
