@@ -166,6 +166,9 @@ class Solver:
             self.psi = torch.zeros((3, self.ny, self.nx, 4), dtype=torch.float32, device=self.device)
         else:
             self.psi = torch.zeros((3, self.ny, self.nx), dtype=self.cdtype, device=self.device)
+        # the two tensors are made on the current stream: their memory may have been another tensor's that
+        # kernels queued there still write, and the zeros above are written there
+        self.stream.wait_stream(torch.cuda.current_stream(self.device))
         self._check(self.lib.sgpe_bind(self.ctx, self.psi.data_ptr(), self.workspace.data_ptr()))
         self.physics = None
 
@@ -459,6 +462,7 @@ class BatchSolver:
         self.offsets = [int(o) for o in offs]
         self.psi = torch.zeros(int(ne.value), dtype=self.cdtype, device=self.device)
         self.workspace = torch.empty(int(nb.value), dtype=torch.uint8, device=self.device)
+        self.stream.wait_stream(torch.cuda.current_stream(self.device))  # as Solver: memory of the current stream
         self._check(self.lib.sgpe_batch_bind(self.b, self.psi.data_ptr(), self.workspace.data_ptr()))
 
     def _check(self, rc):
