@@ -145,8 +145,48 @@ __device__ __forceinline__ R calcnu_adjoint(const cx<R> (&u1)[3], cx<R> (&g)[3],
     return w[0] + w[1] + w[2];
 }
 
-// Per point: recompute SO and CALCNU of psi_n, reverse HERM and CALCNU on g
-// (in place), and accumulate FP64 partial sums of dL/dOt and the trap sums.
+// Per point: recompute SO and CALCNU of psi_n, reverse HERM and CALCNU; g returns the
+// cotangent at the SO output, gOt the point's share of dL/dOt and W that of dL/dV.
+template <typename R>
+__device__ __forceinline__ void reverse_point(const typename V2<R>::T* __restrict__ psi,
+                                              const typename V2<R>::T* G, const KParams& p, R Ot, int ix,
+                                              int iy, size_t c, size_t plane, cx<R> (&g)[3], R* gOt, R* W) {
+    const cx<R> zero = {R(0), R(0)};
+    cx<R> u[3];
+#pragma unroll
+    for (int j = 0; j < 3; j++) u[j] = ld<R>(psi, j * plane + c);
+    if (p.so_case) {
+        cx<R> X[3], Y[3];
+#pragma unroll
+        for (int j = 0; j < 3; j++) {
+            cx<R> xp = (ix + 1 < p.nx) ? ld<R>(psi, j * plane + c + 1) : zero;
+            cx<R> xm = (ix > 0) ? ld<R>(psi, j * plane + c - 1) : zero;
+            X[j] = sub(xp, xm);
+            if (p.dim == 2) {
+                cx<R> yp = (iy + 1 < p.ny) ? ld<R>(psi, j * plane + c + p.nx) : zero;
+                cx<R> ym = (iy > 0) ? ld<R>(psi, j * plane + c - p.nx) : zero;
+                Y[j] = sub(yp, ym);
+            } else {
+                Y[j] = zero;
+            }
+        }
+        R gx[3] = {(R)p.hx, (R)p.hx, (R)p.hx}, gy[3] = {(R)p.hy, (R)p.hy, (R)p.hy};
+        so_point<false>(u, X, Y, gx, gy, p.so_case);
+    }
+    const int kx = ix - p.nx / 2, ky = iy - p.ny / 2;
+    const R V = (R)p.vx * (R)(kx * kx) + (p.dim == 2 ? (R)p.vy * (R)(ky * ky) : R(0));
+    const R dt = (R)p.dt;
+    cx<R> u2[3] = {u[0], u[1], u[2]};
+    calcnu_point<false>(u2, V, (R)p.c0, (R)p.c2, dt);
+#pragma unroll
+    for (int j = 0; j < 3; j++) g[j] = ld<R>(G, j * plane + c);
+    *gOt = herm_adjoint<R>(u2, g, (R)p.c2, Ot, dt);
+    *W = calcnu_adjoint<R>(u, g, V, (R)p.c0, (R)p.c2, dt);
+}
+
+// complex128: the reverse of HERM and CALCNU on g in place, with FP64 partial sums of dL/dOt
+// and the trap sums; the reverse SO and the sum of the partials are launches of their own
+// (the ring of ka_reverse would repeat a quarter to a half of this kernel's FP64 work, which bounds it).
 // Block 32 x 4, one point per thread.
 template <typename R>
 __global__ void __launch_bounds__(128) ka_pointwise(const typename V2<R>::T* __restrict__ psi,
@@ -159,38 +199,10 @@ __global__ void __launch_bounds__(128) ka_pointwise(const typename V2<R>::T* __r
     double acc[3] = {0.0, 0.0, 0.0};  // dL/dOt, sum W wx x^2, sum W wy y^2
     if (ix < p.nx && iy < p.ny) {
         const size_t plane = (size_t)p.nx * p.ny, c = (size_t)iy * p.nx + ix;
-        const cx<R> zero = {R(0), R(0)};
-        cx<R> u[3];
-#pragma unroll
-        for (int j = 0; j < 3; j++) u[j] = ld<R>(psi, j * plane + c);
-        if (p.so_case) {
-            cx<R> X[3], Y[3];
-#pragma unroll
-            for (int j = 0; j < 3; j++) {
-                cx<R> xp = (ix + 1 < p.nx) ? ld<R>(psi, j * plane + c + 1) : zero;
-                cx<R> xm = (ix > 0) ? ld<R>(psi, j * plane + c - 1) : zero;
-                X[j] = sub(xp, xm);
-                if (p.dim == 2) {
-                    cx<R> yp = (iy + 1 < p.ny) ? ld<R>(psi, j * plane + c + p.nx) : zero;
-                    cx<R> ym = (iy > 0) ? ld<R>(psi, j * plane + c - p.nx) : zero;
-                    Y[j] = sub(yp, ym);
-                } else {
-                    Y[j] = zero;
-                }
-            }
-            R gx[3] = {(R)p.hx, (R)p.hx, (R)p.hx}, gy[3] = {(R)p.hy, (R)p.hy, (R)p.hy};
-            so_point<false>(u, X, Y, gx, gy, p.so_case);
-        }
         const int kx = ix - p.nx / 2, ky = iy - p.ny / 2;
-        const R V = (R)p.vx * (R)(kx * kx) + (p.dim == 2 ? (R)p.vy * (R)(ky * ky) : R(0));
-        const R dt = (R)p.dt;
-        cx<R> u2[3] = {u[0], u[1], u[2]};
-        calcnu_point<false>(u2, V, (R)p.c0, (R)p.c2, dt);
         cx<R> g[3];
-#pragma unroll
-        for (int j = 0; j < 3; j++) g[j] = ld<R>(G, j * plane + c);
-        const R gOt = herm_adjoint<R>(u2, g, (R)p.c2, (R)Ot, dt);
-        const R W = calcnu_adjoint<R>(u, g, V, (R)p.c0, (R)p.c2, dt);
+        R gOt, W;
+        reverse_point<R>(psi, G, p, (R)Ot, ix, iy, c, plane, g, &gOt, &W);
 #pragma unroll
         for (int j = 0; j < 3; j++) st<R>(G, j * plane + c, g[j]);
         acc[0] = (double)gOt;
@@ -252,23 +264,146 @@ __global__ void __launch_bounds__(128) ka_loss(const typename V2<R>::T* __restri
     }
 }
 
-// One block: out[0] = sum of part[3b + 0] / sqrt2 (dL/dOmega_n) and dw[0..1] +=
-// sums of part[3b + 1..2]; with stride 1 (loss), out[0] = sum part[b].
-__global__ void __launch_bounds__(256) ka_reduce(const double* part, int nblk, int stride, double* out, double* dw) {
-    __shared__ double red[8 * 3];
+// out[0] = sum of part[3b + 0] / sqrt2 (dL/dOmega_n) and dw[0..1] += sums of part[3b + 1..2],
+// by one block in a fixed order. red: 3 doubles a warp.
+__device__ __forceinline__ void reduce_partials(const double* part, int nblk, double* out, double* dw, double* red) {
     double s[3] = {0.0, 0.0, 0.0};
     for (int b = threadIdx.x; b < nblk; b += blockDim.x)
-        for (int q = 0; q < stride; q++) s[q] += part[(size_t)stride * b + q];
+        for (int q = 0; q < 3; q++) s[q] += part[3 * (size_t)b + q];
     block_reduce<3>(s, red);
     if (threadIdx.x == 0) {
-        if (stride == 1) {
-            out[0] = s[0];
-        } else {
-            out[0] = s[0] * 0.70710678118654752440;
-            dw[0] += s[1];
-            dw[1] += s[2];
-        }
+        out[0] = s[0] * 0.70710678118654752440;
+        dw[0] += s[1];
+        dw[1] += s[2];
     }
+}
+
+// complex64: a whole reverse pointwise stage in one launch. Block b >= 1 owns a tile of
+// 32 x 8 points (tile b - 1): it reverses HERM and CALCNU of its points and of the ring of
+// neighbours that the SO stencil reads (a thread a point: 256 + 80 of the block's 352), keeps
+// those cotangents in shared memory, and applies the reverse SO (dt -> -dt) from there; Gin
+// and Gout differ. Block 0 sums the partials that the previous launch left in part_prev (the
+// next-later step's, whose dL/dOmega goes to out_prev), which otherwise is a launch of its own
+// between two steps: the partials have two halves that the launches use in turn.
+//
+// What bounds it: latency (256 tiles at 256^2 are one wave). The FP64 part is the sums of
+// dL/dOt, W kx^2 and W ky^2: ten FP64 instructions a warp (fold_sum3; the factors
+// wx dx^2, wy dy^2 are applied to the block's sums) instead of 25.
+// Measured (256^2, 100 steps, a gradient by propagate_real): 5.62 -> 4.32 ms against three
+// launches (in place 8.7 us, the sum 5.1, SO 2.9, and their gaps). The y sweep stays in place:
+// on row tiles (to the other buffer) 4.12 ms, but the gradient's error against 64 bits grows
+// from 1.1e-6 to 1.2e-6.
+constexpr int kRevX = 32, kRevY = 8;
+constexpr int kRevPts = kRevX * kRevY, kRevRing = 2 * (kRevX + kRevY);
+constexpr int kRevThreads = 32 * ((kRevPts + kRevRing + 31) / 32);
+
+// Sums of three values over the warp in six additions a lane: lanes 0, 8 and 16 return the
+// sums of a, b and c. Each exchange halves the values a lane still holds.
+__device__ __forceinline__ double fold_sum3(double a, double b, double c) {
+    const int lane = threadIdx.x & 31;
+    const bool up = lane & 16, odd = lane & 8;
+    double x = (up ? c : a) + __shfl_xor_sync(0xffffffffu, up ? a : c, 16);
+    const double y = (up ? 0.0 : b) + __shfl_xor_sync(0xffffffffu, up ? b : 0.0, 16);
+    const double send = up ? x : (odd ? x : y);
+    const double got = __shfl_xor_sync(0xffffffffu, send, 8);
+    x = ((odd && !up) ? y : x) + got;
+#pragma unroll
+    for (int off = 4; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
+    return x;
+}
+
+__global__ void __launch_bounds__(kRevThreads) ka_reverse(const float2* __restrict__ psi,
+                                                          const float2* __restrict__ Gin, float2* __restrict__ Gout,
+                                                          KParams p, float Ot, double* part, int tiles_x,
+                                                          const double* part_prev, int nblk, double* out_prev,
+                                                          double* dw) {
+    constexpr int kW = kRevX + 2;
+    __shared__ float2 gs[3][kRevY + 2][kW];
+    __shared__ double red[(kRevThreads / 32) * 3];
+    const int t = threadIdx.x;
+    pdl_wait();
+    if (blockIdx.x == 0) {
+        if (part_prev) reduce_partials(part_prev, nblk, out_prev, dw, red);
+        return;
+    }
+    const int tile = blockIdx.x - 1;
+    const int x0 = (tile % tiles_x) * kRevX, y0 = (tile / tiles_x) * kRevY;
+    int lx, ly;
+    if (t < kRevPts) {
+        lx = t % kRevX;
+        ly = t / kRevX;
+    } else if (t < kRevPts + 2 * kRevX) {
+        lx = t % kRevX;
+        ly = t < kRevPts + kRevX ? -1 : kRevY;
+    } else {  // the last threads past the ring repeat its last point without storing it
+        const int h = min(t - (kRevPts + 2 * kRevX), 2 * kRevY - 1);
+        lx = h < kRevY ? -1 : kRevX;
+        ly = h % kRevY;
+    }
+    const int ix = x0 + lx, iy = y0 + ly;
+    const bool in = ix >= 0 && ix < p.nx && iy >= 0 && iy < p.ny;
+    const size_t plane = (size_t)p.nx * p.ny;
+    const cx<float> zero = {0.f, 0.f};
+    cx<float> g[3] = {zero, zero, zero};
+    float gOt = 0.f, W = 0.f;
+    const int kx = ix - p.nx / 2, ky = iy - p.ny / 2;
+    if (in) {
+        const size_t c = (size_t)iy * p.nx + ix;
+        reverse_point<float>(psi, Gin, p, Ot, ix, iy, c, plane, g, &gOt, &W);
+    }
+    if (t < kRevPts + kRevRing) {
+#pragma unroll
+        for (int j = 0; j < 3; j++) gs[j][ly + 1][lx + 1] = make_float2(g[j].re, g[j].im);
+    }
+    if (t < kRevPts) {  // whole warps
+        const double w = (double)W;
+        const double s = fold_sum3((double)gOt, w * (double)(kx * kx), w);
+        const int lane = t & 31;
+        if (!(lane & 7) && lane < 24) red[(t >> 5) * 3 + (lane >> 3)] = s;
+    }
+    __syncthreads();
+    if (t < kRevPts && in) {
+        if (p.so_case) {
+            auto at = [&](int j, int y, int x) { return cx<float>{gs[j][y][x].x, gs[j][y][x].y}; };
+            cx<float> X[3], Y[3];
+#pragma unroll
+            for (int j = 0; j < 3; j++) {
+                X[j] = sub(at(j, ly + 1, lx + 2), at(j, ly + 1, lx));
+                Y[j] = p.dim == 2 ? sub(at(j, ly + 2, lx + 1), at(j, ly, lx + 1)) : zero;
+            }
+            const float hx = -(float)p.hx, hy = -(float)p.hy;
+            const float gx[3] = {hx, hx, hx}, gy[3] = {hy, hy, hy};
+            so_point<false>(g, X, Y, gx, gy, p.so_case);
+        }
+#pragma unroll
+        for (int j = 0; j < 3; j++) st<float>(Gout, j * plane + (size_t)iy * p.nx + ix, g[j]);
+    } else if (t >= kRevPts && t < kRevPts + 3) {
+        // dV/dwx = wx x^2, dV/dwy = wy y^2 (a warp's row has one ky)
+        const int q = t - kRevPts;
+        double s = 0.0;
+#pragma unroll
+        for (int w = 0; w < kRevY; w++) {
+            const int r = y0 + w - p.ny / 2;
+            s = q < 2 ? s + red[w * 3 + q] : fma(red[w * 3 + 2], (double)(r * r), s);
+        }
+        if (q == 1) s *= p.wx * p.dx * p.dx;
+        if (q == 2) s = p.dim == 2 ? s * p.wy * p.dy * p.dy : 0.0;
+        part[3 * tile + q] = s;
+    }
+}
+
+__global__ void __launch_bounds__(256) ka_reduce(const double* part, int nblk, double* out, double* dw) {
+    __shared__ double red[8 * 3];
+    reduce_partials(part, nblk, out, dw, red);
+}
+
+// One block: out[0] = sum of part[b] (the loss).
+__global__ void __launch_bounds__(256) ka_sum(const double* part, int nblk, double* out) {
+    __shared__ double red[8];
+    double s[1] = {0.0};
+    for (int b = threadIdx.x; b < nblk; b += blockDim.x) s[0] += part[b];
+    block_reduce<1>(s, red);
+    if (threadIdx.x == 0) out[0] = s[0];
 }
 
 }  // namespace sgpe
@@ -301,7 +436,8 @@ AdjLayout adj_layout(int nx, int ny, int esz, int nsteps, int K) {
     L.g2 = o;
     o += st;
     L.part = o;
-    o = al(o + sizeof(double) * 3 * (size_t)ceil_div(nx, 32) * ceil_div(ny, 4));
+    // the partials of two launches of 32 x 8 tiles, or of one of 32 x 4 points
+    o = al(o + sizeof(double) * 3 * (size_t)ceil_div(nx, 32) * 2 * ceil_div(ny, 8));
     L.scal = o;
     o = al(o + sizeof(double) * 8);
     L.total = o;
@@ -383,31 +519,47 @@ static cudaError_t adj_reverse(const CtxView& v, int nsteps, const double* omega
     T* G2 = (T*)(ws + L.g2);
     double* part = (double*)(ws + L.part);
     double* scal = (double*)(ws + L.scal);  // [0] loss, [1..2] dw
-    dim3 blk(32, 4), grd(ceil_div(v.nx, 32), ceil_div(v.ny, 4));
-    const int nblk = grd.x * grd.y;
     KParams kneg = v.kp;  // SO with dt -> -dt
     kneg.hx = -kneg.hx;
     kneg.hy = -kneg.hy;
     cudaError_t e = cudaSuccess;
+    // complex64: the launch before's partials, summed by block 0 of the next
+    const double* prev = nullptr;
+    double* prev_out = nullptr;
+    const int tiles_x = ceil_div(v.nx, kRevX), tiles = tiles_x * ceil_div(v.ny, kRevY);
     for (int sg = L.nck - 1; sg >= 0 && !e; sg--) {
         const int s0 = sg * K, s1 = (s0 + K < nsteps) ? s0 + K : nsteps;
-        e = cudaMemcpyAsync(seg(0), ckpt(sg), st, cudaMemcpyDeviceToDevice, s);
-        for (int k2 = 0; k2 + 1 < s1 - s0 && !e; k2++) e = adj_forward_step<R>(v, seg(k2), seg(k2 + 1), omega_host[s0 + k2]);
+        // psi_n of this segment: its first state is the checkpoint itself
+        auto state = [&](int k) { return k ? seg(k) : ckpt(sg); };
+        for (int k = 0; k + 1 < s1 - s0 && !e; k++) e = adj_forward_step<R>(v, state(k), seg(k + 1), omega_host[s0 + k]);
         for (int n = s1 - 1; n >= s0 && !e; n--) {
+            const T* psi = (const T*)state(n - s0);
+            const double Ot = omega_host[n] * 0.70710678118654752440;
             if (v.dim == 2)
                 e = Launcher<R>::cn_y(s, false, G, G, v.kp, v.tabs_adj[1], *v.geo, v.partials, v.sc, 0, 0, 0);
             if (!e) e = Launcher<R>::cn_x(s, false, false, G, G, v.kp, v.tabs_adj[0], *v.geo, v.partials, v.sc, 0, 0);
-            if (!e) {
-                ka_pointwise<R><<<grd, blk, 0, s>>>((const T*)seg(n - s0), G, v.kp, omega_host[n] * 0.70710678118654752440,
-                                                    part);
-                ka_reduce<<<1, 256, 0, s>>>(part, nblk, 3, domega_dev + n, scal + 1);
+            if (e) break;
+            if constexpr (std::is_same<R, float>::value) {
+                double* pn = part + (size_t)(n & 1) * 3 * tiles;
+                e = launch_pdl(ka_reverse, dim3(1 + tiles), dim3(kRevThreads), 0, s, psi, (const T*)G, G2, v.kp,
+                               (float)Ot, pn, tiles_x, prev, tiles, prev_out, scal + 1);
+                prev = pn;
+                prev_out = domega_dev + n;
+            } else {
+                dim3 blk(32, 4), grd(ceil_div(v.nx, 32), ceil_div(v.ny, 4));
+                ka_pointwise<R><<<grd, blk, 0, s>>>(psi, G, v.kp, Ot, part);
+                ka_reduce<<<1, 256, 0, s>>>(part, grd.x * grd.y, domega_dev + n, scal + 1);
                 e = cudaGetLastError();
+                if (!e) e = Launcher<R>::pointwise(s, false, G, G2, kneg, v.sc, nullptr, 1);
             }
-            if (!e) e = Launcher<R>::pointwise(s, false, G, G2, kneg, v.sc, nullptr, 1);
             T* t = G;
             G = G2;
             G2 = t;
         }
+    }
+    if (prev && !e) {
+        ka_reduce<<<1, 256, 0, s>>>(prev, tiles, prev_out, scal + 1);
+        e = cudaGetLastError();
     }
     *result = G;
     return e;
@@ -429,7 +581,7 @@ static sgpe_status adj_run(sgpe_ctx* c, const CtxView& v, int nsteps, const doub
     // loss and its gradient at psi_N
     if (!e) {
         ka_loss<R><<<grd, blk, 0, s>>>((const T*)v.psi, tgt, G, v.kp, part);
-        ka_reduce<<<1, 256, 0, s>>>(part, nblk, 1, scal, nullptr);
+        ka_sum<<<1, 256, 0, s>>>(part, nblk, scal);
         e = cudaGetLastError();
     }
     T* g0 = nullptr;

@@ -166,3 +166,34 @@ def test_1d_complex64_loop(nx, bt, imag):
     N = s.normalize()
     ref = O.observables(prob, O.step(prob, psi, 15, imag))
     assert np.max(np.abs(N - [ref["N+"], ref["N0"], ref["N-"]])) < 1e-5
+
+
+@pytest.mark.parametrize("dim,nx,ny,so", [(2, 20, 16, 1), (2, 32, 8, 2), (2, 33, 9, 1), (2, 31, 7, 3), (2, 64, 17, 0),
+                                          (2, 5, 3, 1), (1, 48, 1, 2), (1, 33, 1, 1), (1, 32, 1, 3)])
+def test_adjoint_tiles_complex64(dim, nx, ny, so):
+    """The complex64 reverse stage in tiles of 32 x 8 points: grids of one tile, a tile and a
+    point more, partial tiles, a line; odd and even numbers of steps and a last segment of one.
+    Against the complex128 gradient of the same inputs. Bounds: psi_0's cotangent passes 2 x 13
+    steps of some 30 roundings of 6e-8 (5e-5 if all add up; 1e-4); dL/dOmega and dL/dw cancel
+    over the grid (the precision form's 2e-3 of the largest)."""
+    import torch
+    from paper_2009_13507_gb300 import sgpe
+    phys = dict(c0=15.0, c2=-1.5, so_type=so, gamma=0.7, omega=0.5, wx=1.1, wy=0.9, dt=1e-2, renorm=0)
+    om = 0.5 + 0.3 * np.sin(np.arange(13) * 0.7)
+    grads = {}
+    for prec in ("c128", "c64"):
+        prob, s = make_pair(dim, nx, ny, dx=0.35, dy=0.4 if dim == 2 else None, precision=prec, **phys)
+        psi = _rand(prob, nx + ny, env=3.0)
+        target = _rand(prob, 7 + nx, env=3.0)
+        p0 = torch.from_numpy(psi).to(s.cdtype).cuda().requires_grad_(True)
+        omt = torch.tensor(om, dtype=torch.float64, device="cuda:0", requires_grad=True)
+        w = torch.tensor([1.1, 0.9], dtype=torch.float64, device="cuda:0", requires_grad=True)
+        out = sgpe.propagate_real(p0, omt, w, s, 4)
+        t = torch.from_numpy(target).to(s.cdtype).cuda().reshape(out.shape)
+        rho = out.real ** 2 + out.imag ** 2
+        ((torch.conj(t) * out).real.sum() + (rho * (t.real ** 2)).sum()).backward()
+        grads[prec] = (p0.grad.cpu().numpy().astype(np.complex128), omt.grad.cpu().numpy(), w.grad.cpu().numpy())
+    a, b = grads["c64"], grads["c128"]
+    assert np.linalg.norm(a[0] - b[0]) < 1e-4 * np.linalg.norm(b[0])
+    assert np.max(np.abs(a[1] - b[1])) < 2e-3 * np.max(np.abs(b[1]))
+    assert np.max(np.abs(a[2] - b[2])) < 2e-3 * np.max(np.abs(b[2]))
