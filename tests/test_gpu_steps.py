@@ -197,3 +197,34 @@ def test_adjoint_tiles_complex64(dim, nx, ny, so):
     assert np.linalg.norm(a[0] - b[0]) < 1e-4 * np.linalg.norm(b[0])
     assert np.max(np.abs(a[1] - b[1])) < 2e-3 * np.max(np.abs(b[1]))
     assert np.max(np.abs(a[2] - b[2])) < 2e-3 * np.max(np.abs(b[2]))
+
+
+@pytest.mark.parametrize("precision", ["c128", "c64"])
+@pytest.mark.parametrize("K", [1, 4, 12, 13, 50])
+def test_adjoint_tape_is_reusable(K, precision):
+    """The first reverse pass of a tape takes the last segment's states from the forward pass, a
+    second one recomputes them (one segment, segments of one step, a last segment of one step, a
+    full last one): the same bits, also where loss_grad's own reverse pass used the workspace
+    before."""
+    import ctypes
+    import torch
+    prob, s = make_pair(2, 36, 20, dx=0.35, precision=precision, c0=15.0, c2=-1.5, so_type=1, gamma=0.7, omega=0.5, dt=1e-2)
+    psi = _rand(prob, 1)
+    om = 0.5 + 0.3 * np.sin(np.arange(13) * 0.7)
+    lam = torch.from_numpy(_rand(prob, 2)).to(s.cdtype).cuda()
+    s.set_state(psi)
+    tape = s.adjoint_forward(om, K)
+    runs = [s.adjoint_step(tape, lam) for _ in range(2)]
+    final = s.get_state()
+    s.set_state(psi)
+    tgt = torch.zeros(20, 36, dtype=torch.float64, device="cuda:0")
+    dom, dw, L = torch.zeros(13, dtype=torch.float64, device="cuda:0"), np.zeros(2), np.zeros(1)
+    torch.cuda.synchronize()
+    s._check(s.lib.sgpe_adjoint_loss_grad(s.ctx, 13, tape["omega"].data_ptr(), tgt.data_ptr(), K, tape["ws"].data_ptr(),
+                                          L.ctypes.data, dom.data_ptr(), dw.ctypes.data))
+    runs.append(s.adjoint_step(tape, lam))
+    s.synchronize()
+    assert np.array_equal(final, s.get_state())
+    assert relerr(final, O.step(prob, psi, 13, False, om)) < (1e-11 if precision == "c128" else 1e-5)
+    for g, d, w in runs[1:]:
+        assert torch.equal(g, runs[0][0]) and torch.equal(d, runs[0][1]) and w == runs[0][2]
