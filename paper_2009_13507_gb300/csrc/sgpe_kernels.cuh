@@ -510,7 +510,8 @@ __device__ __forceinline__ double sum_partials_warp(const double* q, int m) {
     double v[8];
 #pragma unroll
     for (int k = 0; k < 8; k++) v[k] = (lane + 32 * k < m) ? __ldcg(q + lane + 32 * k) : 0.0;
-    double s = ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
+    double s = (v[0] + v[1]) + (v[2] + v[3]);
+    if (m > 128) s += (v[4] + v[5]) + (v[6] + v[7]);  // (zeros otherwise)
     for (int b = lane + 256; b < m; b += 32) s += __ldcg(q + b);
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);

@@ -14,8 +14,8 @@
 // step -> this one): 128 x 112, 30 steps at dt = 2e-4, imaginary time 7.1e-16 -> 4.3e-16,
 // real time 3.8e-15 -> 1.2e-15; 64 x 80, 60 steps at bt = 0.075 4.4e-16 -> 4.7e-16 and
 // 5.5e-15 -> 4.5e-15; double-float 1.8e-14 -> 3.8e-15 and 6.6e-14 -> 9.0e-15. Measured,
-// us a step: complex128 256^2 imaginary / real time 42.9 / 49.8 -> 25.2 / 24.5, 512^2 158 /
-// 195 -> 97 / 97, 161^2 real time 42.2 -> 20.9, 2048^2 2118 -> 1025; double-float 256^2 20.1
+// us a step: complex128 256^2 imaginary / real time 42.9 / 49.8 -> 24.0 / 24.7, 512^2 158 /
+// 195 -> 91 / 91, 161^2 real time 42.2 -> 19.9, 2048^2 2118 -> 1025; double-float 256^2 20.1
 // / 27.2 -> 17.6 / 18.2, 1024^2 217 / 357 -> 211 / 235.
 //
 // Pairs here are "lazy": products keep the exact error of the leading product and
@@ -192,6 +192,17 @@ constexpr unsigned kBias0 = 896u << 20;
 // (and for zero, infinities and NaN).
 __device__ __forceinline__ int pair_shift(unsigned mx) {
     return (mx >= (983u << 20) && mx < (1063u << 20)) || mx == 0u || mx >= 0x7ff00000u ? 0 : 1023 - (int)(mx >> 20);
+}
+
+// The pending factors as d - 1 in a pair, where they are one factor with |d - 1| < 2^-6 (*is_far
+// otherwise, NaN too). One thread's chain that the whole block waits for: comparisons and the
+// split on the integer pipe, where an FP64 instruction would take its 64 cycles.
+__device__ __forceinline__ void pair_near(const double* d, df* dm, int* is_far) {
+    const double e = d[0] - 1.0;
+    const long long b = __double_as_longlong(d[0]);
+    *is_far = b != __double_as_longlong(d[1]) || b != __double_as_longlong(d[2]) ||
+              ((unsigned)__double2hiint(e) & 0x7fffffffu) >= (1017u << 20);
+    *dm = split64(e, kBias0);
 }
 
 // -- pointwise substeps -------------------------------------------------------------
@@ -393,9 +404,7 @@ __global__ void __launch_bounds__(kPairXThreads, 2)
         } else {
             for (int c = 0; c < 3; c++) dsh[c] = sc->scale[c];
         }
-        const double e0 = dsh[0] - 1.0;
-        far_s = dsh[0] != dsh[1] || dsh[0] != dsh[2] || !(e0 < 0.015625 && e0 > -0.015625);
-        dms = df_from(e0);
+        pair_near(dsh, &dms, &far_s);
     }
     __syncthreads();
     // SO: rows +1 and -1 of H_SO take psi_0 (X with the sign +, -), row 0 psi_-1 - psi_+1 and their sum
@@ -652,9 +661,7 @@ __global__ void __launch_bounds__(kPairPPts, 2)
         } else {
             for (int c = 0; c < 3; c++) dsh[c] = sc->scale[c];
         }
-        const double e0 = dsh[0] - 1.0;
-        far_s = dsh[0] != dsh[1] || dsh[0] != dsh[2] || !(e0 < 0.015625 && e0 > -0.015625);
-        dms = df_from(e0);
+        pair_near(dsh, &dms, &far_s);
     }
     __syncthreads();
     const df hx = kpair(p, KC_HX), hy = kpair(p, KC_HY);
@@ -833,6 +840,7 @@ __global__ void __launch_bounds__(256, 3)
     constexpr int CW = kPairCols, H = kPairTaps;
     __shared__ cd Ms[(kPairRows + 2 * H) * CW];  // (H + r) * CW + column: the link from row o0 + r to the next
     __shared__ typename PartT<R>::T red[8];
+    __shared__ long long zred[8];
     __shared__ unsigned wmax[8];
     const int tid = threadIdx.x, cc = tid % CW, rl = tid / CW;
     const int nct = (p.nx + CW - 1) / CW;
@@ -908,9 +916,11 @@ __global__ void __launch_bounds__(256, 3)
         }
     }
     if (!part) return;
-    // the tile's sum. complex128: the warp's as 64-bit integers in units of 2^-57 of the most a
-    // thread can hold (pairs would round it to 2^-49, FP64 shuffle sums cost 7 FP64 instructions a
-    // warp), the warps' in FP64; double-float: in pairs
+    // the tile's sum. complex128: 64-bit integers in units of 2^-57 of the most a thread can hold
+    // (pairs would round it to 2^-49, FP64 shuffle sums cost 7 FP64 instructions a warp), four FP64
+    // instructions at the end (the warps' sums and the power of two in FP64 were some 30, one
+    // after the other at the end of every block: with the pending factors' chain 256^2 25.2 -> 24.0 us a
+    // step, 512^2 97.7 -> 90.9, 64^2 12.95 -> 12.0); double-float: in pairs
     double q;
     if constexpr (PS::kShift) {
         // |x 2^k| < 2^(E + 1): a thread's four squares stay below 2^(2E + 4)
@@ -919,12 +929,19 @@ __global__ void __launch_bounds__(256, 3)
         long long z = __float2ll_rn(acc.hi * f * g) + (__float2ll_rn(acc.lo * f * g) + __float2ll_rn(acc2 * f * g));
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) z += __shfl_xor_sync(0xffffffffu, z, off);
-        if ((tid & 31) == 0) red[tid >> 5] = (double)z;
+        if ((tid & 31) == 0) zred[tid >> 5] = z;
         __syncthreads();
         q = 0.0;
         if (tid == 0) {
-            for (int w = 0; w < 8; w++) q += red[w];
-            q *= exp2((double)(2 * E - 53));
+            // (the eight sums do not fit 64 bits: their high and low parts apart, one rounding at the end)
+            long long zh = 0;
+            int zl = 0;
+#pragma unroll
+            for (int w = 0; w < 8; w++) {
+                zh += zred[w] >> 12;
+                zl += (int)(zred[w] & 4095);
+            }
+            q = fma((double)zh, 4096.0, (double)zl) * __hiloint2double((1023 + 2 * E - 53) << 20, 0);
         }
     } else {
         const df ps = block_part(fast_two_sum(acc.hi, acc.lo + acc2), red);
