@@ -4,7 +4,9 @@ Workload (one benchmark step): the 2D spin-1 imaginary-time run on a 256 x 256
 grid, dx = dy = 0.05 on [-6.4, 6.4)^2, isotropic trap, c0 = 50, c2 = 1, Rashba
 SO gamma = 0.8, Rabi Omega = 0.5, random-phase Gaussian initial state (seeded),
 dt = 2e-4, 2000 time steps with renormalisation every step, then the
-observables (energy, norms, rms sizes). Complex128 state (plain FP64 form).
+observables (energy, norms, rms sizes). Complex128 state; the step forms its
+increments in FP32 pairs and adds them to the FP64 state (its error against an
+80-bit reference is below that of plain FP64 substeps).
 Metric: grid point-steps per second (one point = all three spin components
 advanced by one full time step).
 
@@ -42,7 +44,7 @@ NSTEPS = 2000
 PHYS = dict(c0=50.0, c2=1.0, so_type=1, gamma=0.8, omega=0.5, dt=2e-4, renorm=1)
 WORKLOAD = "2D spin-1 imaginary time, 256x256, dx=0.05, c0=50, c2=1, Rashba gamma=0.8, Omega=0.5, dt=2e-4, 2000 steps"
 METRIC = "point-steps/s"
-# Algorithmic FP64 flops per grid point of the pointwise kernel (SO + CALCNU +
+# Algorithmic FP64 flops per grid point of the pointwise substeps (SO + CALCNU +
 # HERM, imaginary time, 2D Rashba), counted from the formulas it evaluates
 # (FMA = 2 flops; exp by its degree-9 Taylor polynomial).
 POINTWISE_FLOPS = 263
@@ -56,9 +58,12 @@ FP64_PEAK_TFLOPS = 1.259
 # and 600 steps on one thread (~8 s).
 CPU_SAMPLE_STEPS = NSTEPS
 CPU_SINGLE_STEPS = 600
-# DRAM bytes (read + write) of one launch of the dominant kernel on this workload in an ncu capture
-# (cold L2): None whenever the kernel changed after the capture.
-HEAD_TRAFFIC_BYTES = 3251968
+# DRAM bytes (read + write, cold L2) and executed warp instructions of one launch of the dominant
+# kernel on this workload in an ncu capture (profiles/k_pair_2d256.md).
+HEAD_TRAFFIC_BYTES = 3232512
+HEAD_WARP_INSTRUCTIONS = 6301565
+# Warp instructions the GPU can issue: 152 SMs x 4 schedulers x 2.07 GHz.
+ISSUE_PEAK_GINST = 1258.6
 
 
 def _dist():
@@ -134,7 +139,7 @@ def measured_hbm_gbs():
 def hbm_view(effective_gbps: float) -> dict:
     """Effective bandwidth of the step's two streaming passes (192 algorithmic bytes per
     point-step) against the measured HBM copy peak; the state is L2-resident, so this is
-    context, not the binding roof (the FP64 ALU is)."""
+    context, not the binding roof (instruction issue is)."""
     peak = measured_hbm_gbs()
     return {"algorithmic_bytes_per_point_step": 192, "effective_GBps": effective_gbps,
             "peak_GBps": peak, "peak_source": "measured copy bandwidth" if peak else None,
@@ -216,6 +221,7 @@ def run_reference(args):
         "impl": "reference", "metric": METRIC, "value": value, "unit": METRIC, "n_gpus": args.gpus,
         "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms, "higher_is_better": True,
         "scaling": "weak", "vs_baseline": None, "dtype": "f64", "data": "synthetic",
+        "arithmetic": "FP64 state, sums and norms; increments in FP32 pairs (about 2^-47 of an increment)",
         "time_steps_per_bench_step": steps_per,
         "config": bench_config(ws),
         "cpu_baseline": {"value": value, "unit": METRIC, "cores": cores, "kind": "oracle", "sample": sample,
@@ -522,8 +528,8 @@ def main():
     share = {n: kms[i] / kms.sum() for i, n in enumerate(names) if int(kcnt[i]) > 0}
     dom_ms = kavg[names[0]]
     dom_flops = POINTWISE_FLOPS + (CN_FLOPS if fused else 0)
-    dom_name = ("k_pwx<double, imag, 8> (SO+CALCNU+HERM, CN-x)" if fused
-                else "k_pointwise<double> (SO+CALCNU+HERM)")
+    dom_name = "k_pair_xp<double, imag> (SO+CALCNU+HERM, CN-x as increments in FP32 pairs)"
+    achieved_ginst = HEAD_WARP_INSTRUCTIONS / (dom_ms * 1e-3) / 1e9
     achieved_tflops = dom_flops * NX * NY / (dom_ms * 1e-3) / 1e12
     # the FP64 roof measured on this GPU in this run (FMA-chain kernel, CUDA events)
     try:
@@ -600,10 +606,14 @@ def main():
         "time_steps_per_bench_step": NSTEPS,
         "config": bench_config(ws),
         "roofline": {"bound": "alu", "kernel": dom_name,
-                     "achieved": achieved_tflops, "peak": fp64_peak, "unit": "TFLOP/s",
-                     "frac": achieved_tflops / fp64_peak, "traffic": HEAD_TRAFFIC_BYTES,
-                     "peak_source": peak_source, "nominal_peak": FP64_PEAK_TFLOPS,
-                     "flops_per_point": dom_flops, "avg_launch_ms": dom_ms},
+                     "achieved": achieved_ginst, "peak": ISSUE_PEAK_GINST, "unit": "G warp instructions/s",
+                     "frac": achieved_ginst / ISSUE_PEAK_GINST, "traffic": HEAD_TRAFFIC_BYTES,
+                     "peak_source": "152 SMs x 4 schedulers x 2.07 GHz; instructions per launch from ncu",
+                     "avg_launch_ms": dom_ms,
+                     # the same work counted as FP64 flops, against what the FP64 pipe could do
+                     "fp64_view": {"flops_per_point": dom_flops, "achieved_tflops": achieved_tflops,
+                                   "fp64_peak_tflops": fp64_peak, "ratio": achieved_tflops / fp64_peak,
+                                   "peak_source": peak_source, "nominal_peak": FP64_PEAK_TFLOPS}},
         "kernels": {"avg_ms": kavg, "share": share, "dominant": dom},
         "hbm_view": hbm_view(value / ws * 192 / 1e9),
         "chosen": {"form": "complex64 state, FP64 reductions", "value": replica_value(point_steps, ws, t32),

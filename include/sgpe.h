@@ -51,7 +51,10 @@ typedef enum {
 
 /*
  * Arithmetic of the step:
- *  SGPE_C128  complex128 state, FP64 arithmetic (the plain FP64 form).
+ *  SGPE_C128  complex128 state and reductions at FP64 accuracy. 2D Lie steps
+ *             with small dt form each substep's increment in pairs of FP32
+ *             numbers and add it to the FP64 state; everything else is FP64
+ *             arithmetic.
  *  SGPE_C64   complex64 state and sweeps, FP64 reductions (the precision form).
  *  SGPE_CDF   "double-float": every real number is a pair of FP32 numbers
  *             (about 48 significant bits), all step arithmetic on the FP32

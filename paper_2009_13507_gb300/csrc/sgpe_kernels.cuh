@@ -3,7 +3,10 @@
 // (double: complex128 state; float: complex64 state) and on the time mode
 // (IMAG: z = dt, imaginary time; otherwise z = i dt, real time).
 //
-// One step, 2D with lines of at most 1024 points (sgpe_cn.cuh):
+// The 2D steps of complex128 and double-float grids within the pair step's range are in
+// sgpe_pair.cuh, the 1D step loops in sgpe_step1d_cl.cuh (complex128), sgpe_step1d_conv.cuh
+// (complex64) and sgpe_cn.cuh.
+// One step, 2D with lines of at most 1024 points otherwise (sgpe_cn.cuh):
 //   k_pwx      (A -> B): pending scale, SO, CALCNU, HERM, then Crank-Nicolson
 //                        along x from shared memory, one block per row
 //   k_cny_reg  (B -> A): Crank-Nicolson along y, one warp per column (pair),

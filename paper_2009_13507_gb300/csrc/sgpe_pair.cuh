@@ -15,8 +15,8 @@
 // real time 3.8e-15 -> 1.2e-15; 64 x 80, 60 steps at bt = 0.075 4.4e-16 -> 4.7e-16 and
 // 5.5e-15 -> 4.5e-15; double-float 1.8e-14 -> 3.8e-15 and 6.6e-14 -> 9.0e-15. Measured,
 // us a step: complex128 256^2 imaginary / real time 42.9 / 49.8 -> 21.7 / 22.8, 512^2 158 /
-// 195 -> 86 / 86, 161^2 real time 42.2 -> 18.2, 2048^2 2118 -> 1025; double-float 256^2 20.1
-// / 27.2 -> 17.6 / 18.2, 1024^2 217 / 357 -> 211 / 235.
+// 195 -> 86 / 91, 161^2 real time 42.2 -> 18.2, 2048^2 2118 -> 1010; double-float 256^2 20.1
+// / 27.2 -> 17.3 / 17.9, 1024^2 217 / 357 -> 209 / 233.
 //
 // Pairs here are "lazy": products keep the exact error of the leading product and
 // both cross terms, sums keep the exact rounding error of the leading sum, and
