@@ -126,7 +126,7 @@ class ClockSampler:
 
 
 def measured_hbm_gbs():
-    """The HBM copy bandwidth measured on this GPU pool (MEASURED_PEAKS.json beside this
+    """The HBM copy bandwidth measured on a GB300 (MEASURED_PEAKS.json beside this
     file, GB/s), or None when the file is absent."""
     path = os.path.join(os.path.dirname(os.path.abspath(__file__)), "MEASURED_PEAKS.json")
     try:
@@ -166,7 +166,7 @@ def replica_value(points_per_rank: int, world_size: int, t_ms: float) -> float:
 
 def bench_config(ws: int) -> dict:
     """The workload description shared by both arms (the oracle arm reports the same dict)."""
-    return {"workload": WORKLOAD, "precision": "complex128 (plain FP64 form)", "grid": [NX, NY],
+    return {"workload": WORKLOAD, "precision": "complex128 (FP64 state)", "grid": [NX, NY],
             "l2": "GPU arm: 256 MiB L2 flush between benchmark steps (the 3 MiB state is L2-resident within a "
                   "run); oracle arm: host caches as they are",
             "parallelism": "replicas" if ws > 1 else "single GPU"}
