@@ -273,7 +273,7 @@ sgpe_status sgpe_eval_expm1f(void* cuda_stream, const float* x_dev, float* y_dev
  *  obs_dev  device output, SGPE_NOBS doubles (8-byte aligned), same indices as
  *           sgpe_energy; written asynchronously on cuda_stream.
  *  p        physics (c0, c2, so_type, gamma, omega, wx, wy used; dt ignored).
- * Scratch: a static 1 MiB device array inside the library, present on every
+ * Scratch: a static device array of 1 MiB + 256 bytes inside the library, present on every
  * GPU that loads the library until the process exits. Grids needing more
  * reduction blocks than it holds (ceil(nx/32)*ceil(ny/4) > 11912, roughly more
  * than 1.5 million points) are rejected with SGPE_EUNSUPPORTED before anything

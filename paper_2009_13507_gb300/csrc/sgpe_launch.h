@@ -84,6 +84,15 @@ inline int obs_rows(int nx, int ny) {
     const int r = (int)(((long long)ceil_div(nx, 32) * ny + 607) / 608);
     return r < 1 ? 1 : r > 16 ? 16 : r;
 }
+// The grid of the observables kernel (128 threads a block).
+inline dim3 obs_grid(int dim, int nx, int ny) {
+    return dim == 2 ? dim3(ceil_div(nx, 32), ceil_div(ny, 4 * obs_rows(nx, ny))) : dim3(ceil_div(nx, 128));
+}
+// Static scratch of sgpe_observables_noalloc (sgpe_static.cu): the scalars' slot, then the
+// partial sums of up to kObsMaxBlocks blocks.
+constexpr size_t kObsScratchBytes = (1u << 20) + 256;
+constexpr size_t kObsScalarsBytes = 512;
+constexpr size_t kObsMaxBlocks = (kObsScratchBytes - kObsScalarsBytes) / (kObsAcc * sizeof(double));
 constexpr int kNormBlocks = 304;
 
 // The pair step (sgpe_pair.cuh): most taps of a sweep (as pairs, in all); points of a row

@@ -617,8 +617,7 @@ cudaError_t Launcher<R>::observables(cudaStream_t s, const void* A, const KParam
                                      double* partials, DevScalars* sc) {
     using T = typename V2<R>::T;
     const int rows = obs_rows(p.nx, p.ny);
-    const dim3 grid = p.dim == 2 ? dim3(ceil_div(p.nx, 32), ceil_div(p.ny, 4 * rows)) : dim3(ceil_div(p.nx, 128));
-    k_observables<R><<<grid, 128, 0, s>>>((const T*)A, p, omega_t, partials, sc, rows);
+    k_observables<R><<<obs_grid(p.dim, p.nx, p.ny), 128, 0, s>>>((const T*)A, p, omega_t, partials, sc, rows);
     return cudaGetLastError();
 }
 

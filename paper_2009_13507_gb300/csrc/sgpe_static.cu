@@ -25,15 +25,15 @@ using namespace sgpe;
 namespace {
 
 // Scratch: a DevScalars block (tickets, error flag, observables) in the first
-// 512 bytes, then the per-block partial sums (kObsAcc doubles per block). The limit on the
-// grid counts one block per 32 x 4 points, kMaxBlocks of them; the kernel launches fewer
-// (strips of obs_rows rows a warp: at most 16 x 608 warps' worth on the largest grids).
-constexpr size_t kScratchBytes = 1u << 20;  // 1 MiB per device
-constexpr size_t kScalarsBytes = 512;
-constexpr size_t kMaxBlocks = (kScratchBytes - 256) / (kObsAcc * sizeof(double));
-static_assert(sizeof(DevScalars) <= kScalarsBytes, "DevScalars must fit its slot");
+// kObsScalarsBytes, then the per-block partial sums (kObsAcc doubles per block). The limit
+// on the grid counts one block per 32 x 4 points, kObsMaxBlocks of them. The kernel launches
+// obs_grid of them: fewer where a warp takes several rows, but just as many on grids of at
+// most four rows, so the room is for all kObsMaxBlocks.
+static_assert(sizeof(DevScalars) <= kObsScalarsBytes, "DevScalars must fit its slot");
+static_assert(kObsScalarsBytes + kObsMaxBlocks * kObsAcc * sizeof(double) <= kObsScratchBytes,
+              "the partial sums of the largest accepted grid must fit the scratch");
 
-static __device__ __align__(256) unsigned char g_obs_scratch[kScratchBytes];
+static __device__ __align__(256) unsigned char g_obs_scratch[kObsScratchBytes];
 
 constexpr int kMaxDevices = 64;
 std::mutex g_mutex;
@@ -85,12 +85,12 @@ extern "C" sgpe_status sgpe_observables_noalloc(const void* psi_dev, int dim, in
         return SGPE_EINVAL;
     }
     const size_t blocks = (size_t)ceil_div(nx, 32) * (size_t)ceil_div(ny, 4);
-    if (blocks > kMaxBlocks) {
+    if (blocks > kObsMaxBlocks) {
         char msg[200];
         snprintf(msg, sizeof(msg),
                  "sgpe_observables_noalloc: grid %dx%d needs %zu reduction blocks, the static scratch holds %zu "
                  "(at most about %zu grid points)",
-                 nx, ny, blocks, kMaxBlocks, kMaxBlocks * 128);
+                 nx, ny, blocks, kObsMaxBlocks, kObsMaxBlocks * 128);
         set_thread_error(msg);
         return SGPE_EUNSUPPORTED;
     }
@@ -100,7 +100,7 @@ extern "C" sgpe_status sgpe_observables_noalloc(const void* psi_dev, int dim, in
     // the same kernel constants as a context's sgpe_energy (dt plays no part in the observables)
     const KParams k = make_kparams(dim, nx, ny, dx, dy, p);
     DevScalars* sc = (DevScalars*)base;
-    double* partials = (double*)(base + kScalarsBytes);
+    double* partials = (double*)(base + kObsScalarsBytes);
     // The scratch keeps the previous call's contents: the ticket and the error
     // flag must start at zero.
     if (e == cudaSuccess) e = cudaMemsetAsync(sc, 0, sizeof(DevScalars), s);
