@@ -968,6 +968,9 @@ __global__ void __launch_bounds__(256, 3)
     }
     if (tid == 0) {
         if (k != 0) q = q * exp2(-(double)k) * exp2(-(double)k);
+        // (integers carry no NaN: infinities and NaN among the tile's values make its sum one, so that
+        // the step sets the error flag and leaves the scale at 1)
+        if (PS::kShift && umx >= 0x7ff00000u) q = __longlong_as_double(0x7ff8000000000000ll);
         part[blockIdx.x] = q;
     }
 }
