@@ -53,8 +53,13 @@ typedef enum {
  * Arithmetic of the step:
  *  SGPE_C128  complex128 state and reductions at FP64 accuracy. 2D Lie steps
  *             with small dt form each substep's increment in pairs of FP32
- *             numbers and add it to the FP64 state; everything else is FP64
- *             arithmetic.
+ *             numbers (48 bits) where it is small against the state, and add it
+ *             to the FP64 state; large increments (strong SO, structure near the
+ *             grid scale, large dt mu) and everything else are FP64 arithmetic.
+ *             A substep's rounding is about 2^-53 of the largest |psi| within the
+ *             sweep's taps (at most 16 points along an axis), or 2^-58 of the
+ *             grid's largest |psi| where that is more: values far below the
+ *             largest ones keep that absolute, not a relative accuracy.
  *  SGPE_C64   complex64 state and sweeps, FP64 reductions (the precision form).
  *  SGPE_CDF   "double-float": every real number is a pair of FP32 numbers
  *             (about 48 significant bits), all step arithmetic on the FP32

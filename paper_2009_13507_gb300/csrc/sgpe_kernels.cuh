@@ -41,6 +41,7 @@ struct DevScalars {
     // state as the y sweep of step k saw it in umax[k % 3] (0: unknown); umax_slot: the running step's
     int pair_tick, umax_slot;
     unsigned umax[3];
+    unsigned umax_prev;  // that of the step before, where this step may compare with it (0: unknown)
 };
 
 // Crank-Nicolson coefficient tables for one axis and one time mode.

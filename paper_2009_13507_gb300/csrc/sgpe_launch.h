@@ -99,6 +99,7 @@ constexpr int kNormBlocks = 304;
 // segment's block (three threads a point); columns and rows of a y tile.
 constexpr int kPairPairTaps = 8;
 constexpr int kPairTaps = 16;
+constexpr int kPairNear = 2;  // taps that rough states take in FP64
 constexpr int kPairXPts = 160;
 constexpr int kPairPPts = 256;  // (of a block with one thread a point)
 constexpr int kPairCols = 8, kPairRows = 64;

@@ -546,6 +546,8 @@ static inline PairTab pair_tab(const PairHost& h) {
     }
     t.kp = h.kp;
     t.kt = h.kt;
+    t.v2 = (float)(h.wr[0] * h.wr[0] + h.wi[0] * h.wi[0]);
+    for (int k = 0; k < kPairNear; k++) t.near[k] = make_double2(h.wr[k], h.wi[k]);
     return t;
 }
 

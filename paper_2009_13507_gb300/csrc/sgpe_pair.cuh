@@ -7,9 +7,11 @@
 // FP64 pipe busy. But a step changes psi by little: SO, CALCNU, HERM and the
 // Crank-Nicolson sweeps each add an increment of size dt times an energy, 2^-6 to
 // 2^-15 of |psi| at the steps the method is used with. An increment formed in FP32
-// pairs (hi + lo, about 2^-47 relative) is then exact to 2^-53 |psi| and better,
+// pairs (hi + lo, about 2^-48 relative) is then exact to 2^-53 |psi| and better,
 // which is a rounding of the FP64 state itself; the sum state + increment is the
-// only operation that needs the state's full width. The FP64 evaluation rounds the
+// only operation that needs the state's full width. Increments that are not small
+// (large dt mu, strong SO, structure near the grid scale) are formed in FP64, see
+// pair_large. The FP64 evaluation rounds the
 // whole state some ten times a step instead. Error against an 80-bit reference (FP64
 // step -> this one): 128 x 112, 30 steps at dt = 2e-4, imaginary time 7.1e-16 -> 4.3e-16,
 // real time 3.8e-15 -> 1.2e-15; 64 x 80, 60 steps at bt = 0.075 4.4e-16 -> 4.7e-16 and
@@ -27,8 +29,9 @@
 // State values are split through the integer pipe (FP64 conversions would queue on
 // the FP64 pipe): hi rounded to 24 bits, lo the signed rest rounded to 24. A block
 // whose largest value lies outside 2^-40 .. 2^40 shifts all its values by a power
-// of two on the way in and out, so far tails and states of any scale keep their
-// relative accuracy.
+// of two on the way in and out, so states of any scale are treated alike. What is far below a
+// block's largest value (2^-74 without a shift) loses its lo to FP32's range, and so the
+// relative, not the absolute accuracy of its increments.
 //
 // The sweeps are short convolutions. T = tridiag(-bt, 1 + 2bt, -bt) = u (I - gS)(I -
 // gS^T), g = bt/u, has the Green's function g^|k| / (u (1 - g^2)) on the infinite line,
@@ -50,6 +53,8 @@ namespace sgpe {
 struct PairTab {
     float4 wr[kPairPairTaps], wi[kPairPairTaps], wf[kPairTaps];
     int kp, kt;
+    float v2;               // |v_0|^2
+    double2 near[kPairNear];  // v_0, v_1 in FP64
 };
 
 // -- lazy pairs -------------------------------------------------------------------
@@ -203,6 +208,9 @@ template <typename R> __device__ __forceinline__ cd pair_of(cx<R> a, unsigned bi
 template <typename R> __device__ __forceinline__ cd pair_diff(cx<R> a, cx<R> b, unsigned bias) {
     return cd(PairState<R>::diff(a.re, b.re, bias), PairState<R>::diff(a.im, b.im, bias));
 }
+template <typename R> __device__ __forceinline__ cx<R> pair_plus(cx<R> x, cd inc, unsigned bias) {
+    return {PairState<R>::plus(x.re, inc.re(), bias), PairState<R>::plus(x.im, inc.im(), bias)};
+}
 template <typename R> __device__ __forceinline__ unsigned pair_mag(cx<R> a) {
     return max(PairState<R>::mag(a.re), PairState<R>::mag(a.im));
 }
@@ -311,13 +319,21 @@ __device__ __noinline__ void nonlin_wide(double2* x, int st, const KParams& p, d
     for (int j = 0; j < 3; j++) x[j * st] = pack(u[j]);
 }
 
-// The sweep's increment at a point: M points at M_i of its line, st entries between links.
-template <bool IMAG> __device__ __forceinline__ cd pair_taps(const cd* M, int st, const PairTab& t) {
+// All pointwise substeps of one point in FP64, from the state in memory (d: the pending factors).
+template <bool IMAG>
+__device__ __noinline__ void point_wide(const double2* __restrict__ A, const KParams& p, const double* d, double Ot,
+                                        int ix, int iy, cx<double> (&u)[3]) {
+    pointwise_point<double, IMAG>(A, p, d, Ot, ix, iy, 7, u);
+}
+
+// The sweep's increment at a point by the taps k >= k0: M points at M_i of its line, st entries
+// between links.
+template <bool IMAG> __device__ __forceinline__ cd pair_taps(const cd* M, int st, const PairTab& t, int k0) {
     const int kp = t.kp, kt = t.kt;
     float2 f = make_float2(0.0f, 0.0f);
 #pragma unroll
     for (int k = kPairTaps - 1; k >= 1; k--) {
-        if (k < kp || k >= kt) continue;
+        if (k < kp || k >= kt || k < k0) continue;
         const float2 d = p_sub(M[k * st].h, M[-(k + 1) * st].h);
         f = __ffma2_rn(make_float2(t.wf[k].x, t.wf[k].y), d, f);
         if constexpr (!IMAG) f = __ffma2_rn(make_float2(t.wf[k].z, t.wf[k].w), make_float2(d.y, d.x), f);
@@ -325,7 +341,7 @@ template <bool IMAG> __device__ __forceinline__ cd pair_taps(const cd* M, int st
     cd acc(f, make_float2(0.0f, 0.0f));
 #pragma unroll
     for (int k = kPairPairTaps - 1; k >= 0; k--) {
-        if (k >= kp) continue;
+        if (k >= kp || k < k0) continue;
         const cd d = csub(M[k * st], M[-(k + 1) * st]);
         acc = cadd(acc, cscl2(make_float2(t.wr[k].x, t.wr[k].y), make_float2(t.wr[k].z, t.wr[k].w), d));
         if constexpr (!IMAG)
@@ -333,6 +349,75 @@ template <bool IMAG> __device__ __forceinline__ cd pair_taps(const cd* M, int st
     }
     return acc;
 }
+
+// The same by the taps k < kPairNear in FP64, of the point x_i and its two neighbours on either
+// side: at(q) is point i + q, zero at the ghost points -1 and n, and beyond those the line
+// continues oddly. (Out of line: the kernels' registers stay what the pairs need.)
+template <bool IMAG, typename At>
+__device__ __forceinline__ double2 near_taps(At&& at, int i, int n, double2 a, double2 b) {
+    const cx<double> zero = {0.0, 0.0};
+    const cx<double> x = at(0), m1 = i > 0 ? at(-1) : zero, p1 = i < n - 1 ? at(1) : zero;
+    const cx<double> m2 = i > 1 ? at(-2) : i == 1 ? zero : cx<double>{-x.re, -x.im};
+    const cx<double> p2 = i < n - 2 ? at(2) : i == n - 2 ? zero : cx<double>{-x.re, -x.im};
+    const cx<double> d0 = {fma(-2.0, x.re, m1.re + p1.re), fma(-2.0, x.im, m1.im + p1.im)};
+    const cx<double> d1 = {(m2.re - m1.re) + (p2.re - p1.re), (m2.im - m1.im) + (p2.im - p1.im)};
+    if constexpr (IMAG) return make_double2(fma(a.x, d0.re, b.x * d1.re), fma(a.x, d0.im, b.x * d1.im));
+    return make_double2(fma(a.x, d0.re, fma(-a.y, d0.im, fma(b.x, d1.re, -b.y * d1.im))),
+                        fma(a.x, d0.im, fma(a.y, d0.re, fma(b.x, d1.im, b.y * d1.re))));
+}
+// x: the point in memory, st entries between points.
+template <bool IMAG>
+__device__ __noinline__ double2 near_mem(const double2* x, int st, int i, int n, double2 a, double2 b) {
+    return near_taps<IMAG>([&](int q) { return unpack(x[q * st]); }, i, n, a, b);
+}
+// The same for points x + s (s: increments).
+template <bool IMAG>
+__device__ __noinline__ double2 near_inc(const double2* x, const cd* s, unsigned bias, int i, int n, double2 a, double2 b) {
+    return near_taps<IMAG>([&](int q) { return pair_plus<double>(unpack(x[q]), s[q], bias); }, i, n, a, b);
+}
+
+// -- what leaves the increments (complex128) -----------------------------------------------
+// A pair is exact to about 2^-48 of the increment, so an increment is as exact as the FP64
+// step's own roundings as long as it is small: below 2^-6 of the spinor at the point in
+// imaginary time, 2^-5 in real time (where the FP64 sweeps' complex products round more) and
+// for dt mu, or below 2^-10 of the grid's largest |psi| (known from the step before), where the
+// error stays under 2^-58 of that. Each kernel checks its increments against this; larger
+// ones are formed in FP64:
+//   kNonlin  dt mu or dt A: the block votes, and the warps that hold such points (three warps a
+//            group of points in k_pair_x) take CALCNU and HERM in FP64
+//   kSo      SO (strong coupling, structure near the grid scale): the block takes all pointwise
+//            substeps in FP64, from the state in memory
+//   kRough   a sweep (structure near the grid scale): the warp takes v_0 and v_1, which carry all
+//            but |g|^2 <= 2^-7 of it, in FP64
+// A block that has voted takes dt mu from 2^-6 on in FP64 (kNonlinLow).
+// Error against an 80-bit reference of 10 steps of independent random values, FP64 step /
+// increments without these checks / this: bt = 0.0625 imaginary time 5.9e-16 / 1.5e-15 / 3.1e-16,
+// bt = 0.08 real time 1.4e-15 / 8.1e-15 / 7.7e-16, gamma = 20 (dt = 2.5e-3, dx = 0.1) real time
+// 2.3e-15 / 6.1e-15 / 7.6e-16. They cost about 3 % of a step of a smooth state.
+constexpr unsigned kNonlin = 1u, kSo = 2u, kRough = 4u, kNonlinLow = 8u;
+// (U 2^(k - 4))^2 for the largest |psi| U of the step before as a high word (0: unknown), 2^k the block's shift
+__device__ __forceinline__ float pair_floor2(unsigned umax, int k) {
+    const int e = (int)(umax >> 20) - 1023 + k - 4;
+    return umax < (1u << 20) ? 0.0f : __int_as_float((127 + 2 * max(-60, min(60, e))) << 23);
+}
+// The squared limit of SO's and a sweep's increments next to rho (NaN stays in the increments).
+template <bool IMAG> __device__ __forceinline__ float pair_limit2(float rho, float floor2) {
+    return (IMAG ? 0.000244140625f : 0.0009765625f) * fmaxf(rho, floor2);
+}
+// What is too large at a point: so2, sw2 the squared increments of SO and of the sweep, ae the
+// largest |dt mu|, w = (dt A)^2.
+template <bool IMAG>
+__device__ __forceinline__ unsigned pair_large(float so2, float sw2, float rho, float floor2, float ae, float w) {
+    const float lim = pair_limit2<IMAG>(rho, floor2);
+    unsigned b = (so2 > lim ? kSo : 0u) | (sw2 > lim ? kRough : 0u);
+    if ((!(ae < 0.015625f) || !(w < 2.44140625e-4f)) && rho > 0.0f) {
+        // dt mu up to 2: against the floor; beyond (2^-40 of it), the value itself would lose its relative accuracy
+        const float big = ae < 2.0f ? rho * fmaxf(ae * ae, w) : rho * 2.81474976710656e14f;
+        if (big >= 0.000244140625f * floor2) b |= !(ae < 0.03125f) || !(w < 2.44140625e-4f) ? kNonlin | kNonlinLow : kNonlinLow;
+    }
+    return b;
+}
+__device__ __forceinline__ float norm2(float2 a) { return fmaf(a.x, a.x, a.y * a.y); }
 
 // -- kernel 1: pending scale, SO, CALCNU, HERM, Crank-Nicolson along x ------------------
 // One block per row segment (segment sg of nseg writes the points [o0, o1) of row iy and
@@ -347,11 +432,9 @@ template <bool IMAG> __device__ __forceinline__ cd pair_taps(const cd* M, int st
 // neighbouring state values, taken in the state's own width and then split (a rounding
 // of 2^-48 of the difference, not of the values), plus the differences of the increments.
 //
-// CALCNU's increment is as exact as the state's rounding for |dt mu| < 2^-5, or where
-// |psi| is below 2^-8 of the grid's largest (known from the step before), HERM's for
-// |dt A| < 2^-6. A block with a point outside that (complex128 only: larger steps, a wide
-// trap in the first step) runs both substeps in FP64 and restarts the increments from
-// the result.
+// A block with an increment too large for a pair (pair_large; complex128 only: larger steps, a
+// wide trap in the first step, rough states) takes what it has to FP64 and restarts the
+// increments from the result.
 constexpr int kPairXThreads = 3 * kPairXPts;
 
 template <typename R, bool IMAG>
@@ -368,13 +451,13 @@ __global__ void __launch_bounds__(kPairXThreads, 2)
     __shared__ double red[3], dsh[3];
     __shared__ df dms;
     __shared__ int far_s;
-    __shared__ unsigned wmax[kPairXThreads / 32];
+    __shared__ unsigned wmax[kPairXThreads / 32], large_s[kPairXPts / 32];
     const int tid = threadIdx.x, warp = tid >> 5, nw = blockDim.x >> 5, nwp = nw / 3;
     const int iy = blockIdx.x / nseg;
     const PairSeg sg = pair_seg(p.nx, nseg, t.kt + 1, blockIdx.x - iy * nseg);
     const int np = sg.a1 - sg.a0;
     const int j = warp / nwp, i = (warp - j * nwp) * 32 + (tid & 31), ix = sg.a0 + i;
-    const bool in = i < np, so = p.so_case != 0;
+    const bool in = i < np, out = in && ix >= sg.o0 && ix < sg.o1, so = p.so_case != 0;
     const size_t plane = (size_t)p.nx * p.ny, at = j * plane + (size_t)iy * p.nx + ix;
     const cx<R> zr = {R(0), R(0)};
     pdl_wait();
@@ -383,21 +466,21 @@ __global__ void __launch_bounds__(kPairXThreads, 2)
     const cx<R> ym = in && so && iy > 0 ? ld<R>(A, at - p.nx) : zr;
     const cx<R> yp = in && so && iy + 1 < p.ny ? ld<R>(A, at + p.nx) : zr;
     const bool from_parts = partials && *(volatile const int*)&sc->scale_src;
-    float U = 0.0f;  // a power of two at most the grid's largest |psi| of the step before (0: unknown)
+    unsigned um = 0u;  // the grid's largest |psi| of the step before (high word; 0: unknown)
     if (from_parts && warp < 3) {
         const double q = sum_partials_warp(partials + (size_t)warp * m, m);
         if ((tid & 31) == 0) red[warp] = q;
     }
     if constexpr (PS::kShift) {
         const int tick = *(volatile const int*)&sc->pair_tick;
-        const int e = (int)(*(volatile const unsigned*)&sc->umax[(tick + 2) % 3] >> 20) - 1023 + 127;
-        U = e < 1 ? 0.0f : __int_as_float(min(e, 254) << 23);
+        um = *(volatile const unsigned*)&sc->umax[(tick + 2) % 3];
         if (blockIdx.x == 0 && tid == 0) {  // the slot of this step's y sweep; the next step's is cleared
             sc->umax_slot = tick % 3;
             sc->umax[(tick + 1) % 3] = 0u;
         }
         const unsigned mx = __reduce_max_sync(0xffffffffu, max(pair_mag(x), max(pair_mag(ym), pair_mag(yp))));
         if ((tid & 31) == 0) wmax[warp] = mx;
+        if (tid < nwp) large_s[tid] = 0u;
     }
     __syncthreads();
     int k = 0;
@@ -424,6 +507,8 @@ __global__ void __launch_bounds__(kPairXThreads, 2)
             for (int c = 0; c < 3; c++) dsh[c] = sc->scale[c];
         }
         pair_near(dsh, &dms, &far_s);
+        // (the step before's values are not this one's after a factor far from 1)
+        if (PS::kShift && blockIdx.x == 0) sc->umax_prev = far_s ? 0u : um;
     }
     __syncthreads();
     // SO: rows +1 and -1 of H_SO take psi_0 (X with the sign +, -), row 0 psi_-1 - psi_+1 and their sum
@@ -442,6 +527,7 @@ __global__ void __launch_bounds__(kPairXThreads, 2)
         s = mz<IMAG>(so_form(hx, hy, P, Q));
     }
     bool relink = false;
+    float so2 = norm2(s.h);
     {
         const df dm = dms;
         if (far_s) {
@@ -465,6 +551,7 @@ __global__ void __launch_bounds__(kPairXThreads, 2)
                     h = cadd(h, so_form(lscale(lmul(hx, dc), f), lscale(lmul(hy, dc), f), P, Us[c][i]));
                 }
                 s = mz<IMAG>(h);
+                so2 = norm2(s.h);
             }
             x = {PS::times(x.re, dsh[j]), PS::times(x.im, dsh[j])};
             u = pair_of(x, bias);
@@ -482,7 +569,7 @@ __global__ void __launch_bounds__(kPairXThreads, 2)
     const df Ot = omega_tab ? df_from(__ldg(omega_tab + sc->step_idx) * 0.70710678118654752440) : kpair(p, KC_OMEGA);
     const df c2 = lscale(kpair(p, KC_C2), f);
     cd tn;
-    bool wide = false;
+    unsigned large = 0u;
     {
         const df rp = rs[0][i], r0 = rs[1][i], rm = rs[2][i], rpm = ladd(rp, rm);
         const int kx = ix - p.nx / 2, ky = iy - p.ny / 2;  // |k| <= 2048: k^2 is exact in FP32
@@ -492,12 +579,13 @@ __global__ void __launch_bounds__(kPairXThreads, 2)
         if (j != 1) q = ladd(r0, j == 0 ? lsub(rp, rm) : lsub(rm, rp));
         const df e = lfma(lscale(kpair(p, KC_NC2), f), q, base);
         if constexpr (PS::kShift) {
-            const float um = fmaxf(fabsf(u.h.x), fabsf(u.h.y)) * __int_as_float((127 + max(-126, min(126, -k))) << 23);
-            const float ae = fabsf(e.hi), ot = fabsf(Ot.hi);
+            const float ot = fabsf(Ot.hi);
             const float ea = fmaf(fabsf(c2.hi), sqrtf(rm.hi * r0.hi), ot), eb = fmaf(fabsf(c2.hi), sqrtf(r0.hi * rp.hi), ot);
-            const float w = p.kf[KC_DT2] * fmaf(ea, ea, eb * eb);
-            const bool big = um * (ae < 2.0f ? 256.0f : 1.0e12f) >= U;
-            wide = in && um > 0.0f && big && (!(ae < 0.03125f) || !(w < 2.44140625e-4f));
+            // (the first point of a segment inside the row has no link to its left, and writes nothing)
+            const float2 r = p_sub(Ls[j][H + i].h, Ls[j][H + i - 1].h);
+            if (in && (i > 0 || sg.a0 == 0))
+                large = pair_large<IMAG>(so2, relink ? 0.0f : t.v2 * norm2(r), rpm.hi + r0.hi, pair_floor2(relink ? 0u : um, k),
+                                   fabsf(e.hi), p.kf[KC_DT2] * fmaf(ea, ea, eb * eb));
         }
         if constexpr (IMAG) {
             tn = cscl(em1_pair(e), u);
@@ -508,16 +596,24 @@ __global__ void __launch_bounds__(kPairXThreads, 2)
         }
     }
     Us[j][i] = cadd(u, tn);
-    bool slow = relink;
-    if constexpr (PS::kShift)
-        slow = __syncthreads_or(wide || relink) != 0;
-    else
+    bool slow = relink, f64 = false;  // f64: this group of points takes CALCNU and HERM in FP64
+    unsigned bits = 0u;
+    const int grp = warp - j * nwp;
+    if constexpr (PS::kShift) {
+        if (large & (kNonlinLow | kSo)) atomicOr(&large_s[grp], large);
+        slow = __syncthreads_or(relink || (large & (kNonlin | kSo))) != 0;
+        if (slow) {
+            for (int w = 0; w < nwp; w++) bits |= large_s[w];
+            f64 = ((large_s[grp] & kNonlinLow) | (bits & kSo)) != 0u;
+        }
+    } else {
         __syncthreads();
+    }
     T* xs = reinterpret_cast<T*>(&Us[0][0]);  // [3][kPairXPts]
-    if (!PS::kShift || !slow) {
+    if (!f64) {
         s = cadd(s, tn);
-        const cd up = Us[0][i], u0 = Us[1][i], um = Us[2][i];
-        cd a = cscl(c2, cmulc(um, u0)), b = cscl(c2, cmulc(u0, up));
+        const cd up = Us[0][i], u0 = Us[1][i], um_ = Us[2][i];
+        cd a = cscl(c2, cmulc(um_, u0)), b = cscl(c2, cmulc(u0, up));
         a = cd(ladd(a.re(), Ot), a.im());
         b = cd(ladd(b.re(), Ot), b.im());
         const float w = p.kf[KC_DT2] *
@@ -534,21 +630,30 @@ __global__ void __launch_bounds__(kPairXThreads, 2)
         }
         // -s_z A u + k A^2 u: (A u)_0 = a* u_+ + b u_-; the rows +1, -1 are a, b* times -s_z u_0 +
         // k (A u)_0; (A^2 u)_0 = (|a|^2 + |b|^2) u_0
-        const cd A0 = cadd(cmulc(a, up), cmulp(b, um));
+        const cd A0 = cadd(cmulc(a, up), cmulp(b, um_));
         if (j == 1)
             s = cadd(s, cadd(mz<IMAG>(cscl(cs, A0)), cscl(lmul(ck, ladd(cnrm(a), cnrm(b))), u0)));
         else
             s = cadd(s, cmulp(j == 0 ? a : cjg(b), cadd(mz<IMAG>(cscl(cs, u0)), cscl(ck, A0))));
-        __syncthreads();  // every Us has been read
     }
+    __syncthreads();  // every Us has been read
+    int k0 = 0;
     if (slow) {
         if constexpr (PS::kShift) {
-            // the increments so far into the state, both substeps in FP64, increments from zero
+            // the increments so far into the state, the large ones in FP64, increments from zero
             if (in)
                 xs[j * kPairXPts + i] = pack(cx<R>{PS::plus(x.re, s.re(), bias), PS::plus(x.im, s.im(), bias)});
             __syncthreads();
             const double otd = omega_tab ? __ldg(omega_tab + sc->step_idx) * 0.70710678118654752440 : p.kd[KC_OMEGA];
-            if (tid < np) nonlin_wide<IMAG>(xs + tid, kPairXPts, p, otd, sg.a0 + tid, iy);
+            if (j == 0 && in && f64) {
+                if (bits & kSo) {
+                    cx<double> v[3];
+                    point_wide<IMAG>(A, p, dsh, otd, ix, iy, v);
+                    for (int c = 0; c < 3; c++) xs[c * kPairXPts + i] = pack(v[c]);
+                } else {
+                    nonlin_wide<IMAG>(xs + i, kPairXPts, p, otd, ix, iy);
+                }
+            }
             __syncthreads();
             x = in ? unpack(xs[j * kPairXPts + i]) : zr;
             s = czero();
@@ -559,6 +664,12 @@ __global__ void __launch_bounds__(kPairXThreads, 2)
         if (in) {
             Ls[j][H + i] = pair_diff(i + 1 < np ? unpack(xs[j * kPairXPts + i + 1]) : zr, x, bias);
             if (i == 0) Ls[j][H - 1] = sg.a0 == 0 ? pair_of(x, bias) : czero();
+        }
+        if constexpr (PS::kShift) {
+            if (__any_sync(0xffffffffu, relink || (bits & kSo) || (large & kRough))) {
+                k0 = kPairNear;
+                if (out) x = add(x, unpack(near_mem<IMAG>(xs + j * kPairXPts + i, 1, ix, p.nx, t.near[0], t.near[1])));
+            }
         }
         __syncthreads();
     }
@@ -583,9 +694,15 @@ __global__ void __launch_bounds__(kPairXThreads, 2)
         if (sg.a1 != p.nx && i < H) L[np + i] = czero();
     }
     __syncthreads();
-    if (in && ix >= sg.o0 && ix < sg.o1) {
-        const cd inc = cadd(s, pair_taps<IMAG>(Ls[j] + H + i, 1, t));
-        st<R>(Bout, at, cx<R>{PS::plus(x.re, inc.re(), bias), PS::plus(x.im, inc.im(), bias)});
+    if constexpr (PS::kShift) {
+        if (!slow && __any_sync(0xffffffffu, large & kRough)) {
+            k0 = kPairNear;
+            if (out) x = add(x, unpack(near_inc<IMAG>(A + at, &Us[j][i], bias, ix, p.nx, t.near[0], t.near[1])));
+        }
+    }
+    if (out) {
+        const cd inc = cadd(s, pair_taps<IMAG>(Ls[j] + H + i, 1, t, k0));
+        st<R>(Bout, at, pair_plus<R>(x, inc, bias));
     }
 }
 
@@ -614,12 +731,12 @@ __global__ void __launch_bounds__(kPairPPts, 2)
     __shared__ double red[3], dsh[3];
     __shared__ df dms;
     __shared__ int far_s;
-    __shared__ unsigned wmax[kPairPPts / 32];
+    __shared__ unsigned wmax[kPairPPts / 32], large_s[kPairPPts / 32];
     const int i = threadIdx.x, warp = i >> 5, nw = blockDim.x >> 5;
     const int iy = blockIdx.x / nseg;
     const PairSeg sg = pair_seg(p.nx, nseg, t.kt + 1, blockIdx.x - iy * nseg);
     const int np = sg.a1 - sg.a0, ix = sg.a0 + i;
-    const bool in = i < np, so = p.so_case != 0;
+    const bool in = i < np, out = in && ix >= sg.o0 && ix < sg.o1, so = p.so_case != 0;
     const size_t plane = (size_t)p.nx * p.ny, at = (size_t)iy * p.nx + ix;
     const cx<R> zr = {R(0), R(0)};
     pdl_wait();
@@ -632,7 +749,7 @@ __global__ void __launch_bounds__(kPairPPts, 2)
         yp[j] = in && so && iy + 1 < p.ny ? ld<R>(A, j * plane + at + p.nx) : zr;
     }
     const bool from_parts = partials && *(volatile const int*)&sc->scale_src;
-    float U = 0.0f;
+    unsigned um = 0u;
     if (from_parts)
         for (int j = warp; j < 3; j += nw) {
             const double q = sum_partials_warp(partials + (size_t)j * m, m);
@@ -640,8 +757,7 @@ __global__ void __launch_bounds__(kPairPPts, 2)
         }
     if constexpr (PS::kShift) {
         const int tick = *(volatile const int*)&sc->pair_tick;
-        const int e = (int)(*(volatile const unsigned*)&sc->umax[(tick + 2) % 3] >> 20) - 1023 + 127;
-        U = e < 1 ? 0.0f : __int_as_float(min(e, 254) << 23);
+        um = *(volatile const unsigned*)&sc->umax[(tick + 2) % 3];
         if (blockIdx.x == 0 && i == 0) {
             sc->umax_slot = tick % 3;
             sc->umax[(tick + 1) % 3] = 0u;
@@ -650,7 +766,10 @@ __global__ void __launch_bounds__(kPairPPts, 2)
 #pragma unroll
         for (int j = 0; j < 3; j++) mx = max(mx, max(pair_mag(x[j]), max(pair_mag(ym[j]), pair_mag(yp[j]))));
         mx = __reduce_max_sync(0xffffffffu, mx);
-        if ((i & 31) == 0) wmax[warp] = mx;
+        if ((i & 31) == 0) {
+            wmax[warp] = mx;
+            large_s[warp] = 0u;
+        }
     }
     __syncthreads();
     int k = 0;
@@ -681,10 +800,16 @@ __global__ void __launch_bounds__(kPairPPts, 2)
             for (int c = 0; c < 3; c++) dsh[c] = sc->scale[c];
         }
         pair_near(dsh, &dms, &far_s);
+        if (PS::kShift && blockIdx.x == 0) sc->umax_prev = far_s ? 0u : um;
     }
     __syncthreads();
     const df hx = kpair(p, KC_HX), hy = kpair(p, KC_HY);
     const bool relink = far_s != 0;
+    float so2 = 0.0f, r2 = 0.0f;
+    if (PS::kShift && !relink) {
+#pragma unroll
+        for (int j = 0; j < 3; j++) r2 += norm2(p_sub(L[j].h, Ls[j][H + i - 1].h));
+    }
     if (so) {
         cd X[3];
 #pragma unroll
@@ -711,6 +836,7 @@ __global__ void __launch_bounds__(kPairPPts, 2)
             s[2] = mz<IMAG>(csub(ay, ax));
             s[1] = mz<IMAG>(so_form(hx, hy, csub(X[2], X[0]), cadd(Y[0], Y[2])));
         }
+        so2 = norm2(s[0].h) + norm2(s[1].h) + norm2(s[2].h);
     }
     if (relink) {
         if (fabs(dsh[0]) > 1e6 || fabs(dsh[0]) < 1e-6) {
@@ -733,7 +859,7 @@ __global__ void __launch_bounds__(kPairPPts, 2)
     const df Ot = omega_tab ? df_from(__ldg(omega_tab + sc->step_idx) * 0.70710678118654752440) : kpair(p, KC_OMEGA);
     const df c2 = lscale(kpair(p, KC_C2), f);
     df e[3];
-    bool wide = false;
+    unsigned large = 0u;
     {
         const df rp = cnrm(u[0]), r0 = cnrm(u[1]), rm = cnrm(u[2]), rpm = ladd(rp, rm), dpm = lsub(rp, rm);
         const int kx = ix - p.nx / 2, ky = iy - p.ny / 2;
@@ -743,17 +869,26 @@ __global__ void __launch_bounds__(kPairPPts, 2)
         e[1] = lfma(nc2, rpm, base);
         e[2] = lfma(nc2, lsub(r0, dpm), base);
         if constexpr (PS::kShift) {
-            const float um = sqrtf(fmaxf(rp.hi, fmaxf(r0.hi, rm.hi))) * __int_as_float((127 + max(-126, min(126, -k))) << 23);
             const float ae = fmaxf(fabsf(e[0].hi), fmaxf(fabsf(e[1].hi), fabsf(e[2].hi))), ot = fabsf(Ot.hi);
             const float ea = fmaf(fabsf(c2.hi), sqrtf(rm.hi * r0.hi), ot), eb = fmaf(fabsf(c2.hi), sqrtf(r0.hi * rp.hi), ot);
-            const float w = p.kf[KC_DT2] * fmaf(ea, ea, eb * eb);
-            wide = in && um > 0.0f && um * (ae < 2.0f ? 256.0f : 1.0e12f) >= U && (!(ae < 0.03125f) || !(w < 2.44140625e-4f));
+            if (in && (i > 0 || sg.a0 == 0))
+                large = pair_large<IMAG>(so2, t.v2 * r2, rpm.hi + r0.hi, pair_floor2(relink ? 0u : um, k), ae,
+                                   p.kf[KC_DT2] * fmaf(ea, ea, eb * eb));
         }
     }
-    bool slow = relink;
-    if constexpr (PS::kShift) slow = __syncthreads_or(wide || relink) != 0;
+    bool slow = relink, f64 = false;
+    unsigned bits = 0u;
+    if constexpr (PS::kShift) {
+        if (large & (kNonlinLow | kSo)) atomicOr(&large_s[warp], large);
+        slow = __syncthreads_or(relink || (large & (kNonlin | kSo))) != 0;
+        if (slow) {
+            for (int w = 0; w < nw; w++) bits |= large_s[w];
+            f64 = ((large_s[warp] & kNonlinLow) | (bits & kSo)) != 0u;
+        }
+    }
     T* xs = reinterpret_cast<T*>(&Us[0][0]);  // [3][kPairPPts]
-    if (!PS::kShift || !slow) {
+    int k0 = 0;
+    if (!f64) {
 #pragma unroll
         for (int j = 0; j < 3; j++) {
             cd tn;
@@ -797,7 +932,12 @@ __global__ void __launch_bounds__(kPairPPts, 2)
                 v[j] = {PS::plus(x[j].re, s[j].re(), bias), PS::plus(x[j].im, s[j].im(), bias)};
                 s[j] = czero();
             }
-            nonlin_wide3<IMAG>(v, p, otd, ix, iy);
+            if (f64) {
+                if (!(bits & kSo))
+                    nonlin_wide3<IMAG>(v, p, otd, ix, iy);
+                else if (in)
+                    point_wide<IMAG>(A, p, dsh, otd, ix, iy, v);
+            }
 #pragma unroll
             for (int j = 0; j < 3; j++) x[j] = {v[j].re, v[j].im};
         }
@@ -810,11 +950,31 @@ __global__ void __launch_bounds__(kPairPPts, 2)
             L[j] = pair_diff(i + 1 < np ? unpack(xs[j * kPairPPts + i + 1]) : zr, x[j], bias);
             if (i == 0) Ls[j][H - 1] = sg.a0 == 0 ? pair_of(x[j], bias) : czero();
         }
+        if constexpr (PS::kShift) {
+            if (__any_sync(0xffffffffu, relink || (bits & kSo) || (large & kRough))) {
+                k0 = kPairNear;
+                if (out) {
+#pragma unroll
+                    for (int j = 0; j < 3; j++)
+                        x[j] = add(x[j], unpack(near_mem<IMAG>(xs + j * kPairPPts + i, 1, ix, p.nx, t.near[0], t.near[1])));
+                }
+            }
+        }
         __syncthreads();
     }
 #pragma unroll
     for (int j = 0; j < 3; j++) Us[j][i] = in ? s[j] : czero();
     __syncthreads();
+    if constexpr (PS::kShift) {
+        if (!slow && __any_sync(0xffffffffu, large & kRough)) {
+            k0 = kPairNear;
+            if (out) {
+#pragma unroll
+                for (int j = 0; j < 3; j++)
+                    x[j] = add(x[j], unpack(near_inc<IMAG>(A + j * plane + at, &Us[j][i], bias, ix, p.nx, t.near[0], t.near[1])));
+            }
+        }
+    }
 #pragma unroll
     for (int j = 0; j < 3; j++) {
         cd* Lj = Ls[j] + H;
@@ -833,10 +993,10 @@ __global__ void __launch_bounds__(kPairPPts, 2)
         if (sg.a1 != p.nx && i < H) Lj[np + i] = czero();
     }
     __syncthreads();
-    if (in && ix >= sg.o0 && ix < sg.o1) {
+    if (out) {
         // (one copy of the taps' code; the increments of this thread's own points)
 #pragma unroll 1
-        for (int j = 0; j < 3; j++) Us[j][i] = cadd(Us[j][i], pair_taps<IMAG>(Ls[j] + H + i, 1, t));
+        for (int j = 0; j < 3; j++) Us[j][i] = cadd(Us[j][i], pair_taps<IMAG>(Ls[j] + H + i, 1, t, k0));
 #pragma unroll
         for (int j = 0; j < 3; j++) {
             const cd inc = Us[j][i];
@@ -852,7 +1012,7 @@ __global__ void __launch_bounds__(kPairPPts, 2)
 // o0 - 1 - r, the others o1 + r - 16. Norm partials per tile: pairs per thread and block,
 // the tile's sum in FP64.
 template <typename R, bool IMAG>
-__global__ void __launch_bounds__(256, 3)
+__global__ void __launch_bounds__(256, 4)
     k_pair_y(const typename V2<R>::T* __restrict__ in, typename V2<R>::T* __restrict__ out, KParams p, PairTab t, int nrt,
              double* __restrict__ part, DevScalars* sc, int head, int renorm, int advance) {
     using PS = PairState<R>;
@@ -889,7 +1049,9 @@ __global__ void __launch_bounds__(256, 3)
     const cx<R> xh = row(rh), yh = row(rh + 1);
     int k = 0;
     unsigned umx = 0u;
+    float floor2 = 0.0f;
     if constexpr (PS::kShift) {
+        const unsigned um = *(volatile const unsigned*)&sc->umax_prev;
         unsigned mx = max(max(pair_mag(x0), pair_mag(x1)), pair_mag(xh));
         mx = __reduce_max_sync(0xffffffffu, mx);
         if ((tid & 31) == 0) wmax[tid >> 5] = mx;
@@ -898,6 +1060,7 @@ __global__ void __launch_bounds__(256, 3)
         for (int w = 0; w < 8; w++) mx = max(mx, wmax[w]);
         k = pair_shift(mx);
         umx = mx;
+        floor2 = pair_floor2(um, k);
         if (tid == 0) atomicMax(&sc->umax[sc->umax_slot], mx);
     }
     const unsigned bias = (unsigned)(896 - k) << 20;
@@ -922,14 +1085,27 @@ __global__ void __launch_bounds__(256, 3)
 #pragma unroll 1
     for (int q = 0; q < 2; q++) {
         const int r = o0 + 32 * q + rl;
-        if (r < n && colok) {
-            const cx<R> x = q ? x1 : x0;
-            const cd inc = pair_taps<IMAG>(M + (32 * q + rl) * CW, CW, t);
+        const bool act = r < n && colok;
+        const cd* Mr = M + (32 * q + rl) * CW;
+        cx<R> x = q ? x1 : x0;
+        cd xh = pair_of(x, bias);
+        int k0 = 0;
+        if constexpr (PS::kShift) {
+            // (one component is at hand: the check is against its own value)
+            const float2 d = p_sub(Mr[0].h, Mr[-CW].h);
+            if (__any_sync(0xffffffffu, act && t.v2 * norm2(d) > pair_limit2<IMAG>(norm2(xh.h), floor2))) {
+                k0 = kPairNear;
+                if (act) x = add(x, unpack(near_mem<IMAG>(in + base + (size_t)r * p.nx, p.nx, r, n, t.near[0], t.near[1])));
+                xh = pair_of(x, bias);
+            }
+        }
+        if (act) {
+            const cd inc = pair_taps<IMAG>(Mr, CW, t, k0);
             st<R>(out, base + (size_t)r * p.nx,
                   cx<R>{PS::plus(x.re, inc.re(), bias), PS::plus(x.im, inc.im(), bias)});
             // |o|^2: the squares of the low parts (all positive, below the rounding of the products'
             // error terms) are summed apart; dropped, they would bias the norm by 2^-49
-            const cd o = cadd(pair_of(x, bias), inc);
+            const cd o = cadd(xh, inc);
             acc = ladd(acc, cnrm(o));
             acc2 = fmaf(o.l.x, o.l.x, fmaf(o.l.y, o.l.y, acc2));
         }

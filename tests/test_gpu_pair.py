@@ -34,3 +34,77 @@ def test_a_non_finite_norm_suspends_the_renormalisation(nx, ny, what):
     got, ref = s.get_state()[:, 60:], f.get_state()[:, 60:]
     assert not np.any(np.isnan(got))
     assert np.linalg.norm(got - ref) <= 1e-15 * np.linalg.norm(ref)
+
+
+LD, CL = np.longdouble, np.clongdouble
+
+
+def _long_sweep(p, b, ax):
+    """(I - b L)^-1 (I + b L) p along an axis, L = tridiag(1, -2, 1), in long double."""
+    p = np.moveaxis(p, ax, 0)
+    d = (1 - 2 * b) * p
+    d[1:] += b * p[:-1]
+    d[:-1] += b * p[1:]
+    c = np.zeros(len(p), CL)
+    m = 1 + 2 * b
+    c[0], d[0] = -b / m, d[0] / m
+    for i in range(1, len(p)):
+        m = 1 + 2 * b + b * c[i - 1]
+        c[i], d[i] = -b / m, (d[i] + b * d[i - 1]) / m
+    for i in range(len(p) - 2, -1, -1):
+        d[i] -= c[i] * d[i + 1]
+    return np.moveaxis(d, 0, ax)
+
+
+def _long_steps(psi, steps, imag, dx, dt, c0, c2, gamma, omega):
+    """The Lie step with Rashba SO by explicit Euler (renormalised in imaginary time), in long double."""
+    psi, dx, dt = psi.astype(CL), LD(dx), LD(dt)
+    z = CL(dt) if imag else CL(1j) * dt
+    g, ot = LD(gamma) / np.sqrt(LD(2)), LD(omega) / np.sqrt(LD(2))
+    ny, nx = psi.shape[1:]
+    V = ((((np.arange(nx) - nx // 2) * dx) ** 2)[None, :] + (((np.arange(ny) - ny // 2) * dx) ** 2)[:, None]) / 2
+
+    def diff(u, ax):
+        o = np.zeros_like(u)
+        a, b = np.moveaxis(u, ax, 0), np.moveaxis(o, ax, 0)
+        b[:-1] += a[1:]
+        b[1:] -= a[:-1]
+        return o / (2 * dx)
+    for _ in range(steps):
+        X, Y = diff(psi, 2), diff(psi, 1)
+        psi = psi - z * g * np.stack([X[1] - 1j * Y[1], X[2] - X[0] - 1j * (Y[0] + Y[2]), -X[1] - 1j * Y[1]])
+        r = psi.real ** 2 + psi.imag ** 2
+        mu = np.stack([(r[0] - r[2]) + r[1], r[0] + r[2], (r[2] - r[0]) + r[1]]) * LD(c2) + V + LD(c0) * r.sum(0)
+        psi = psi * np.exp(-z * mu)
+        a, b = c2 * psi[2].conj() * psi[1] + ot, c2 * psi[1].conj() * psi[0] + ot
+        v = (z * z).real * (abs(a) ** 2 + abs(b) ** 2)
+        s = 1 + v / 6 * (1 + v / 20 * (1 + v / 42 * (1 + v / 72)))
+        k = LD(1) / 2 + v / 24 * (1 + v / 30 * (1 + v / 56 * (1 + v / 90)))
+        A1 = np.stack([a * psi[1], a.conj() * psi[0] + b * psi[2], b.conj() * psi[1]])
+        A2 = np.stack([a * A1[1], a.conj() * A1[0] + b * A1[2], b.conj() * A1[1]])
+        psi = psi - z * s * A1 + (z * z).real * k * A2
+        for ax in (2, 1):
+            psi = _long_sweep(psi, z / (4 * dx * dx), ax)
+        if imag:
+            psi = psi / np.sqrt((psi.real ** 2 + psi.imag ** 2).sum() * dx * dx)
+    return psi
+
+
+@pytest.mark.parametrize("imag", [True, False])
+@pytest.mark.parametrize("nx,ny,steps,dx,dt,gamma", [
+    (64, 48, 10, 0.1, 2.5e-3, 0.8), (64, 48, 10, 0.05, 8e-4, 0.8), (64, 48, 10, 0.1, 2.5e-3, 20.0),
+    (64, 48, 10, 0.05, 2e-4, 0.8), (168, 100, 5, 0.05, 8e-4, 0.8), (168, 100, 5, 0.1, 2.5e-3, 20.0)])
+def test_rough_states_keep_the_accuracy_of_fp64(nx, ny, steps, dx, dt, gamma, imag):
+    """Independent random values at every point, bt up to the most taps, strong SO: SO's and the
+    sweeps' increments are no longer small and leave the pairs. Against long double; the
+    bound is what nine roundings of 2^-53 a step (SO, CALCNU, HERM, two sweeps, the state between
+    them) leave when their signs are random: 3 * 2^-53 * sqrt(steps)."""
+    if np.finfo(LD).eps > 2.0 ** -60:
+        pytest.skip("long double is no wider than double here")
+    prob, s = make_pair(2, nx, ny, dx=dx, dt=dt, c0=20.0, c2=1.0, so_type=1, gamma=gamma, omega=0.5, renorm=1 if imag else 0)
+    psi = _rand(prob, nx + ny, env=8.0)
+    s.set_state(psi)
+    (s.step_imag if imag else s.step_real)(steps)
+    ref = _long_steps(psi, steps, imag, dx, dt, 20.0, 1.0, gamma, 0.5)
+    err = np.sqrt((abs(s.get_state() - ref) ** 2).sum() / (abs(ref) ** 2).sum())
+    assert err < 3 * 2.0 ** -53 * np.sqrt(steps)
