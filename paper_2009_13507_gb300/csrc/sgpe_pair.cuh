@@ -221,14 +221,17 @@ __device__ __forceinline__ int pair_shift(unsigned mx) {
     return (mx >= (983u << 20) && mx < (1063u << 20)) || mx == 0u || mx >= 0x7ff00000u ? 0 : 1023 - (int)(mx >> 20);
 }
 
-// The pending factors as d - 1 in a pair, where they are one factor with |d - 1| < 2^-6 (*is_far
-// otherwise, NaN too). One thread's chain that the whole block waits for: comparisons and the
+// The pending factors as d - 1 in a pair, where they are one factor with |d - 1| < 2^-6; *is_far 1
+// otherwise, 2 where one lies outside 1/2 .. 2 (NaN too): the step before's values then say nothing
+// about this one's. One thread's chain that the whole block waits for: comparisons and the
 // split on the integer pipe, where an FP64 instruction would take its 64 cycles.
 __device__ __forceinline__ void pair_near(const double* d, df* dm, int* is_far) {
     const double e = d[0] - 1.0;
     const long long b = __double_as_longlong(d[0]);
     *is_far = b != __double_as_longlong(d[1]) || b != __double_as_longlong(d[2]) ||
               ((unsigned)__double2hiint(e) & 0x7fffffffu) >= (1017u << 20);
+    for (int j = 0; j < 3; j++)
+        if ((unsigned)__double2hiint(d[j]) - (1022u << 20) >= (2u << 20)) *is_far = 2;
     *dm = split64(e, kBias0);
 }
 
@@ -242,11 +245,23 @@ static __device__ __noinline__ void sc_wide(df x, df* cm1, df* sn) {
     *cm1 = df_from(-2.0 * s * s);
     *sn = df_from(2.0 * s * c);
 }
-template <bool IMAG> __device__ __noinline__ void herm_wide(cd a, cd b, double dt, df* s, df* k) {
+// The HERM coefficients s, k for w = (dt A)^2 >= 2^-20: below 2^-12, all that stays in pairs, by the
+// series in pairs (the last term in FP32: its rounding is below 2^-55 of the coefficients), larger
+// through FP64.
+template <bool IMAG> __device__ __noinline__ void herm_wide(cd a, cd b, const KParams& p, df* s, df* k) {
+    const df w = lmul(kpair(p, KC_DT2), ladd(cnrm(a), cnrm(b)));
+    if (w.hi < 2.44140625e-4f) {
+        const df v = IMAG ? w : lneg(w);
+        const float rs = fmaf(v.hi, p.kf[KC_HS0 + 3], p.kf[KC_HS0 + 2]), rk = fmaf(v.hi, p.kf[KC_HK0 + 3], p.kf[KC_HK0 + 2]);
+        *s = lfma(ladd(kpair(p, KC_HS0 + 1), lmulf(v, rs)), v, kpair(p, KC_HS0));
+        const df q = lfma(ladd(kpair(p, KC_HK0 + 1), lmulf(v, rk)), v, kpair(p, KC_HK0));
+        *k = IMAG ? q : lneg(q);
+        return;
+    }
     const double ar = (double)a.h.x + (double)a.l.x, ai = (double)a.h.y + (double)a.l.y;
     const double br = (double)b.h.x + (double)b.l.x, bi = (double)b.h.y + (double)b.l.y;
     double sd, kd;
-    herm_coeffs<IMAG>(ar * ar + ai * ai + br * br + bi * bi, dt, &sd, &kd);
+    herm_coeffs<IMAG>(ar * ar + ai * ai + br * br + bi * bi, p.dt, &sd, &kd);
     *s = df_from(sd);
     *k = df_from(kd);
 }
@@ -309,14 +324,27 @@ __device__ __forceinline__ cd so_form(df gx, df gy, cd P, cd Q) {
     return cadd(cscl(gx, P), cscl(gy, cmulni(Q)));
 }
 
-// CALCNU and HERM of one point in FP64 (the blocks whose increments would be too large).
+// CALCNU of one point in FP64, and HERM where herm is set.
 template <bool IMAG>
-__device__ __noinline__ void nonlin_wide(double2* x, int st, const KParams& p, double Ot, int ix, int iy) {
-    cx<double> u[3] = {unpack(x[0]), unpack(x[st]), unpack(x[2 * st])};
+__device__ __noinline__ void nonlin_wide(cx<double> (&u)[3], const KParams& p, double Ot, int ix, int iy, bool herm) {
     const int kx = ix - p.nx / 2, ky = iy - p.ny / 2;
     calcnu_point_dt<IMAG>(u, p.kd[KC_NVX] * (kx * kx) + p.kd[KC_NVY] * (ky * ky), p);
-    herm_point<IMAG>(u, p.kd[KC_C2], Ot, p.kd[KC_DT], &p);
-    for (int j = 0; j < 3; j++) x[j * st] = pack(u[j]);
+    if (herm) herm_point<IMAG>(u, p.kd[KC_C2], Ot, p.kd[KC_DT], &p);
+}
+// CALCNU of component j of the point x (st entries between components) in FP64.
+template <bool IMAG>
+__device__ __noinline__ double2 calcnu_own(const double2* x, int st, int j, const KParams& p, int ix, int iy) {
+    const cx<double> u[3] = {unpack(x[0]), unpack(x[st]), unpack(x[2 * st])};
+    const int kx = ix - p.nx / 2, ky = iy - p.ny / 2;
+    const double rp = nrm(u[0]), r0 = nrm(u[1]), rm = nrm(u[2]);
+    const double base = fma(p.kd[KC_NC0], rp + r0 + rm, p.kd[KC_NVX] * (kx * kx) + p.kd[KC_NVY] * (ky * ky));
+    const double q = j == 1 ? rp + rm : j == 0 ? rp - rm + r0 : rm - rp + r0;
+    const double e = fma(p.kd[KC_NC2], q, base);
+    const cx<double> v = j == 0 ? u[0] : j == 1 ? u[1] : u[2];
+    if constexpr (IMAG) return pack(scl(exp_small(e), v));
+    double s, c;
+    sincos_small(e, &s, &c);
+    return pack(mul(cx<double>{c, s}, v));
 }
 
 // All pointwise substeps of one point in FP64, from the state in memory (d: the pending factors).
@@ -383,18 +411,18 @@ __device__ __noinline__ double2 near_inc(const double2* x, const cd* s, unsigned
 // for dt mu, or below 2^-10 of the grid's largest |psi| (known from the step before), where the
 // error stays under 2^-58 of that. Each kernel checks its increments against this; larger
 // ones are formed in FP64:
-//   kNonlin  dt mu or dt A: the block votes, and the warps that hold such points (three warps a
-//            group of points in k_pair_x) take CALCNU and HERM in FP64
+//   kNonlin  dt mu: the block takes CALCNU in FP64, HERM's increments start from there
+//   kHerm    dt A: the block takes CALCNU and HERM in FP64
 //   kSo      SO (strong coupling, structure near the grid scale): the block takes all pointwise
 //            substeps in FP64, from the state in memory
 //   kRough   a sweep (structure near the grid scale): the warp takes v_0 and v_1, which carry all
 //            but |g|^2 <= 2^-7 of it, in FP64
-// A block that has voted takes dt mu from 2^-6 on in FP64 (kNonlinLow).
 // Error against an 80-bit reference of 10 steps of independent random values, FP64 step /
 // increments without these checks / this: bt = 0.0625 imaginary time 5.9e-16 / 1.5e-15 / 3.1e-16,
 // bt = 0.08 real time 1.4e-15 / 8.1e-15 / 7.7e-16, gamma = 20 (dt = 2.5e-3, dx = 0.1) real time
 // 2.3e-15 / 6.1e-15 / 7.6e-16. They cost about 3 % of a step of a smooth state.
-constexpr unsigned kNonlin = 1u, kSo = 2u, kRough = 4u, kNonlinLow = 8u;
+constexpr unsigned kNonlin = 1u, kSo = 2u, kRough = 4u, kHerm = 8u;
+constexpr unsigned kWide = kNonlin | kSo | kHerm;  // pointwise substeps in FP64
 // (U 2^(k - 4))^2 for the largest |psi| U of the step before as a high word (0: unknown), 2^k the block's shift
 __device__ __forceinline__ float pair_floor2(unsigned umax, int k) {
     const int e = (int)(umax >> 20) - 1023 + k - 4;
@@ -410,19 +438,29 @@ template <bool IMAG>
 __device__ __forceinline__ unsigned pair_large(float so2, float sw2, float rho, float floor2, float ae, float w) {
     const float lim = pair_limit2<IMAG>(rho, floor2);
     unsigned b = (so2 > lim ? kSo : 0u) | (sw2 > lim ? kRough : 0u);
-    if ((!(ae < 0.015625f) || !(w < 2.44140625e-4f)) && rho > 0.0f) {
+    const bool wbig = !(w < 2.44140625e-4f);
+    if ((!(ae < 0.03125f) || wbig) && rho > 0.0f) {
         // dt mu up to 2: against the floor; beyond (2^-40 of it), the value itself would lose its relative accuracy
         const float big = ae < 2.0f ? rho * fmaxf(ae * ae, w) : rho * 2.81474976710656e14f;
-        if (big >= 0.000244140625f * floor2) b |= !(ae < 0.03125f) || !(w < 2.44140625e-4f) ? kNonlin | kNonlinLow : kNonlinLow;
+        if (big >= 0.000244140625f * floor2) b |= wbig ? kNonlin | kHerm : kNonlin;
     }
     return b;
+}
+// |x_(i+1) - 2 x_i + x_(i-1)|^2 of a point in memory (zero ghosts outside 0..n-1), from the leading 24 bits
+// of the values.
+__device__ __forceinline__ float bend2(const double2* x, int i, int n, unsigned bias) {
+    const double2 c = x[0], zero = make_double2(0.0, 0.0), l = i > 0 ? x[-1] : zero, r = i < n - 1 ? x[1] : zero;
+    const float a = split64(l.x, bias).hi + split64(r.x, bias).hi - 2.0f * split64(c.x, bias).hi;
+    const float b = split64(l.y, bias).hi + split64(r.y, bias).hi - 2.0f * split64(c.y, bias).hi;
+    return fmaf(a, a, b * b);
 }
 __device__ __forceinline__ float norm2(float2 a) { return fmaf(a.x, a.x, a.y * a.y); }
 
 // -- kernel 1: pending scale, SO, CALCNU, HERM, Crank-Nicolson along x ------------------
 // One block per row segment (segment sg of nseg writes the points [o0, o1) of row iy and
 // works on [a0, a1), kt + 1 points more at each end inside the row), one thread per point
-// and component, the components in warps of their own: each substep is the same short
+// and component, the components in warps of their own (three neighbouring warps a group of
+// 32 points, on different sub-partitions): each substep is the same short
 // code for all three, so a block's warps share its instruction lines and a small grid's
 // few blocks have three times the warps (64^2: 16.7 us a step with one thread a point, 12.9
 // so). The components meet in shared memory: the differences before SO, the densities
@@ -451,12 +489,12 @@ __global__ void __launch_bounds__(kPairXThreads, 2)
     __shared__ double red[3], dsh[3];
     __shared__ df dms;
     __shared__ int far_s;
-    __shared__ unsigned wmax[kPairXThreads / 32], large_s[kPairXPts / 32];
+    __shared__ unsigned wmax[kPairXThreads / 32], large_s;
     const int tid = threadIdx.x, warp = tid >> 5, nw = blockDim.x >> 5, nwp = nw / 3;
     const int iy = blockIdx.x / nseg;
     const PairSeg sg = pair_seg(p.nx, nseg, t.kt + 1, blockIdx.x - iy * nseg);
     const int np = sg.a1 - sg.a0;
-    const int j = warp / nwp, i = (warp - j * nwp) * 32 + (tid & 31), ix = sg.a0 + i;
+    const int grp = warp / 3, j = warp - 3 * grp, i = grp * 32 + (tid & 31), ix = sg.a0 + i;
     const bool in = i < np, out = in && ix >= sg.o0 && ix < sg.o1, so = p.so_case != 0;
     const size_t plane = (size_t)p.nx * p.ny, at = j * plane + (size_t)iy * p.nx + ix;
     const cx<R> zr = {R(0), R(0)};
@@ -480,7 +518,7 @@ __global__ void __launch_bounds__(kPairXThreads, 2)
         }
         const unsigned mx = __reduce_max_sync(0xffffffffu, max(pair_mag(x), max(pair_mag(ym), pair_mag(yp))));
         if ((tid & 31) == 0) wmax[warp] = mx;
-        if (tid < nwp) large_s[tid] = 0u;
+        if (tid == 0) large_s = 0u;
     }
     __syncthreads();
     int k = 0;
@@ -507,10 +545,10 @@ __global__ void __launch_bounds__(kPairXThreads, 2)
             for (int c = 0; c < 3; c++) dsh[c] = sc->scale[c];
         }
         pair_near(dsh, &dms, &far_s);
-        // (the step before's values are not this one's after a factor far from 1)
-        if (PS::kShift && blockIdx.x == 0) sc->umax_prev = far_s ? 0u : um;
+        if (PS::kShift && blockIdx.x == 0) sc->umax_prev = far_s > 1 ? 0u : um;
     }
     __syncthreads();
+    if (far_s > 1) um = 0u;
     // SO: rows +1 and -1 of H_SO take psi_0 (X with the sign +, -), row 0 psi_-1 - psi_+1 and their sum
     const df hx = kpair(p, KC_HX), hy = kpair(p, KC_HY);
     auto xdiff = [&](int c) { return cadd(Ls[c][H + i], Ls[c][H + i - 1]); };
@@ -584,7 +622,7 @@ __global__ void __launch_bounds__(kPairXThreads, 2)
             // (the first point of a segment inside the row has no link to its left, and writes nothing)
             const float2 r = p_sub(Ls[j][H + i].h, Ls[j][H + i - 1].h);
             if (in && (i > 0 || sg.a0 == 0))
-                large = pair_large<IMAG>(so2, relink ? 0.0f : t.v2 * norm2(r), rpm.hi + r0.hi, pair_floor2(relink ? 0u : um, k),
+                large = pair_large<IMAG>(so2, t.v2 * norm2(r), rpm.hi + r0.hi, pair_floor2(um, k),
                                    fabsf(e.hi), p.kf[KC_DT2] * fmaf(ea, ea, eb * eb));
         }
         if constexpr (IMAG) {
@@ -596,23 +634,62 @@ __global__ void __launch_bounds__(kPairXThreads, 2)
         }
     }
     Us[j][i] = cadd(u, tn);
-    bool slow = relink, f64 = false;  // f64: this group of points takes CALCNU and HERM in FP64
+    bool slow = relink, herm = true;  // herm: HERM in pairs
     unsigned bits = 0u;
-    const int grp = warp - j * nwp;
+    const unsigned votes = kWide | (relink ? kRough : 0u);  // (links anew anyway: rough blocks restart too)
     if constexpr (PS::kShift) {
-        if (large & (kNonlinLow | kSo)) atomicOr(&large_s[grp], large);
-        slow = __syncthreads_or(relink || (large & (kNonlin | kSo))) != 0;
-        if (slow) {
-            for (int w = 0; w < nwp; w++) bits |= large_s[w];
-            f64 = ((large_s[grp] & kNonlinLow) | (bits & kSo)) != 0u;
+        if (__any_sync(0xffffffffu, large & votes)) {
+            const unsigned all = __reduce_or_sync(0xffffffffu, large);
+            if ((threadIdx.x & 31) == 0) atomicOr(&large_s, all);
         }
+        if (__syncthreads_or(large & votes)) bits = large_s;
+        if (far_s > 1) bits |= kRough;
+        slow = relink || bits;
     } else {
         __syncthreads();
     }
     T* xs = reinterpret_cast<T*>(&Us[0][0]);  // [3][kPairXPts]
-    if (!f64) {
+    cd up, u0, um_;
+    if (PS::kShift && bits) {
+        if constexpr (PS::kShift) {
+            // the increments so far into the state, the large ones in FP64; HERM's from there
+            if (!(bits & kWide)) s = cadd(s, tn);
+            if (in) xs[j * kPairXPts + i] = pack(pair_plus<R>(x, s, bias));
+            __syncthreads();
+            // CALCNU by each component for itself; where HERM or SO is large too, one thread a point takes all
+            herm = !(bits & (kHerm | kSo));
+            if (in && (bits & kWide)) {
+                if (herm) {
+                    x = unpack(calcnu_own<IMAG>(xs + i, kPairXPts, j, p, ix, iy));
+                } else if (j == 0) {
+                    const double otd = omega_tab ? __ldg(omega_tab + sc->step_idx) * 0.70710678118654752440 : p.kd[KC_OMEGA];
+                    cx<double> v[3];
+                    for (int c = 0; c < 3; c++) v[c] = unpack(xs[c * kPairXPts + i]);
+                    if (bits & kSo)
+                        point_wide<IMAG>(A, p, dsh, otd, ix, iy, v);
+                    else
+                        nonlin_wide<IMAG>(v, p, otd, ix, iy, true);
+                    for (int c = 0; c < 3; c++) xs[c * kPairXPts + i] = pack(v[c]);
+                }
+            }
+            __syncthreads();
+            if (in && (bits & kWide) && herm) xs[j * kPairXPts + i] = pack(x);
+            __syncthreads();
+            x = in ? unpack(xs[j * kPairXPts + i]) : zr;
+            s = up = u0 = um_ = czero();
+            if (in && herm) {
+                up = pair_of(unpack(xs[i]), bias);
+                u0 = pair_of(unpack(xs[kPairXPts + i]), bias);
+                um_ = pair_of(unpack(xs[2 * kPairXPts + i]), bias);
+            }
+        }
+    } else {
         s = cadd(s, tn);
-        const cd up = Us[0][i], u0 = Us[1][i], um_ = Us[2][i];
+        up = Us[0][i];
+        u0 = Us[1][i];
+        um_ = Us[2][i];
+    }
+    if (herm) {
         cd a = cscl(c2, cmulc(um_, u0)), b = cscl(c2, cmulc(u0, up));
         a = cd(ladd(a.re(), Ot), a.im());
         b = cd(ladd(b.re(), Ot), b.im());
@@ -626,7 +703,7 @@ __global__ void __launch_bounds__(kPairXThreads, 2)
             ck = laddf(kpair(p, KC_HK0), v * fmaf(p.kf[KC_HK0 + 2], v, p.kf[KC_HK0 + 1]));
             if (!IMAG) ck = lneg(ck);
         } else {
-            herm_wide<IMAG>(a, b, p.dt, &cs, &ck);
+            herm_wide<IMAG>(a, b, p, &cs, &ck);
         }
         // -s_z A u + k A^2 u: (A u)_0 = a* u_+ + b u_-; the rows +1, -1 are a, b* times -s_z u_0 +
         // k (A u)_0; (A^2 u)_0 = (|a|^2 + |b|^2) u_0
@@ -636,51 +713,41 @@ __global__ void __launch_bounds__(kPairXThreads, 2)
         else
             s = cadd(s, cmulp(j == 0 ? a : cjg(b), cadd(mz<IMAG>(cscl(cs, u0)), cscl(ck, A0))));
     }
-    __syncthreads();  // every Us has been read
+    __syncthreads();  // every Us (xs) has been read
     int k0 = 0;
+    const bool fresh = PS::kShift && bits;  // the increments start from zero
     if (slow) {
-        if constexpr (PS::kShift) {
-            // the increments so far into the state, the large ones in FP64, increments from zero
-            if (in)
-                xs[j * kPairXPts + i] = pack(cx<R>{PS::plus(x.re, s.re(), bias), PS::plus(x.im, s.im(), bias)});
-            __syncthreads();
-            const double otd = omega_tab ? __ldg(omega_tab + sc->step_idx) * 0.70710678118654752440 : p.kd[KC_OMEGA];
-            if (j == 0 && in && f64) {
-                if (bits & kSo) {
-                    cx<double> v[3];
-                    point_wide<IMAG>(A, p, dsh, otd, ix, iy, v);
-                    for (int c = 0; c < 3; c++) xs[c * kPairXPts + i] = pack(v[c]);
-                } else {
-                    nonlin_wide<IMAG>(xs + i, kPairXPts, p, otd, ix, iy);
-                }
-            }
-            __syncthreads();
-            x = in ? unpack(xs[j * kPairXPts + i]) : zr;
+        if (fresh) {
+            x = pair_plus<R>(x, s, bias);
             s = czero();
-        } else {
-            if (in) xs[j * kPairXPts + i] = pack(x);
-            __syncthreads();
         }
+        if (in) xs[j * kPairXPts + i] = pack(x);
+        __syncthreads();
         if (in) {
             Ls[j][H + i] = pair_diff(i + 1 < np ? unpack(xs[j * kPairXPts + i + 1]) : zr, x, bias);
             if (i == 0) Ls[j][H - 1] = sg.a0 == 0 ? pair_of(x, bias) : czero();
         }
         if constexpr (PS::kShift) {
-            if (__any_sync(0xffffffffu, relink || (bits & kSo) || (large & kRough))) {
-                k0 = kPairNear;
-                if (out) x = add(x, unpack(near_mem<IMAG>(xs + j * kPairXPts + i, 1, ix, p.nx, t.near[0], t.near[1])));
+            if (fresh) {
+                if (__any_sync(0xffffffffu, out && t.v2 * bend2(xs + j * kPairXPts + i, ix, p.nx, bias) >
+                                                       pair_limit2<IMAG>(norm2(pair_of(x, bias).h), pair_floor2(um, k)))) {
+                    k0 = kPairNear;
+                    if (out) x = add(x, unpack(near_mem<IMAG>(xs + j * kPairXPts + i, 1, ix, p.nx, t.near[0], t.near[1])));
+                }
             }
         }
         __syncthreads();
     }
     // the links of the updated state, mirrored about the line's ghost points (zero past the
     // ends of a segment inside the row: those links weigh less than 2^-56)
-    Us[j][i] = in ? s : czero();
-    __syncthreads();
+    if (!fresh) {
+        Us[j][i] = in ? s : czero();
+        __syncthreads();
+    }
     {
         cd* L = Ls[j] + H;
         if (in) {
-            const cd M = cadd(L[i], csub(i + 1 < np ? Us[j][i + 1] : czero(), s));
+            const cd M = fresh ? L[i] : cadd(L[i], csub(i + 1 < np ? Us[j][i + 1] : czero(), s));
             L[i] = M;
             if (sg.a0 == 0 && i < H - 2) L[-3 - i] = M;                      // M_(-2-k) = M_(-1+k)
             if (sg.a1 == p.nx && np - 1 - i < H) L[2 * np - 1 - i] = M;      // M_(n+k) = M_(n-1-k)
@@ -711,13 +778,6 @@ __global__ void __launch_bounds__(kPairXThreads, 2)
 // three times: 4.9 M against 10.9 M at 256^2) and needs half the barriers (256^2: 41 -> 25 us
 // a step). Bound by instruction issue and the FP64 pipe's 24 instructions a point. Segments
 // of up to kPairPPts points.
-template <bool IMAG>
-__device__ __noinline__ void nonlin_wide3(cx<double> (&u)[3], const KParams& p, double Ot, int ix, int iy) {
-    const int kx = ix - p.nx / 2, ky = iy - p.ny / 2;
-    calcnu_point_dt<IMAG>(u, p.kd[KC_NVX] * (kx * kx) + p.kd[KC_NVY] * (ky * ky), p);
-    herm_point<IMAG>(u, p.kd[KC_C2], Ot, p.kd[KC_DT], &p);
-}
-
 template <typename R, bool IMAG>
 __global__ void __launch_bounds__(kPairPPts, 2)
     k_pair_xp(const typename V2<R>::T* __restrict__ A, typename V2<R>::T* __restrict__ Bout, KParams p, DevScalars* sc,
@@ -731,7 +791,7 @@ __global__ void __launch_bounds__(kPairPPts, 2)
     __shared__ double red[3], dsh[3];
     __shared__ df dms;
     __shared__ int far_s;
-    __shared__ unsigned wmax[kPairPPts / 32], large_s[kPairPPts / 32];
+    __shared__ unsigned wmax[kPairPPts / 32], large_s;
     const int i = threadIdx.x, warp = i >> 5, nw = blockDim.x >> 5;
     const int iy = blockIdx.x / nseg;
     const PairSeg sg = pair_seg(p.nx, nseg, t.kt + 1, blockIdx.x - iy * nseg);
@@ -766,10 +826,8 @@ __global__ void __launch_bounds__(kPairPPts, 2)
 #pragma unroll
         for (int j = 0; j < 3; j++) mx = max(mx, max(pair_mag(x[j]), max(pair_mag(ym[j]), pair_mag(yp[j]))));
         mx = __reduce_max_sync(0xffffffffu, mx);
-        if ((i & 31) == 0) {
-            wmax[warp] = mx;
-            large_s[warp] = 0u;
-        }
+        if ((i & 31) == 0) wmax[warp] = mx;
+        if (i == 0) large_s = 0u;
     }
     __syncthreads();
     int k = 0;
@@ -800,13 +858,14 @@ __global__ void __launch_bounds__(kPairPPts, 2)
             for (int c = 0; c < 3; c++) dsh[c] = sc->scale[c];
         }
         pair_near(dsh, &dms, &far_s);
-        if (PS::kShift && blockIdx.x == 0) sc->umax_prev = far_s ? 0u : um;
+        if (PS::kShift && blockIdx.x == 0) sc->umax_prev = far_s > 1 ? 0u : um;
     }
     __syncthreads();
+    if (far_s > 1) um = 0u;
     const df hx = kpair(p, KC_HX), hy = kpair(p, KC_HY);
     const bool relink = far_s != 0;
     float so2 = 0.0f, r2 = 0.0f;
-    if (PS::kShift && !relink) {
+    if (PS::kShift) {
 #pragma unroll
         for (int j = 0; j < 3; j++) r2 += norm2(p_sub(L[j].h, Ls[j][H + i - 1].h));
     }
@@ -872,23 +931,25 @@ __global__ void __launch_bounds__(kPairPPts, 2)
             const float ae = fmaxf(fabsf(e[0].hi), fmaxf(fabsf(e[1].hi), fabsf(e[2].hi))), ot = fabsf(Ot.hi);
             const float ea = fmaf(fabsf(c2.hi), sqrtf(rm.hi * r0.hi), ot), eb = fmaf(fabsf(c2.hi), sqrtf(r0.hi * rp.hi), ot);
             if (in && (i > 0 || sg.a0 == 0))
-                large = pair_large<IMAG>(so2, t.v2 * r2, rpm.hi + r0.hi, pair_floor2(relink ? 0u : um, k), ae,
+                large = pair_large<IMAG>(so2, t.v2 * r2, rpm.hi + r0.hi, pair_floor2(um, k), ae,
                                    p.kf[KC_DT2] * fmaf(ea, ea, eb * eb));
         }
     }
-    bool slow = relink, f64 = false;
+    bool slow = relink, herm = true;
     unsigned bits = 0u;
+    const unsigned votes = kWide | (relink ? kRough : 0u);
     if constexpr (PS::kShift) {
-        if (large & (kNonlinLow | kSo)) atomicOr(&large_s[warp], large);
-        slow = __syncthreads_or(relink || (large & (kNonlin | kSo))) != 0;
-        if (slow) {
-            for (int w = 0; w < nw; w++) bits |= large_s[w];
-            f64 = ((large_s[warp] & kNonlinLow) | (bits & kSo)) != 0u;
+        if (__any_sync(0xffffffffu, large & votes)) {
+            const unsigned all = __reduce_or_sync(0xffffffffu, large);
+            if ((threadIdx.x & 31) == 0) atomicOr(&large_s, all);
         }
+        if (__syncthreads_or(large & votes)) bits = large_s;
+        if (far_s > 1) bits |= kRough;
+        slow = relink || bits;
     }
     T* xs = reinterpret_cast<T*>(&Us[0][0]);  // [3][kPairPPts]
     int k0 = 0;
-    if (!f64) {
+    if (!(bits & kWide)) {
 #pragma unroll
         for (int j = 0; j < 3; j++) {
             cd tn;
@@ -902,6 +963,26 @@ __global__ void __launch_bounds__(kPairPPts, 2)
             s[j] = cadd(s[j], tn);
             u[j] = cadd(u[j], tn);
         }
+    } else {
+        if constexpr (PS::kShift) {
+            const double otd = omega_tab ? __ldg(omega_tab + sc->step_idx) * 0.70710678118654752440 : p.kd[KC_OMEGA];
+            herm = !(bits & (kHerm | kSo));
+            cx<double> v[3];
+#pragma unroll
+            for (int j = 0; j < 3; j++) v[j] = pair_plus<R>(x[j], s[j], bias);
+            if (!(bits & kSo))
+                nonlin_wide<IMAG>(v, p, otd, ix, iy, !herm);
+            else if (in)
+                point_wide<IMAG>(A, p, dsh, otd, ix, iy, v);
+#pragma unroll
+            for (int j = 0; j < 3; j++) {
+                x[j] = v[j];
+                u[j] = pair_of(v[j], bias);
+                s[j] = czero();
+            }
+        }
+    }
+    if (herm) {
         cd a = cscl(c2, cmulc(u[2], u[1])), b = cscl(c2, cmulc(u[1], u[0]));
         a = cd(ladd(a.re(), Ot), a.im());
         b = cd(ladd(b.re(), Ot), b.im());
@@ -914,7 +995,7 @@ __global__ void __launch_bounds__(kPairPPts, 2)
             ck = laddf(kpair(p, KC_HK0), v * fmaf(p.kf[KC_HK0 + 2], v, p.kf[KC_HK0 + 1]));
             if (!IMAG) ck = lneg(ck);
         } else {
-            herm_wide<IMAG>(a, b, p.dt, &cs, &ck);
+            herm_wide<IMAG>(a, b, p, &cs, &ck);
         }
         // -s_z A u + k A^2 u = A (-s_z u + k A u) row by row, (A^2 u)_0 = (|a|^2 + |b|^2) u_0
         const cd A0 = cadd(cmulc(a, u[0]), cmulp(b, u[2]));
@@ -923,23 +1004,14 @@ __global__ void __launch_bounds__(kPairPPts, 2)
         s[2] = cadd(s[2], cmulc(b, m0));
         s[1] = cadd(s[1], cadd(mz<IMAG>(cscl(cs, A0)), cscl(lmul(ck, ladd(cnrm(a), cnrm(b))), u[1])));
     }
+    const bool fresh = PS::kShift && bits;  // the increments start from zero
     if (slow) {
-        if constexpr (PS::kShift) {
-            const double otd = omega_tab ? __ldg(omega_tab + sc->step_idx) * 0.70710678118654752440 : p.kd[KC_OMEGA];
-            cx<double> v[3];
+        if (fresh) {
 #pragma unroll
             for (int j = 0; j < 3; j++) {
-                v[j] = {PS::plus(x[j].re, s[j].re(), bias), PS::plus(x[j].im, s[j].im(), bias)};
+                if (herm) x[j] = pair_plus<R>(x[j], s[j], bias);
                 s[j] = czero();
             }
-            if (f64) {
-                if (!(bits & kSo))
-                    nonlin_wide3<IMAG>(v, p, otd, ix, iy);
-                else if (in)
-                    point_wide<IMAG>(A, p, dsh, otd, ix, iy, v);
-            }
-#pragma unroll
-            for (int j = 0; j < 3; j++) x[j] = {v[j].re, v[j].im};
         }
 #pragma unroll
         for (int j = 0; j < 3; j++)
@@ -951,12 +1023,22 @@ __global__ void __launch_bounds__(kPairPPts, 2)
             if (i == 0) Ls[j][H - 1] = sg.a0 == 0 ? pair_of(x[j], bias) : czero();
         }
         if constexpr (PS::kShift) {
-            if (__any_sync(0xffffffffu, relink || (bits & kSo) || (large & kRough))) {
-                k0 = kPairNear;
+            if (fresh) {
+                float b2 = 0.0f, rho = 0.0f;
                 if (out) {
 #pragma unroll
-                    for (int j = 0; j < 3; j++)
-                        x[j] = add(x[j], unpack(near_mem<IMAG>(xs + j * kPairPPts + i, 1, ix, p.nx, t.near[0], t.near[1])));
+                    for (int j = 0; j < 3; j++) {
+                        b2 += bend2(xs + j * kPairPPts + i, ix, p.nx, bias);
+                        rho += norm2(pair_of(x[j], bias).h);
+                    }
+                }
+                if (__any_sync(0xffffffffu, t.v2 * b2 > pair_limit2<IMAG>(rho, pair_floor2(um, k)))) {
+                    k0 = kPairNear;
+                    if (out) {
+#pragma unroll
+                        for (int j = 0; j < 3; j++)
+                            x[j] = add(x[j], unpack(near_mem<IMAG>(xs + j * kPairPPts + i, 1, ix, p.nx, t.near[0], t.near[1])));
+                    }
                 }
             }
         }

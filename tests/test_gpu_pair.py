@@ -108,3 +108,25 @@ def test_rough_states_keep_the_accuracy_of_fp64(nx, ny, steps, dx, dt, gamma, im
     ref = _long_steps(psi, steps, imag, dx, dt, 20.0, 1.0, gamma, 0.5)
     err = np.sqrt((abs(s.get_state() - ref) ** 2).sum() / (abs(ref) ** 2).sum())
     assert err < 3 * 2.0 ** -53 * np.sqrt(steps)
+
+
+@pytest.mark.parametrize("imag", [True, False])
+@pytest.mark.parametrize("nx,ny", [(64, 48), (168, 100)])
+@pytest.mark.parametrize("what", ["herm", "density", "both"])
+def test_large_nonlinear_increments(what, nx, ny, imag):
+    """dt A between 2^-10 and 2^-6 (the HERM coefficients as a series in pairs), and a dense narrow
+    state: blocks whose dt mu sends them to FP64 from the start (its centre), after the vote (its
+    flanks) and not at all. Against long double, the bound of the rough states."""
+    if np.finfo(LD).eps > 2.0 ** -60:
+        pytest.skip("long double is no wider than double here")
+    omega, c0 = (0.5 if what == "density" else 7.0), (5.0 if what == "herm" else 60.0)
+    dx, dt, steps = 0.05, 8e-4, 8
+    prob, s = make_pair(2, nx, ny, dx=dx, dt=dt, c0=c0, c2=1.0, so_type=1, gamma=0.5, omega=omega, renorm=1 if imag else 0)
+    x, y = (np.arange(nx) - nx // 2) * dx, (np.arange(ny) - ny // 2) * dx
+    psi = np.stack([a * np.exp(-((x[None] - b) ** 2 + y[:, None] ** 2) / 0.32 + 0.3j * x[None]) for a, b in ((1.0, 0.05), (0.9, 0.0), (0.8j, -0.05))])
+    psi = psi / np.sqrt((abs(psi) ** 2).sum() * dx * dx)
+    s.set_state(psi)
+    (s.step_imag if imag else s.step_real)(steps)
+    ref = _long_steps(psi, steps, imag, dx, dt, c0, 1.0, 0.5, omega)
+    err = np.sqrt((abs(s.get_state() - ref) ** 2).sum() / (abs(ref) ** 2).sum())
+    assert err < 3 * 2.0 ** -53 * np.sqrt(steps)
