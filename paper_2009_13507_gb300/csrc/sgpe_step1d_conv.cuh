@@ -44,7 +44,6 @@ __global__ void __launch_bounds__(1024, 1)
                   int nsteps, int renorm) {
     extern __shared__ __align__(16) unsigned char step1d_conv_smem_raw[];
     __shared__ df red[3][32];
-    __shared__ float dsh[3];
     const int nx = p.nx, i = threadIdx.x, warp = i >> 5, lane = i & 31, nw = blockDim.x >> 5;
     float2* v0 = reinterpret_cast<float2*>(step1d_conv_smem_raw);  // [3][nx] the state
     float2* v1 = v0 + 3 * nx;                                       // [3][nx] after the pointwise substeps
@@ -128,14 +127,13 @@ __global__ void __launch_bounds__(1024, 1)
         }
         __syncthreads();
         if (IMAG && renorm && !last) {
+            // the next pending scale, by every warp for itself (the same sums in the same order)
             const df z = df(0.0f, 0.0f);
             if (all) {
-                // the next pending scale, by every warp for itself (the same sums in the same order)
                 const df N = warp_sum(lane < nw ? red[0][lane] : z) * df_from(p.cell);
                 const bool ok = isfinite(N.hi) && N.hi > 0.0f;
                 ds[0] = ds[1] = ds[2] = ok ? df_rsqrt(N).hi : 1.0f;
-            } else if (warp == 0) {
-                // Eq. (DJ): a chain of FP64 square roots and quotients, by one warp for the block
+            } else {
                 df S[3], f[3];
                 double d[3], N[3];
                 bool finite;
@@ -143,14 +141,9 @@ __global__ void __launch_bounds__(1024, 1)
                 for (int j = 0; j < 3; j++) S[j] = warp_sum(lane < nw ? red[j][lane] : z);
                 scale_from_df_sums(S, p.cell, renorm, p.mag, f, d, N, finite);
 #pragma unroll
-                for (int j = 0; j < 3; j++)
-                    if (lane == j) dsh[j] = f[j].hi;
+                for (int j = 0; j < 3; j++) ds[j] = f[j].hi;
             }
             __syncthreads();  // red is free for the next step's sums
-            if (!all) {
-#pragma unroll
-                for (int j = 0; j < 3; j++) ds[j] = dsh[j];
-            }
         } else if (!IMAG || !renorm) {
             ds[0] = ds[1] = ds[2] = 1.0f;
         }
