@@ -221,7 +221,7 @@ def run_reference(args):
         "impl": "reference", "metric": METRIC, "value": value, "unit": METRIC, "n_gpus": args.gpus,
         "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms, "higher_is_better": True,
         "scaling": "weak", "vs_baseline": None, "dtype": "f64", "data": "synthetic",
-        "arithmetic": "FP64 state, sums and norms; increments in FP32 pairs (about 2^-47 of an increment)",
+        "arithmetic": "FP64 throughout (CPU)",
         "time_steps_per_bench_step": steps_per,
         "config": bench_config(ws),
         "cpu_baseline": {"value": value, "unit": METRIC, "cores": cores, "kind": "oracle", "sample": sample,
@@ -603,6 +603,8 @@ def main():
         "metric": METRIC, "value": value, "unit": METRIC, "n_gpus": ws, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": t_step, "higher_is_better": True, "scaling": "weak",
         "vs_baseline": None, "dtype": "f64", "data": "synthetic",
+        "arithmetic": "FP64 state, sums and norms; small increments in FP32 pairs (about 2^-48 of an increment), "
+                      "large ones in FP64",
         "time_steps_per_bench_step": NSTEPS,
         "config": bench_config(ws),
         "roofline": {"bound": "alu", "kernel": dom_name,
