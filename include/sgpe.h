@@ -397,7 +397,9 @@ sgpe_status sgpe_batch_offsets(const sgpe_batch* b, size_t* offsets);
 /*
  * Bind the caller-owned batch state (state_elems complex elements, 16-byte
  * aligned) and workspace (256-byte aligned); uploads the work lists and builds
- * every instance's Crank-Nicolson tables. Synchronises the stream.
+ * every instance's Crank-Nicolson tables. The first call makes the batch's own
+ * streams and events (13 and 15: instances run side by side on them) on the device
+ * that was current at sgpe_batch_create. Synchronises the stream. SGPE_ECUDA if one of these fails.
  */
 sgpe_status sgpe_batch_bind(sgpe_batch* b, void* psi_dev, void* workspace_dev);
 

@@ -364,6 +364,7 @@ struct sgpe_batch {
     // the batch's own streams (kernels that may run side by side) and the events that order them
     cudaStream_t side[kSideStreams];
     cudaEvent_t ev_side[kSideStreams], ev_fork, ev_fork1;
+    int device;  // current at sgpe_batch_create (-1: none)
     char err[512];
 };
 
@@ -418,6 +419,24 @@ static cudaError_t kb_step1d_c(unsigned blocks, int nxmax, cudaStream_t s, typen
                                const typename V2<R>::T* pool, const int* ids, DevScalars* sc, int nsteps) {
     kb_step1d<R, IMAG, C><<<blocks, kStep1dThreads, step1d_smem_bytes<R, C>(nxmax), s>>>(A, I, pool, ids, sc, nsteps);
     return cudaGetLastError();
+}
+
+// The batch's streams and events, made where they do not exist yet (at the first bind: creating and
+// sizing a batch is host work) on the device that was current when the batch was created.
+static cudaError_t bstreams(sgpe_batch* b) {
+    int cur = 0;
+    cudaError_t e = cudaGetDevice(&cur);
+    const bool other = !e && b->device >= 0 && b->device != cur;
+    if (other) e = cudaSetDevice(b->device);
+    if (e) return e;
+    e = b->ev_fork ? cudaSuccess : cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming);
+    if (!e && !b->ev_fork1) e = cudaEventCreateWithFlags(&b->ev_fork1, cudaEventDisableTiming);
+    for (int i = 0; i < kSideStreams && !e; i++) {
+        if (!b->side[i]) e = cudaStreamCreateWithFlags(&b->side[i], cudaStreamNonBlocking);
+        if (!e && !b->ev_side[i]) e = cudaEventCreateWithFlags(&b->ev_side[i], cudaEventDisableTiming);
+    }
+    if (other) cudaSetDevice(cur);
+    return e;
 }
 
 // Fork: the side streams [first, first + count) of the batch start from the main
@@ -694,6 +713,10 @@ sgpe_status sgpe_batch_create(sgpe_batch** out, int n, const sgpe_instance* inst
     b->prec = prec;
     b->esz = prec == SGPE_C128 ? 16 : 8;
     b->stream = (cudaStream_t)cuda_stream;
+    if (cudaGetDevice(&b->device) != cudaSuccess) {
+        b->device = -1;
+        cudaGetLastError();
+    }
     b->inst.assign(inst, inst + n);
     b->psi = nullptr;
     b->work = nullptr;
@@ -835,17 +858,6 @@ sgpe_status sgpe_batch_create(sgpe_batch** out, int n, const sgpe_instance* inst
     b->o_mid = o;
     o = al256(o + (size_t)b->esz * b->state_elems);
     b->total = o;
-    cudaError_t e = cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming);
-    if (!e) e = cudaEventCreateWithFlags(&b->ev_fork1, cudaEventDisableTiming);
-    for (int i = 0; i < kSideStreams && !e; i++) {
-        e = cudaStreamCreateWithFlags(&b->side[i], cudaStreamNonBlocking);
-        if (!e) e = cudaEventCreateWithFlags(&b->ev_side[i], cudaEventDisableTiming);
-    }
-    if (e) {
-        set_thread_error("sgpe_batch_create: streams");
-        sgpe_batch_destroy(b);
-        return SGPE_ECUDA;
-    }
     *out = b;
     return SGPE_OK;
 }
@@ -868,6 +880,7 @@ sgpe_status sgpe_batch_bind(sgpe_batch* b, void* psi_dev, void* workspace_dev) {
     if (!psi_dev || !workspace_dev) return bfail(b, SGPE_EINVAL, "sgpe_batch_bind: null buffer");
     if (((uintptr_t)psi_dev & 15) || ((uintptr_t)workspace_dev & 255))
         return bfail(b, SGPE_EINVAL, "sgpe_batch_bind: psi must be 16-byte and workspace 256-byte aligned");
+    BCK(bstreams(b), "streams");
     binvalidate(b);
     b->psi = psi_dev;
     b->work = (unsigned char*)workspace_dev;

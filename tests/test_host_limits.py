@@ -48,3 +48,23 @@ def test_static_observables_scratch_holds_every_accepted_grid(tmp_path):
         counted = -(-nx // 32) * -(-ny // 4)
         assert counted <= limit and blocks <= counted, (dim, nx, ny)
         assert slot + blocks * NACC * 8 <= scratch, (dim, nx, ny, blocks)
+
+
+def test_a_batch_is_created_and_sized_without_a_gpu():
+    """sgpe_batch_create, _sizes and _offsets are host work: a caller can plan its buffers where no
+    GPU is (the batch's streams are made when it is bound)."""
+    import ctypes
+
+    from paper_2009_13507_gb300 import sgpe
+    lib = sgpe.load()
+    inst = (sgpe.Instance * 2)()
+    for i, (dim, nx, ny) in enumerate(((1, 128, 1), (2, 131, 140))):
+        inst[i].dim, inst[i].nx, inst[i].ny, inst[i].dx, inst[i].dy = dim, nx, ny, 0.1, 0.1
+        inst[i].params = sgpe.Physics(c0=1.0, dt=1e-3).c()
+    b = ctypes.c_void_p()
+    assert lib.sgpe_batch_create(ctypes.byref(b), 2, inst, sgpe.C64, None) == sgpe.OK
+    elems, nbytes, offs = ctypes.c_size_t(), ctypes.c_size_t(), (ctypes.c_size_t * 2)()
+    assert lib.sgpe_batch_sizes(b, ctypes.byref(elems), ctypes.byref(nbytes)) == sgpe.OK
+    assert lib.sgpe_batch_offsets(b, offs) == sgpe.OK
+    assert elems.value >= 3 * 128 + 3 * 131 * 140 and nbytes.value > 0 and offs[0] == 0 and offs[1] >= 3 * 128
+    assert lib.sgpe_batch_destroy(b) == sgpe.OK
