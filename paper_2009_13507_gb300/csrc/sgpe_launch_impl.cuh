@@ -185,7 +185,7 @@ cudaError_t Launcher<R>::step1d(cudaStream_t s, bool imag, void* A, const KParam
         return e ? e : cudaGetLastError();
     }
     if constexpr (is_f32<R>()) {
-        if (tabs_x.conv.kt > 0) {
+        if (tabs_x.conv.kt > 0 && !(imag && renorm == 2 && p.nx <= kConvDjMinN)) {
             ConvTab ct{};
             ct.kt = tabs_x.conv.kt;
             for (int k = 0; k < kConvTaps; k++) {

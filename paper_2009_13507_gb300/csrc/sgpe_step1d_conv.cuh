@@ -15,6 +15,10 @@
 // real time): 1000 points 11.6 / 13.1 -> 6.2 / 5.4, 500 6.8 -> 3.5, 256 3.0 / 3.0 -> 2.2 / 1.8,
 // 40 2.0 / 1.9 -> 1.6 / 1.3.
 //
+// Under Eq. (DJ) lines of at most kConvDjMinN points keep the lane-chunk loop: the scale is a chain of seven
+// FP64 square roots a step there too, but its sums are FP64 already and need no conversion (us a
+// step, lane chunks / this: 64 points 5.2 / 6.0, 128 5.4 / 6.0, 256 6.3 / 6.4, 384 9.9 / 6.9, 1000 14.7 / 9.8).
+//
 // Norms (imaginary time): squares split exactly, summed in pairs by shuffles and across
 // the warps by every warp for itself; one sum serves Eq. (DJ2), the components' are only
 // formed where Eq. (DJ) or the end of the loop needs them.
@@ -22,6 +26,8 @@
 #include "sgpe_cn.cuh"
 
 namespace sgpe {
+
+constexpr int kConvDjMinN = 256;
 
 // W_k per time mode: (re, re, -im, im).
 struct ConvTab {
@@ -44,6 +50,7 @@ __global__ void __launch_bounds__(1024, 1)
                   int nsteps, int renorm) {
     extern __shared__ __align__(16) unsigned char step1d_conv_smem_raw[];
     __shared__ df red[3][32];
+    __shared__ float dsh[3];
     const int nx = p.nx, i = threadIdx.x, warp = i >> 5, lane = i & 31, nw = blockDim.x >> 5;
     float2* v0 = reinterpret_cast<float2*>(step1d_conv_smem_raw);  // [3][nx] the state
     float2* v1 = v0 + 3 * nx;                                       // [3][nx] after the pointwise substeps
@@ -127,13 +134,15 @@ __global__ void __launch_bounds__(1024, 1)
         }
         __syncthreads();
         if (IMAG && renorm && !last) {
-            // the next pending scale, by every warp for itself (the same sums in the same order)
             const df z = df(0.0f, 0.0f);
             if (all) {
+                // the next pending scale, by every warp for itself (the same sums in the same order)
                 const df N = warp_sum(lane < nw ? red[0][lane] : z) * df_from(p.cell);
                 const bool ok = isfinite(N.hi) && N.hi > 0.0f;
                 ds[0] = ds[1] = ds[2] = ok ? df_rsqrt(N).hi : 1.0f;
-            } else {
+            } else if (warp == 0) {
+                // Eq. (DJ): a chain of FP64 square roots and quotients, by one warp for the block (every warp
+                // for itself, they shared the FP64 pipe: 131 points 6.95 us a step against 6.26)
                 df S[3], f[3];
                 double d[3], N[3];
                 bool finite;
@@ -141,9 +150,14 @@ __global__ void __launch_bounds__(1024, 1)
                 for (int j = 0; j < 3; j++) S[j] = warp_sum(lane < nw ? red[j][lane] : z);
                 scale_from_df_sums(S, p.cell, renorm, p.mag, f, d, N, finite);
 #pragma unroll
-                for (int j = 0; j < 3; j++) ds[j] = f[j].hi;
+                for (int j = 0; j < 3; j++)
+                    if (lane == j) dsh[j] = f[j].hi;
             }
             __syncthreads();  // red is free for the next step's sums
+            if (!all) {
+#pragma unroll
+                for (int j = 0; j < 3; j++) ds[j] = dsh[j];
+            }
         } else if (!IMAG || !renorm) {
             ds[0] = ds[1] = ds[2] = 1.0f;
         }
