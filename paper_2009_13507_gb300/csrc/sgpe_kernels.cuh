@@ -37,8 +37,9 @@ struct DevScalars {
     int step_idx;        // index into a per-step Omega table (real time)
     int err;             // bit 0: non-finite norm
     unsigned ticket[4];  // last-block tickets: 0 step finalize, 1 observables, 2 norms
-    // the pair step (complex128): steps done, and the high word of the largest |Re|, |Im| of the
-    // state as the y sweep of step k saw it in umax[k % 3] (0: unknown); umax_slot: the running step's
+    // the pair step (complex128): the high word of the largest |Re|, |Im| of the state as the y sweep
+    // of step k saw it in umax[k % 3] (0: unknown); pair_tick: the next step's slot, umax_slot: the
+    // running step's (slots, not a count: a count of steps would overflow within hours)
     int pair_tick, umax_slot;
     unsigned umax[3];
     unsigned umax_prev;  // that of the step before, where this step may compare with it (0: unknown)

@@ -513,7 +513,7 @@ __global__ void __launch_bounds__(kPairXThreads, 2)
         const int tick = *(volatile const int*)&sc->pair_tick;
         um = *(volatile const unsigned*)&sc->umax[(tick + 2) % 3];
         if (blockIdx.x == 0 && tid == 0) {  // the slot of this step's y sweep; the next step's is cleared
-            sc->umax_slot = tick % 3;
+            sc->umax_slot = tick;
             sc->umax[(tick + 1) % 3] = 0u;
         }
         const unsigned mx = __reduce_max_sync(0xffffffffu, max(pair_mag(x), max(pair_mag(ym), pair_mag(yp))));
@@ -819,7 +819,7 @@ __global__ void __launch_bounds__(kPairPPts, 2)
         const int tick = *(volatile const int*)&sc->pair_tick;
         um = *(volatile const unsigned*)&sc->umax[(tick + 2) % 3];
         if (blockIdx.x == 0 && i == 0) {
-            sc->umax_slot = tick % 3;
+            sc->umax_slot = tick;
             sc->umax[(tick + 1) % 3] = 0u;
         }
         unsigned mx = 0u;
@@ -1112,7 +1112,7 @@ __global__ void __launch_bounds__(256, 4)
     const cx<R> zr = {R(0), R(0)};
     pdl_wait();
     if (blockIdx.x == 0 && tid < 3) {
-        if (tid == 0) sc->pair_tick += 1;
+        if (tid == 0) sc->pair_tick = (sc->pair_tick + 1) % 3;
         if (head) {  // as k_cny_reg
             if (renorm) {
                 if (tid == 0) sc->scale_src = 1;

@@ -130,3 +130,23 @@ def test_large_nonlinear_increments(what, nx, ny, imag):
     ref = _long_steps(psi, steps, imag, dx, dt, c0, 1.0, 0.5, omega)
     err = np.sqrt((abs(s.get_state() - ref) ** 2).sum() / (abs(ref) ** 2).sum())
     assert err < 3 * 2.0 ** -53 * np.sqrt(steps)
+
+
+def test_the_slot_of_the_largest_value_stays_a_slot(tmp_path):
+    """The step's index into the three slots of the state's largest value counts modulo three: a
+    count of steps passes 2^31 within hours and its remainder then indexes in front of the slots."""
+    import subprocess
+
+    from paper_2009_13507_gb300 import build as B
+    src, exe = tmp_path / "probe.cu", tmp_path / "probe"
+    src.write_text('#include <stddef.h>\n#include <stdio.h>\n#include "sgpe_kernels.cuh"\n'
+                   'int main() { printf("%zu", offsetof(sgpe::DevScalars, pair_tick)); }\n')
+    subprocess.run([B._nvcc(), *B.ARCH, "-std=c++17", "--expt-relaxed-constexpr", "-I", B.CSRC, "-o", str(exe), str(src)],
+                   check=True, capture_output=True)
+    at = int(subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout)
+    _, s = make_pair(2, 64, 48, dx=0.1, c0=1.0, so_type=1, gamma=0.3, dt=1e-3)
+    s.set_state(I.random_state((3, 48, 64), 1, 0.01, 20.0))
+    for n in (1, 1, 1, 7, 40):
+        s.step_imag(n)
+        s.synchronize()
+        assert 0 <= int(s.workspace[at:at + 4].cpu().numpy().view(np.int32)[0]) < 3
