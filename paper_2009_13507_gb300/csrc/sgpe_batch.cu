@@ -133,8 +133,13 @@ __global__ void __launch_bounds__(kPwxThreads, pwx_min_blocks<R, C, IMAG>())
 // and 36 us of the 244 us of a step of the 64-instance complex64 workload, whose 50
 // steps went from 12.2 to 5.2 ms together with the odd rows on the tiled step); here
 // they run under the 2D instances' launches.
-template <typename R, bool IMAG, int C>
-__global__ void __launch_bounds__(kStep1dThreads, 1)
+// MINB: blocks an SM holds. One, with all the registers it wants, is the faster up to a line an SM;
+// beyond, lines of 129..512 points (160 to 255 registers) would run one after the other where the per-step
+// kernels had two on an SM: us a step of 304 lines of 512 points, complex128, Eq. (DJ2) / (DJ), step by
+// step 63.0 / 59.1, one block 65.2 / 66.4, two 56.1 / 53.0; complex64, 608 lines, Eq. (DJ) 32.4, 40.8, 27.3. (1000
+// lines under Eq. (DJ): 184 and 187, complex64 52.0 and 53.8.)
+template <typename R, bool IMAG, int C, int MINB>
+__global__ void __launch_bounds__(kStep1dThreads, MINB)
     kb_step1d(typename V2<R>::T* A, const BInst* __restrict__ insts, const typename V2<R>::T* __restrict__ pool,
               const int* __restrict__ ids, DevScalars* scs, int nsteps) {
     const int i = ids[blockIdx.x];
@@ -365,6 +370,7 @@ struct sgpe_batch {
     cudaStream_t side[kSideStreams];
     cudaEvent_t ev_side[kSideStreams], ev_fork, ev_fork1;
     int device;  // current at sgpe_batch_create (-1: none)
+    int sms;     // its SMs (at the first bind)
     char err[512];
 };
 
@@ -407,17 +413,20 @@ template <typename R, bool IMAG> static cudaError_t kb_pwx_allow() {
     return e;
 }
 
+template <typename R, bool IMAG, int C, int MINB> static cudaError_t kb_step1d_allow_c() {
+    return cudaFuncSetAttribute(kb_step1d<R, IMAG, C, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)step1d_smem_bytes<R, C>(32 * C));
+}
 template <typename R, bool IMAG> static cudaError_t kb_step1d_allow() {
-    cudaError_t e = cudaFuncSetAttribute(kb_step1d<R, IMAG, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)step1d_smem_bytes<R, 16>(32 * 16));
-    if (!e) e = cudaFuncSetAttribute(kb_step1d<R, IMAG, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)step1d_smem_bytes<R, 32>(32 * 32));
+    cudaError_t e = kb_step1d_allow_c<R, IMAG, 16, 1>();
+    if (!e) e = kb_step1d_allow_c<R, IMAG, 16, 2>();
+    if (!e) e = kb_step1d_allow_c<R, IMAG, 32, 1>();
     return e;
 }
-template <typename R, bool IMAG, int C>
+template <typename R, bool IMAG, int C, int MINB = 1>
 static cudaError_t kb_step1d_c(unsigned blocks, int nxmax, cudaStream_t s, typename V2<R>::T* A, const BInst* I,
                                const typename V2<R>::T* pool, const int* ids, DevScalars* sc, int nsteps) {
-    kb_step1d<R, IMAG, C><<<blocks, kStep1dThreads, step1d_smem_bytes<R, C>(nxmax), s>>>(A, I, pool, ids, sc, nsteps);
+    kb_step1d<R, IMAG, C, MINB><<<blocks, kStep1dThreads, step1d_smem_bytes<R, C>(nxmax), s>>>(A, I, pool, ids, sc, nsteps);
     return cudaGetLastError();
 }
 
@@ -435,6 +444,7 @@ static cudaError_t bstreams(sgpe_batch* b) {
         if (!b->side[i]) e = cudaStreamCreateWithFlags(&b->side[i], cudaStreamNonBlocking);
         if (!e && !b->ev_side[i]) e = cudaEventCreateWithFlags(&b->ev_side[i], cudaEventDisableTiming);
     }
+    if (!e) e = cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, other ? b->device : cur);
     if (other) cudaSetDevice(cur);
     return e;
 }
@@ -597,12 +607,19 @@ template <typename R, bool IMAG> static cudaError_t benqueue_n(sgpe_batch* b, in
             const unsigned m = (unsigned)it->second.second;
             const int nm = b->n1max[it->first];
             cudaStream_t s = b->side[k];
+            const bool many = m > (unsigned)b->sms;
             switch (it->first) {
                 case 1: e = kb_step1d_c<R, IMAG, 1>(m, nm, s, A, I, pool, w, sc, n); break;
                 case 2: e = kb_step1d_c<R, IMAG, 2>(m, nm, s, A, I, pool, w, sc, n); break;
                 case 4: e = kb_step1d_c<R, IMAG, 4>(m, nm, s, A, I, pool, w, sc, n); break;
-                case 8: e = kb_step1d_c<R, IMAG, 8>(m, nm, s, A, I, pool, w, sc, n); break;
-                case 16: e = kb_step1d_c<R, IMAG, 16>(m, nm, s, A, I, pool, w, sc, n); break;
+                case 8:
+                    e = many ? kb_step1d_c<R, IMAG, 8, 2>(m, nm, s, A, I, pool, w, sc, n)
+                             : kb_step1d_c<R, IMAG, 8>(m, nm, s, A, I, pool, w, sc, n);
+                    break;
+                case 16:
+                    e = many ? kb_step1d_c<R, IMAG, 16, 2>(m, nm, s, A, I, pool, w, sc, n)
+                             : kb_step1d_c<R, IMAG, 16>(m, nm, s, A, I, pool, w, sc, n);
+                    break;
                 default: e = kb_step1d_c<R, IMAG, 32>(m, nm, s, A, I, pool, w, sc, n); break;
             }
         }
