@@ -494,13 +494,15 @@ static bool general_path(const sgpe_ctx* c) { return c->params.split != 0 || c->
 // imaginary, 1 real) as increments in FP32 pairs (sgpe_pair.cuh), where both axes'
 // sweeps are short convolutions (bt up to about 0.08, lines of more than 16 points).
 // Double-float grids of 320..~630 points an axis keep the tiled step in imaginary time, where it
-// is the faster one (us a step, tiled against pair: 320^2 29.5 / 31.8, 512^2 55 / 68, 700^2 108 /
-// 97; in real time 400 x 330 53 / 37).
+// is the faster one (us a step, tiled against pair: 320^2 29.3 / 31.1, 512^2 55.6 / 66.6, 700^2 107 /
+// 95; in real time 400 x 330 53 / 37).
 constexpr long long kPairCdfTiledMax = 400000;
-// Grids of fewer points keep the register kernels (24 x 20: 15.6 us a step against 17.6; 48 x 40
-// 16.3 / 14.5), and so do complex128 steps longer than this, whose dt mu passes 2^-5 where the
-// state lives so often that most blocks leave the increments (256^2 at dt = 4e-3 with c0 rho = 16:
-// 48 / 53 us; 500 x 400 at 2e-3 167 / 90).
+// Grids of fewer points keep the register kernels. (24 x 20, us a step, register / pair: 15.6 / 17.6 when the
+// line was drawn, 14.4 / 11.3 since the head kernel's chains were shortened; the line has not followed.)
+// So do complex128 steps longer than kPairMaxDt, whose dt mu passes 2^-5 where the state lives so often that most
+// blocks leave the increments: dx = 0.2, c0 = 50, imaginary time 100 x 120 at dt = 4e-3 18.0 / 19.4, at 0.01 17.7 /
+// 24.5, 64^2 at 0.01 15.7 / 18.8. (Grids that fill the GPU would gain there too: 256^2 47.5 / 32.5 and 47.7 /
+// 45.1; the line has not been split by size.)
 constexpr long long kPairMinPoints = 1536;
 constexpr double kPairMaxDt = 2.5e-3;
 static bool pair_mode(const sgpe_ctx* c, int mode) {

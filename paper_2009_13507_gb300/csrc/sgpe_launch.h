@@ -124,8 +124,9 @@ inline int pair_pts(int n, int halo, int pts) {
     const int ns = pair_nseg(n, halo, pts);
     return ns == 1 ? n : ceil_div(n, ns) + 2 * halo;
 }
-// Points of a grid up to which the head kernel takes three threads a point (96^2 13.1 against
-// 17.3 us a step, 128^2 14.7 against 16.4; 144^2 18.5 against 17.3 with one thread a point).
+// Points of a grid up to which the head kernel takes three threads a point (us a step, three threads /
+// one: 96^2 13.0 / 14.5, 128^2 13.7 / 15.0, 144^2 15.5 / 16.1; its rows take two segments from 161 points
+// on, where the halo's work counts three times).
 constexpr int kPairSplitMax = 128 * 128;
 // Tiles of a component in the y sweep (= norm partials).
 inline int pair_parts(int nx, int ny) { return ceil_div(nx, kPairCols) * ceil_div(ny, kPairRows); }

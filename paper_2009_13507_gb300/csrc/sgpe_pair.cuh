@@ -11,14 +11,12 @@
 // which is a rounding of the FP64 state itself; the sum state + increment is the
 // only operation that needs the state's full width. Increments that are not small
 // (large dt mu, strong SO, structure near the grid scale) are formed in FP64, see
-// pair_large. The FP64 evaluation rounds the
-// whole state some ten times a step instead. Error against an 80-bit reference (FP64
-// step -> this one): 128 x 112, 30 steps at dt = 2e-4, imaginary time 7.1e-16 -> 4.3e-16,
-// real time 3.8e-15 -> 1.2e-15; 64 x 80, 60 steps at bt = 0.075 4.4e-16 -> 4.7e-16 and
-// 5.5e-15 -> 4.5e-15; double-float 1.8e-14 -> 3.8e-15 and 6.6e-14 -> 9.0e-15. Measured,
-// us a step: complex128 256^2 imaginary / real time 42.9 / 49.8 -> 21.7 / 22.8, 512^2 158 /
-// 195 -> 86 / 91, 161^2 real time 42.2 -> 18.2, 2048^2 2118 -> 1010; double-float 256^2 20.1
-// / 27.2 -> 17.3 / 17.9, 1024^2 217 / 357 -> 209 / 233.
+// pair_large. The FP64 evaluation rounds the whole state some ten times a step instead. Error
+// against an 80-bit reference (FP64 step -> this one): 128 x 112, 30 steps at dt = 2e-4,
+// imaginary time 7.1e-16 -> 4.3e-16, real time 3.8e-15 -> 1.2e-15; double-float 1.8e-14 ->
+// 3.8e-15 and 6.6e-14 -> 9.0e-15. Measured, us a step: complex128 256^2 imaginary / real time
+// 42.9 / 49.6 -> 22.5 / 23.3, 512^2 158 / 195 -> 88 / 91, 161^2 real time 42.1 -> 18.7, 2048^2 2116 ->
+// 1032; double-float 256^2 19.8 / 27.3 -> 17.3 / 18.0, 1024^2 220 / 352 -> 208 / 233.
 //
 // Pairs here are "lazy": products keep the exact error of the leading product and
 // both cross terms, sums keep the exact rounding error of the leading sum, and
@@ -86,7 +84,7 @@ __device__ __forceinline__ df lscale(df a, float s) { return df(__fmul_rn(a.hi, 
 
 // A complex pair: h = (re.hi, im.hi), l = (re.lo, im.lo), so that sums and products with a
 // real pair take the packed FP32x2 instructions, both parts at once (each lane rounded as the
-// scalar instruction): the kernels are bound by instruction issue.
+// scalar instruction): fewer instructions to fetch and to wait for.
 __device__ __forceinline__ float2 p_add(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ float2 p_sub(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a); }
 __device__ __forceinline__ float2 p_neg(float2 a) { return __fmul2_rn(a, make_float2(-1.0f, -1.0f)); }
@@ -462,7 +460,7 @@ __device__ __forceinline__ float norm2(float2 a) { return fmaf(a.x, a.x, a.y * a
 // and component, the components in warps of their own (three neighbouring warps a group of
 // 32 points, on different sub-partitions): each substep is the same short
 // code for all three, so a block's warps share its instruction lines and a small grid's
-// few blocks have three times the warps (64^2: 16.7 us a step with one thread a point, 12.9
+// few blocks have three times the warps (64^2: 15.1 us a step with one thread a point, 11.9
 // so). The components meet in shared memory: the differences before SO, the densities
 // before CALCNU, the state before HERM, the increments and links before the sweep.
 //
@@ -775,9 +773,10 @@ __global__ void __launch_bounds__(kPairXThreads, 2)
 
 // The same with one thread per point, for grids that fill the GPU: the components meet in
 // registers, which halves the instructions of the by-component kernel (no factor is formed
-// three times: 4.9 M against 10.9 M at 256^2) and needs half the barriers (256^2: 41 -> 25 us
-// a step). Bound by instruction issue and the FP64 pipe's 24 instructions a point. Segments
-// of up to kPairPPts points.
+// three times: 4.9 M against 10.9 M at 256^2 when the two were first compared) and needs half the
+// barriers (256^2: 41 -> 25 us a step then). Bound by latency and instruction fetch: at 256^2 30 % of the
+// issue slots and 17 % of the FP64 pipe are used, 32 % of the fetches miss the instruction cache
+// (3.2 stalls an issue), 256 blocks are 21 % of the warps. Segments of up to kPairPPts points.
 template <typename R, bool IMAG>
 __global__ void __launch_bounds__(kPairPPts, 2)
     k_pair_xp(const typename V2<R>::T* __restrict__ A, typename V2<R>::T* __restrict__ Bout, KParams p, DevScalars* sc,
