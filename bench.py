@@ -58,10 +58,13 @@ FP64_PEAK_TFLOPS = 1.259
 # and 600 steps on one thread (~8 s).
 CPU_SAMPLE_STEPS = NSTEPS
 CPU_SINGLE_STEPS = 600
-# DRAM bytes (read + write, cold L2) and executed warp instructions of one launch of the dominant
-# kernel on this workload in an ncu capture (profiles/k_pair_2d256.md).
-HEAD_TRAFFIC_BYTES = 3232512
-HEAD_WARP_INSTRUCTIONS = 6301565
+# One ncu capture of the dominant kernel on this workload (profiles/k_pair_2d256.md): its name, the
+# source that it was compiled from, the DRAM bytes (read + write, cold L2) and the executed warp
+# instructions of a launch. The line gives None for them where another kernel runs or the source
+# has changed since.
+HEAD_CAPTURE = {"kernel": "k_pair_xp<double, true>", "source_sha16": "6d0b36bcdc952ff4", "traffic_bytes": 3239424,
+                "warp_instructions": 6433008}
+HEAD_SOURCE = os.path.join("paper_2009_13507_gb300", "csrc", "sgpe_pair.cuh")
 # Warp instructions the GPU can issue: 152 SMs x 4 schedulers x 2.07 GHz.
 ISSUE_PEAK_GINST = 1258.6
 
@@ -136,10 +139,40 @@ def measured_hbm_gbs():
         return None
 
 
+def dominant_kernel(run):
+    """The name of the kernel with the most device time in run(), without namespaces and arguments
+    (torch.profiler; only the name is taken, no time), or None where it cannot be had."""
+    try:
+        import torch
+        from torch.profiler import ProfilerActivity, profile
+        def spent(e):
+            t = getattr(e, "self_device_time_total", None)
+            return t if t is not None else getattr(e, "self_cuda_time_total", 0)
+        for _ in range(3):  # (the first session of a process can come back empty)
+            with profile(activities=[ProfilerActivity.CPU, ProfilerActivity.CUDA]) as prof:
+                run()
+                torch.cuda.synchronize()
+            kernels = [e for e in prof.key_averages() if "sgpe::" in e.key]
+            if kernels:
+                name = max(kernels, key=spent).key
+                return name.split("(")[0].replace("void ", "").replace("sgpe::", "").strip()
+        return None
+    except Exception:
+        return None
+
+
+def head_capture(kernel):
+    """HEAD_CAPTURE where it is of this kernel and of the present source, else None."""
+    import hashlib
+    with open(os.path.join(ROOT, HEAD_SOURCE), "rb") as fh:
+        sha = hashlib.sha256(fh.read()).hexdigest()[:16]
+    return HEAD_CAPTURE if kernel == HEAD_CAPTURE["kernel"] and sha == HEAD_CAPTURE["source_sha16"] else None
+
+
 def hbm_view(effective_gbps: float) -> dict:
     """Effective bandwidth of the step's two streaming passes (192 algorithmic bytes per
     point-step) against the measured HBM copy peak; the state is L2-resident, so this is
-    context, not the binding roof (instruction issue is)."""
+    context, not the binding roof (latency and instruction fetch are)."""
     peak = measured_hbm_gbs()
     return {"algorithmic_bytes_per_point_step": 192, "effective_GBps": effective_gbps,
             "peak_GBps": peak, "peak_source": "measured copy bandwidth" if peak else None,
@@ -528,8 +561,6 @@ def main():
     share = {n: kms[i] / kms.sum() for i, n in enumerate(names) if int(kcnt[i]) > 0}
     dom_ms = kavg[names[0]]
     dom_flops = POINTWISE_FLOPS + (CN_FLOPS if fused else 0)
-    dom_name = "k_pair_xp<double, imag> (SO+CALCNU+HERM, CN-x as increments in FP32 pairs)"
-    achieved_ginst = HEAD_WARP_INSTRUCTIONS / (dom_ms * 1e-3) / 1e9
     achieved_tflops = dom_flops * NX * NY / (dom_ms * 1e-3) / 1e12
     # the FP64 roof measured on this GPU in this run (FMA-chain kernel, CUDA events)
     try:
@@ -596,6 +627,10 @@ def main():
                "single_thread": {"value": r1, "cores": 1,
                                  "sample": "%d time steps (%.1f s)" % (CPU_SINGLE_STEPS, t1)}}
 
+    # (after everything that is timed: the profiler stays loaded)
+    dom_name = dominant_kernel(lambda: solver.profile_steps(16, True))
+    capture = head_capture(dom_name)
+    achieved_ginst = capture["warp_instructions"] / (dom_ms * 1e-3) / 1e9 if capture else None
     lps = solver.launches_per_step()
     # + the end-of-steps norm/scale launch of the two-launch 2D step, flush, scale reset, observables
     launches = NSTEPS * lps + (1 if lps == 2 else 0) + 3
@@ -607,10 +642,13 @@ def main():
                       "large ones in FP64",
         "time_steps_per_bench_step": NSTEPS,
         "config": bench_config(ws),
-        "roofline": {"bound": "alu", "kernel": dom_name,
+        # latency and instruction fetch bound the kernel; the nearest roof is instruction issue
+        "roofline": {"bound": "latency", "kernel": dom_name,
                      "achieved": achieved_ginst, "peak": ISSUE_PEAK_GINST, "unit": "G warp instructions/s",
-                     "frac": achieved_ginst / ISSUE_PEAK_GINST, "traffic": HEAD_TRAFFIC_BYTES,
-                     "peak_source": "152 SMs x 4 schedulers x 2.07 GHz; instructions per launch from ncu",
+                     "frac": achieved_ginst / ISSUE_PEAK_GINST if capture else None,
+                     "traffic": capture["traffic_bytes"] if capture else None,
+                     "peak_source": "152 SMs x 4 schedulers x 2.07 GHz; instructions per launch from ncu "
+                                    "(None where the kernel or its source is not the captured one)",
                      "avg_launch_ms": dom_ms,
                      # the same work counted as FP64 flops, against what the FP64 pipe could do
                      "fp64_view": {"flops_per_point": dom_flops, "achieved_tflops": achieved_tflops,
