@@ -150,3 +150,24 @@ def test_the_slot_of_the_largest_value_stays_a_slot(tmp_path):
         s.step_imag(n)
         s.synchronize()
         assert 0 <= int(s.workspace[at:at + 4].cpu().numpy().view(np.int32)[0]) < 3
+
+
+@pytest.mark.parametrize("nx,ny", [(64, 48), (168, 100)])
+@pytest.mark.parametrize("what", ["small_norm", "large_norm", "tiny_rough", "huge_rough"])
+def test_scales_far_from_one(what, nx, ny):
+    """Factors beyond 10^6 in the first renormalised step (the shift starts anew, SO with the factors
+    of its sources), and rough states with strong SO far from order 1 in linear real-time runs (blocks
+    in FP64 under a shift). Against long double, the bound of the rough states."""
+    if np.finfo(LD).eps > 2.0 ** -60:
+        pytest.skip("long double is no wider than double here")
+    imag = what.endswith("norm")
+    scale = {"small_norm": 1e-8, "large_norm": 1e8, "tiny_rough": 1e-80, "huge_rough": 1e60}[what]
+    c0 = 40.0 if what == "small_norm" else 0.0
+    c2, gamma, dx, dt, steps = (1.0 if c0 else 0.0), (0.8 if imag else 20.0), 0.1, 2e-3, 8
+    prob, s = make_pair(2, nx, ny, dx=dx, dt=dt, c0=c0, c2=c2, so_type=1, gamma=gamma, omega=0.5, renorm=1 if imag else 0)
+    psi = _rand(prob, 2 * nx + ny, env=8.0) * scale
+    s.set_state(psi)
+    (s.step_imag if imag else s.step_real)(steps)
+    ref = _long_steps(psi, steps, imag, dx, dt, c0, c2, gamma, 0.5)
+    err = np.sqrt((abs(s.get_state() / scale - ref / scale) ** 2).sum() / (abs(ref / scale) ** 2).sum())
+    assert err < 3 * 2.0 ** -53 * np.sqrt(steps)
